@@ -1,0 +1,798 @@
+// a7 (local prediction) and a8 (local Newton MLE of d) in 59-bit fixed point
+// (fx59.cuh), for designs of up to 128 rows and nuggets below 1.
+//
+// One CTA of 128 threads per location (persistent, atomic work counter), all
+// of its matrices in shared memory.
+//   K_n is factorised as L L^T with the responses (and, for the prediction,
+//   k_n(x)) as further rows: the rows below K_n's become z^T = (L^{-1} Y)^T
+//   and w^T = (L^{-1} k)^T.  For the MLE the factorisation carries its first
+//   and second derivatives in log d along (forward mode): with
+//     M0 = K,  M1 = d K' = t e^-t,  M2 = d^2 K'' = (t^2 - 2t) e^-t,  t = D/d,
+//   column c of L, L1 = d L', L2 = d^2 L'' comes from
+//     S0 = M0 - sum L L^T,  S1 = M1 - sum (L1 L^T + L L1^T),
+//     S2 = M2 - sum (L2 L^T + 2 L1 L1^T + L L2^T)            (sums over k < c)
+//     l = sqrt(S0),  l1 = S1 / (2l),  l2 = (S2/2 - l1^2) / l   on the diagonal,
+//     L = S0 / l,  L1 = (S1 - L l1) / l,  L2 = (S2 - 2 L1 l1 - L l2) / l  below,
+//   and then log|K|, psi = |z|^2 and their derivatives are sums over the
+//   diagonal and over the z row: six products a (row, column, k) triple, n^3
+//   in all, with no inverse, no traces and no second pass.  All entries are
+//   of order one (t e^-t <= 1/e, |t^2 - 2t| e^-t <= 0.47, |L| < sqrt(2)), which
+//   is what fixed point asks for; z is scaled by a power of two.
+//
+// Bound: the integer multiply pipe (the inner products) and the FP64 unit
+// (the n^2/2 exponentials and their products with powers of t) about evenly.
+// Two columns a step: the sums run with a 2 x 2 tile of (rows, columns) a
+// thread, so that a 16-byte shared-memory load (two k) feeds four products,
+// and 4 to 16 lanes share a row's sum, so that the threads stay busy as the
+// rows left shrink; meanwhile one warp makes the 2 x 2 diagonal block, and
+// then one thread a row finishes the two columns.
+//
+// Measured against the FP64 kernels (gp_local.cu), whole calls: the MLE of
+// 20,000 slab locations, n = 60, 4.1 evaluations each, 79.9 -> 29.7 ms; the
+// prediction at 100 locations, n = 50, 112 -> 64 us.  Errors against 64-bit
+// references no larger (l'' 10 to 100 times smaller than from explicit
+// inverses).  The line: above 128 rows the three matrices no longer fit in
+// shared memory; from g = 1 on the factor's entries leave the range.
+//
+// A location whose values leave the fixed-point range (|x| < 2; 1 in the
+// further rows) first widens the scale of z, then goes to the FP64 kernels of
+// gp_local.cu: its status is FX_REDO when this kernel ends, and a second launch redoes it
+// (returning at once when there is none).  Non-finite inputs go there too.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "device_util.cuh"
+#include "exp64.cuh"
+#include "fx59.cuh"
+#include "gp_common.cuh"
+#include "lagp_internal.h"
+
+namespace {
+
+constexpr int FXT = 128, FXW = FXT / 32;
+constexpr int FX_NMAX = 128;
+// z is scaled by 2^-FX_Z0 / max |y| (|z| up to 64 max |y| then fits), else by 2^-FX_Z1
+constexpr int FX_Z0 = 6, FX_Z1 = 14;
+
+// Matrices are stored by pairs of columns: entry (i, k) in the 16-byte word
+// i + q (m - 1) - q^2, q = k / 2, half k mod 2 (rows i >= 2q of m; a pair's
+// rows are adjacent, so that the lanes of a warp read without conflicts).
+__host__ __device__ inline int fx_words(int n, int m) {
+    const int Q = (n + 1) / 2;
+    return Q * (m - 1) - (Q - 1) * (Q - 1) + 1;
+}
+__device__ __forceinline__ int fx_slot(int i, int k, int m) {
+    const int q = k >> 1;
+    return 2 * (i + q * (m - 1) - q * q) + (k & 1);
+}
+
+// What a step's threads need of its 2 x 2 diagonal block (negated where it
+// is subtracted).
+struct __align__(16) FxDiag {
+    Fx y[2];             // 1 / l = y 2^t
+    int t[2];
+    Fx nl1[2], nl2[2];   // -l1, -l2
+    Fx na, nb, ne;       // -L, -L1, -L2 of the lower left entry
+    int pad[2];
+};
+
+// The dynamic shared memory: `words` 16-byte words a matrix from the start,
+// then (at byte y_at) n responses, n reciprocals of the pivots (1 / l = ry
+// 2^(rt - 59)) and their exponents.  Its parts are addressed from the symbol,
+// so that the compiler sees shared memory also behind a call.
+extern __shared__ __align__(16) unsigned char fx_smem[];
+
+struct FxFactor {
+    int words, n, m;  // matrix words, order, rows with the further ones
+    int y_at, nmax;
+};
+
+__device__ __forceinline__ int4 *fx_mat(const FxFactor &F, int mat) {
+    return reinterpret_cast<int4 *>(fx_smem) + mat * F.words;
+}
+__device__ __forceinline__ double *fx_y(const FxFactor &F) { return reinterpret_cast<double *>(fx_smem + F.y_at); }
+__device__ __forceinline__ long long *fx_ry(const FxFactor &F) {
+    return reinterpret_cast<long long *>(fx_smem + F.y_at) + F.nmax;
+}
+__device__ __forceinline__ int *fx_rt(const FxFactor &F) {
+    return reinterpret_cast<int *>(fx_smem + F.y_at) + 4 * F.nmax;
+}
+__device__ __forceinline__ long long *fx_raw(const FxFactor &F, int mat, int slot) {
+    return reinterpret_cast<long long *>(fx_mat(F, mat)) + slot;
+}
+__device__ __forceinline__ void fx_store(const FxFactor &F, int mat, int slot, Fx f) {
+    reinterpret_cast<int2 *>(fx_mat(F, mat))[slot] = make_int2(f.h, f.l);
+}
+__device__ __forceinline__ long long fx_load(const FxFactor &F, int mat, int slot) {
+    const int2 v = reinterpret_cast<const int2 *>(fx_mat(F, mat))[slot];
+    return fx_join(Fx{v.x, v.y});
+}
+
+// v 2^t y, |v 2^t| < 2 (so that the result stays below 2.84)
+__device__ __forceinline__ long long fx_scaled(long long v, int t, Fx y, unsigned &bad) {
+    bad |= fx_beyond(v, 28 - t);
+    return fx_mul(fx_split(v << t), y);
+}
+
+// Nonzero unless |x| < 2 (the high limb may be doubled).
+__device__ __forceinline__ unsigned fx_beyond_h(Fx x) { return (unsigned)(x.h + (1 << 30)) >> 31; }
+
+// One column of a row: L = S0 / l, L1 = (S1 - L l1) / l, L2 = (S2 - 2 L1 l1 - L l2) / l.
+template <int NM>
+struct FxRow {
+    Fx v[NM];
+};
+template <int NM>
+__device__ __forceinline__ void fx_column(const long long (&S)[NM], Fx y, int t, Fx nl1, Fx nl2, FxRow<NM> &r,
+                                          unsigned &bad) {
+    r.v[0] = fx_split(fx_scaled(S[0], t, y, bad));
+    bad |= fx_beyond_h(r.v[0]);
+    if constexpr (NM == 3) {
+        const Fx a = r.v[0];
+        const Fx p = r.v[1] =
+            fx_split(fx_scaled(fx_hi(fx_sum(S[1], fx_mid(FX_HALF, a, nl1)), a, nl1), t, y, bad));
+        bad |= fx_beyond_h(p);
+        long long v = fx_sum(S[2], fx_mid(fx_mid(FX_HALF, a, nl2), p, fx_twice(nl1)));
+        v = fx_hi(fx_hi(fx_hi(v, a, nl2), p, nl1), p, nl1);
+        r.v[2] = fx_split(fx_scaled(v, t, y, bad));
+        bad |= fx_beyond_h(r.v[2]);
+    }
+}
+
+// The next column's S of a row, less the products with this column: (na, nb,
+// ne) are -L, -L1, -L2 of the next column's own row in this column.
+template <int NM>
+__device__ __forceinline__ void fx_update(long long (&S)[NM], const FxRow<NM> &r, Fx na, Fx nb, Fx ne) {
+    const Fx a = r.v[0];
+    S[0] = fx_hi(fx_sum(S[0], fx_mid(FX_HALF, a, na)), a, na);
+    if constexpr (NM == 3) {
+        const Fx p = r.v[1], q = r.v[2];
+        S[1] = fx_sum(S[1], fx_mid(fx_mid(FX_HALF, p, na), a, nb));
+        S[1] = fx_hi(fx_hi(S[1], p, na), a, nb);
+        S[2] = fx_sum(S[2], fx_mid(fx_mid(fx_mid(FX_HALF, q, na), a, ne), p, fx_twice(nb)));
+        S[2] = fx_hi(fx_hi(fx_hi(fx_hi(S[2], q, na), a, ne), p, nb), p, nb);
+    }
+}
+
+// hi += x_h y_h, mid += x_h y_l + x_l y_h
+__device__ __forceinline__ void fx_acc(long long &hi, long long &mid, int xh, int xl, int yh, int yl) {
+    hi = fx_mad(xh, yh, hi);
+    mid = fx_mad(xl, yh, fx_mad(xh, yl, mid));
+}
+
+// The sums of columns c, c + 1 over k < c, subtracted from the rows below the
+// diagonal block, by the warps 1 and up.  2^KL lanes share a row's sum.
+template <int NM, int KL>
+__device__ __forceinline__ void fx_sums(const FxFactor &F, int c, int lane, int warp) {
+    constexpr int RP = 32 >> KL, KS = 1 << KL;  // row pairs and shares of a warp
+    const int m = F.m, n = F.n;
+    const int rp = lane & (RP - 1), ks = lane / RP;
+    for (int base = min(c + 2, n) + (warp - 1) * 2 * RP; base < m; base += (FXW - 1) * 2 * RP) {
+        const int iA = base + rp, iB = iA + RP;
+        const int ia = min(iA, m - 1), ib = min(iB, m - 1), j1 = min(c + 1, m - 1);
+        long long hi[NM][2][2], mid[NM][2][2];
+#pragma unroll
+        for (int g = 0; g < NM; g++)
+#pragma unroll
+            for (int x = 0; x < 4; x++) hi[g][x >> 1][x & 1] = mid[g][x >> 1][x & 1] = 0;
+        int off = ks * (m - 1) - ks * ks;
+        int inc = KS * (m - 1) - 2 * ks * KS - KS * KS;
+        for (int q = ks; q < (c >> 1); q += KS) {
+            int4 r[NM][2], s[NM][2];
+#pragma unroll
+            for (int g = 0; g < NM; g++) {
+                const int4 *P = fx_mat(F, g) + off;
+                r[g][0] = P[ia];
+                r[g][1] = P[ib];
+                s[g][0] = P[c];
+                s[g][1] = P[j1];
+            }
+            off += inc;
+            inc -= 2 * KS * KS;
+#pragma unroll
+            for (int x = 0; x < 2; x++)
+#pragma unroll
+                for (int y = 0; y < 2; y++)
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        const int x0h = k ? r[0][x].z : r[0][x].x, x0l = k ? r[0][x].w : r[0][x].y;
+                        const int y0h = k ? s[0][y].z : s[0][y].x, y0l = k ? s[0][y].w : s[0][y].y;
+                        fx_acc(hi[0][x][y], mid[0][x][y], x0h, x0l, y0h, y0l);
+                        if constexpr (NM == 3) {
+                            const int x1h = k ? r[1][x].z : r[1][x].x, x1l = k ? r[1][x].w : r[1][x].y;
+                            const int y1h = k ? s[1][y].z : s[1][y].x, y1l = k ? s[1][y].w : s[1][y].y;
+                            const int x2h = k ? r[2][x].z : r[2][x].x, x2l = k ? r[2][x].w : r[2][x].y;
+                            const int y2h = k ? s[2][y].z : s[2][y].x, y2l = k ? s[2][y].w : s[2][y].y;
+                            fx_acc(hi[1][x][y], mid[1][x][y], x1h, x1l, y0h, y0l);
+                            fx_acc(hi[1][x][y], mid[1][x][y], x0h, x0l, y1h, y1l);
+                            fx_acc(hi[2][x][y], mid[2][x][y], x2h, x2l, y0h, y0l);
+                            fx_acc(hi[2][x][y], mid[2][x][y], x0h, x0l, y2h, y2l);
+                            fx_acc(hi[2][x][y], mid[2][x][y], x1h, x1l, 2 * y1h, 2 * y1l);
+                        }
+                    }
+        }
+        // the shares added up: first the columns, then the rows of the tile
+        // are split between lanes (half of the values change hands), then
+        // whole values
+        long long v[NM];
+#pragma unroll
+        for (int g = 0; g < NM; g++) {
+            long long w[2];
+#pragma unroll
+            for (int x = 0; x < 2; x++) {
+                const long long v0 = (hi[g][x][0] << 1) + (mid[g][x][0] >> 29);
+                const long long v1 = (hi[g][x][1] << 1) + (mid[g][x][1] >> 29);
+                w[x] = (ks & 1 ? v1 : v0) + __shfl_xor_sync(LAGP_FULL_MASK, ks & 1 ? v0 : v1, RP);
+            }
+            v[g] = (ks & 2 ? w[1] : w[0]) + __shfl_xor_sync(LAGP_FULL_MASK, ks & 2 ? w[0] : w[1], 2 * RP);
+#pragma unroll
+            for (int o = 4 * RP; o < 32; o <<= 1) v[g] += __shfl_xor_sync(LAGP_FULL_MASK, v[g], o);
+        }
+        const int i = ks & 2 ? iB : iA, j = c + (ks & 1);
+        if (ks < 4 && i < m && j < n) {
+            const int slot = fx_slot(i, j, m);
+#pragma unroll
+            for (int g = 0; g < NM; g++) *fx_raw(F, g, slot) -= v[g];
+        }
+    }
+}
+
+// The diagonal block of columns c, c + 1, one warp: the sums of its three
+// entries (eight lanes an entry), then the block's factor, every lane the same.
+template <int NM>
+__device__ __forceinline__ void fx_diagonal(const FxFactor &F, FxDiag *diag, int *flag, int c, int lane) {
+    const int n = F.n, m = F.m;
+    const bool two = c + 1 < n;
+    const int slot[3] = {fx_slot(c, c, m), fx_slot(c + 1, c, m), fx_slot(c + 1, c + 1, m)};
+    long long S[3][NM];  // entries (c, c), (c + 1, c), (c + 1, c + 1)
+#pragma unroll
+    for (int g = 0; g < NM; g++)
+#pragma unroll
+        for (int e = 0; e < 3; e++) S[e][g] = e && !two ? 0 : *fx_raw(F, g, slot[e]);
+    if (c > 0) {
+        const int e = lane >> 3, ks = lane & 7;
+        const int row = min(e == 0 ? c : c + 1, m - 1), col = min(e == 2 ? c + 1 : c, m - 1);
+        long long hi[NM], mid[NM];
+#pragma unroll
+        for (int g = 0; g < NM; g++) hi[g] = mid[g] = 0;
+        for (int q = ks; q < (c >> 1); q += 8) {
+            const int off = q * (m - 1) - q * q;
+            int4 r[NM], s[NM];
+#pragma unroll
+            for (int g = 0; g < NM; g++) {
+                const int4 *P = fx_mat(F, g) + off;
+                r[g] = P[row];
+                s[g] = P[col];
+            }
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const int x0h = k ? r[0].z : r[0].x, x0l = k ? r[0].w : r[0].y;
+                const int y0h = k ? s[0].z : s[0].x, y0l = k ? s[0].w : s[0].y;
+                fx_acc(hi[0], mid[0], x0h, x0l, y0h, y0l);
+                if constexpr (NM == 3) {
+                    const int x1h = k ? r[1].z : r[1].x, x1l = k ? r[1].w : r[1].y;
+                    const int y1h = k ? s[1].z : s[1].x, y1l = k ? s[1].w : s[1].y;
+                    const int x2h = k ? r[2].z : r[2].x, x2l = k ? r[2].w : r[2].y;
+                    const int y2h = k ? s[2].z : s[2].x, y2l = k ? s[2].w : s[2].y;
+                    fx_acc(hi[1], mid[1], x1h, x1l, y0h, y0l);
+                    fx_acc(hi[1], mid[1], x0h, x0l, y1h, y1l);
+                    fx_acc(hi[2], mid[2], x2h, x2l, y0h, y0l);
+                    fx_acc(hi[2], mid[2], x0h, x0l, y2h, y2l);
+                    fx_acc(hi[2], mid[2], x1h, x1l, 2 * y1h, 2 * y1l);
+                }
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < NM; g++) {
+            long long v = (hi[g] << 1) + (mid[g] >> 29);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(LAGP_FULL_MASK, v, o);
+#pragma unroll
+            for (int x = 0; x < 3; x++) S[x][g] -= __shfl_sync(LAGP_FULL_MASK, v, 8 * x);
+        }
+    }
+    unsigned bad = 0;
+    FxDiag D;
+    auto pivot = [&](int j, const long long (&s)[NM]) {
+        long long s0 = s[0], l;
+        // (a pivot below 2^-47, or not positive, is for FP64 to judge)
+        const bool odd = s0 < (1ll << 12) || s0 >= (1ll << 60);
+        bad |= odd;
+        if (odd) s0 = FX_ONE;
+        D.y[j] = fx_rsqrt(s0, &D.t[j], &l);
+        const int at = slot[2 * j];
+        if (lane == 0) {
+            fx_store(F, 0, at, fx_split(l));
+            fx_ry(F)[c + j] = fx_join(D.y[j]);
+            fx_rt(F)[c + j] = D.t[j];
+        }
+        if constexpr (NM == 3) {
+            const Fx l1 = fx_split(fx_scaled(s[1], D.t[j], D.y[j], bad) >> 1);  // (below 1.42)
+            D.nl1[j] = fx_neg(l1);
+            const long long v = fx_hi(fx_sum(s[2] >> 1, fx_mid(FX_HALF, l1, D.nl1[j])), l1, D.nl1[j]);
+            const Fx l2 = fx_split(fx_scaled(v, D.t[j], D.y[j], bad));
+            bad |= fx_beyond_h(l2);
+            D.nl2[j] = fx_neg(l2);
+            if (lane == 0) {
+                fx_store(F, 1, at, l1);
+                fx_store(F, 2, at, l2);
+            }
+        }
+    };
+    __syncwarp();  // every lane has read the entries that are written now
+    pivot(0, S[0]);
+    if (two) {
+        FxRow<NM> r;
+        fx_column<NM>(S[1], D.y[0], D.t[0], D.nl1[0], D.nl2[0], r, bad);
+        D.na = fx_neg(r.v[0]);
+        if constexpr (NM == 3) {
+            D.nb = fx_neg(r.v[1]);
+            D.ne = fx_neg(r.v[2]);
+        }
+        fx_update<NM>(S[2], r, D.na, D.nb, D.ne);
+#pragma unroll
+        for (int g = 0; g < NM; g++)
+            if (lane == 0) fx_store(F, g, slot[1], r.v[g]);
+        pivot(1, S[2]);
+    }
+    if (lane == 0) {
+        *diag = D;
+        if (bad) atomicOr(flag, 1);
+    }
+}
+
+// The factorisation (and its derivatives for NM = 3), in place; shared memory holds
+// the raw values on entry and the limbs of L (L1, L2) after.  Two phases a
+// pair of columns: one thread a row finishes the two columns, then one warp
+// makes the next diagonal block (a serial chain of some 1,500 cycles) while
+// the others form the sums of the next two columns.  Returns the flag
+// (block-uniform).
+template <int NM>
+__device__ int fx_factorise(const FxFactor &F, const Blk &b) {
+    const int n = F.n, m = F.m;
+    __shared__ FxDiag s_diag;
+    __shared__ int s_out;
+    if (b.tid == 0) s_out = 0;
+    __syncthreads();
+    if (b.warp == 0) fx_diagonal<NM>(F, &s_diag, &s_out, 0, b.lane);
+    __syncthreads();
+    for (int c = 0; c < n; c += 2) {
+        const bool two = c + 1 < n;
+        const FxDiag D = s_diag;
+        // (rows from warp 1 on: warp 0 has the serial chains)
+        for (int i = c + (two ? 2 : 1) + (b.warp + FXW - 1) % FXW * 32 + b.lane; i < m; i += FXT) {
+            unsigned bad = 0;
+            const int at = fx_slot(i, c, m);  // columns c, c + 1 of a row are adjacent
+            long long S[NM], T[NM];
+#pragma unroll
+            for (int g = 0; g < NM; g++) {
+                const longlong2 v = *reinterpret_cast<const longlong2 *>(fx_raw(F, g, at));
+                S[g] = v.x;
+                T[g] = v.y;
+            }
+            FxRow<NM> r, q;
+            fx_column<NM>(S, D.y[0], D.t[0], D.nl1[0], D.nl2[0], r, bad);
+            if (two) {
+                fx_update<NM>(T, r, D.na, D.nb, D.ne);
+                fx_column<NM>(T, D.y[1], D.t[1], D.nl1[1], D.nl2[1], q, bad);
+            }
+            // |x| < 1 in the further rows, whose norm nothing bounds
+            if (i >= n)
+#pragma unroll
+                for (int g = 0; g < NM; g++) {
+                    bad |= (unsigned)(r.v[g].h + (1 << 29)) >> 30;
+                    if (two) bad |= (unsigned)(q.v[g].h + (1 << 29)) >> 30;
+                }
+#pragma unroll
+            for (int g = 0; g < NM; g++) {
+                if (two)
+                    *reinterpret_cast<int4 *>(fx_raw(F, g, at)) = make_int4(r.v[g].h, r.v[g].l, q.v[g].h, q.v[g].l);
+                else
+                    fx_store(F, g, at, r.v[g]);
+            }
+            if (bad) atomicOr(&s_out, 1);
+        }
+        __syncthreads();
+        if (c + 2 < n) {
+            const int R = m - (c + 4);
+            if (b.warp == 0) fx_diagonal<NM>(F, &s_diag, &s_out, c + 2, b.lane);
+            else if (R > 24) fx_sums<NM, 2>(F, c + 2, b.lane, b.warp);
+            else if (R > 12) fx_sums<NM, 3>(F, c + 2, b.lane, b.warp);
+            else fx_sums<NM, 4>(F, c + 2, b.lane, b.warp);
+            __syncthreads();
+        }
+    }
+    return s_out;
+}
+
+// Exponent e with max_i |v_i| < 2^e over the block's n values (INT_MAX when
+// one is not finite or all are zero); red: FXW ints.
+__device__ int fx_exponent(const double *v, int n, int *red, const Blk &b) {
+    int top = 0;
+    __syncthreads();
+    for (int i = b.tid; i < n; i += FXT) top = max(top, (__double2hiint(v[i]) >> 20) & 0x7ff);
+    top = __reduce_max_sync(LAGP_FULL_MASK, top);
+    if (b.lane == 0) red[b.warp] = top;
+    __syncthreads();
+    top = max(max(red[0], red[1]), max(red[2], red[3]));
+    __syncthreads();
+    // (subnormal responses and those near the largest double: FP64 kernels)
+    return top < 64 || top > 1983 ? INT32_MAX : top - 1022;
+}
+
+// x 2^e by the exponent field (x = 0 or a result out of range: 0)
+__device__ __forceinline__ double fx_shift(double x, int e) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    return ex == 0 || ex + e <= 0 ? 0.0 : __hiloint2double(hi + (e << 20), __double2loint(x));
+}
+
+__device__ __forceinline__ void fx_tri(int e, int &i, int &k) {  // e-th entry of a lower triangle by rows
+    int r = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+    if ((r + 1) * (r + 2) / 2 <= e) r++;
+    if (r * (r + 1) / 2 > e) r--;
+    i = r;
+    k = e - r * (r + 1) / 2;
+}
+
+struct FxLaunch {
+    int cls_lo, cls_hi;   // this launch takes the locations with cls_lo < n <= cls_hi
+    bool stray;           // and those whose n is out of range
+    int words;            // matrix words for n = cls_hi
+    int *counter, *redo;  // work counter; number of locations left to the FP64 kernels
+    double *dist;         // per CTA: squared distances of the design (MLE)
+};
+
+__device__ __forceinline__ bool fx_mine(const FxLaunch &f, int nm, int nmax) {
+    if (nm < 1 || nm > nmax) return f.stray;
+    return nm > f.cls_lo && nm <= f.cls_hi;
+}
+
+// ------------------------------------------------------------------ predict
+
+__global__ void __launch_bounds__(FXT)
+predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *mean, double *s2, double *df,
+                  int32_t *status) {
+    const int nmax = f.cls_hi, p = a.p;
+    double *y = reinterpret_cast<double *>(fx_smem + f.words * 16);
+    double *xd = y + 3 * nmax, *xq = xd + nmax * p, *kx = xq + p;  // (after y: the pivots)
+    __shared__ int s_loc, s_flag, red[FXW];
+    const Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
+    for (;;) {
+        if (b.tid == 0) s_loc = atomicAdd(f.counter, 1);
+        __syncthreads();
+        const int64_t loc = s_loc;
+        __syncthreads();
+        if (loc >= a.M) break;
+        const int nm = a.n ? a.n[loc] : a.nmax;
+        if (!fx_mine(f, nm, a.nmax)) continue;
+        int st = load_design(a, loc, nm, dv, xd, y, &s_flag, b);
+        double mu = CUDART_NAN, sv = CUDART_NAN, dfv = CUDART_NAN;
+        if (st == LAGP_OK) {
+            const double d = dv[loc], g = a.g, ninv_d = -1.0 / d;
+            for (int i = b.tid; i < p; i += FXT) xq[i] = load_coord64(a.Xref, loc, p, i, a.dtype);
+            __syncthreads();
+            const int m = nm + 2;
+            const FxFactor F{f.words, nm, m, f.words * 16, nmax};
+            st = FX_REDO;
+            int zs = 0, ws = 0;
+            for (int wide = 0; wide < 2 && st != LAGP_OK; wide++) {
+                bool odd = false;  // a distance that is not finite
+                for (int e = b.tid; e < nm * (nm + 1) / 2 + nm; e += FXT) {
+                    int i, k;
+                    fx_tri(e, i, k);
+                    const bool cross = i >= nm;
+                    const double D = sqd(cross ? xq : xd + (size_t)i * p, xd + (size_t)k * p, p);
+                    odd |= !(D < CUDART_INF);
+                    const double E = exp64_tang(D * ninv_d, exp64_table_g);
+                    if (cross) kx[k] = E;
+                    else *fx_raw(F, 0, fx_slot(i, k, m)) = fx_from(i == k ? E + g : E);
+                }
+                const int ex = fx_exponent(kx, nm, red, b), ey = fx_exponent(y, nm, red, b);
+                if (__syncthreads_or(odd) || ex == INT32_MAX || ey == INT32_MAX) break;
+                zs = ey + (wide ? FX_Z1 : FX_Z0);
+                ws = ex + 2;
+                for (int k = b.tid; k < nm; k += FXT) {
+                    *fx_raw(F, 0, fx_slot(nm, k, m)) = fx_from(fx_shift(y[k], -zs));
+                    *fx_raw(F, 0, fx_slot(nm + 1, k, m)) = fx_from(fx_shift(kx[k], -ws));
+                }
+                if (!fx_factorise<1>(F, b)) st = LAGP_OK;
+            }
+            if (st == LAGP_OK) {
+                double v[3] = {0.0, 0.0, 0.0};
+                for (int i = b.tid; i < nm; i += FXT) {
+                    const double z = fx_double(fx_load(F, 0, fx_slot(nm, i, m)));
+                    const double w = fx_double(fx_load(F, 0, fx_slot(nm + 1, i, m)));
+                    v[0] = fma(w, z, v[0]);
+                    v[1] = fma(z, z, v[1]);
+                    v[2] = fma(w, w, v[2]);
+                }
+                block_sums<3>(v, b);
+                mu = scalbn(v[0], zs + ws);
+                const double psi = scalbn(v[1], 2 * zs), kk = scalbn(v[2], 2 * ws);
+                sv = psi * ((1.0 + g) - kk) / nm;
+                dfv = nm;
+            }
+        }
+        if (b.tid == 0) {
+            if (st == FX_REDO) atomicAdd(f.redo, 1);
+            mean[loc] = mu;
+            s2[loc] = sv;
+            df[loc] = dfv;
+            status[loc] = st;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------- MLE
+
+struct FxEval {
+    double l, dl, d2l;
+    int flag;  // fx_factorise's
+};
+
+// l, l', l'' of Eq. (gpk) at d from the packed squared distances; zs: the
+// power of two that z is scaled by; lgam: log Gamma(n/2) - (n/2) log 2 pi.
+__device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, double d, double g, int zs,
+                          double lgam, const Blk &b) {
+    const int n = F.n, m = F.m;
+    const double ninv_d = -1.0 / d;
+    for (int e = b.tid; e < n * (n + 1) / 2; e += FXT) {
+        int i, k;
+        fx_tri(e, i, k);
+        const double t = -(dist[e] * ninv_d);
+        const double E = exp64_tang(-t, exp64_table_g);
+        const double K1 = E > 0.0 ? t * E : 0.0, K2 = E > 0.0 ? K1 * (t - 2.0) : 0.0;
+        const int s = fx_slot(i, k, m);
+        *fx_raw(F, 0, s) = fx_from(i == k ? E + g : E);
+        *fx_raw(F, 1, s) = fx_from(K1);
+        *fx_raw(F, 2, s) = fx_from(K2);
+    }
+    for (int k = b.tid; k < n; k += FXT) {
+        const int s = fx_slot(n, k, m);
+        *fx_raw(F, 0, s) = fx_from(fx_shift(fx_y(F)[k], -zs));
+        *fx_raw(F, 1, s) = 0;
+        *fx_raw(F, 2, s) = 0;
+    }
+    FxEval r;
+    r.flag = fx_factorise<3>(F, b);
+    r.l = r.dl = r.d2l = CUDART_NAN;
+    if (r.flag) return r;
+    // log|K| = -2 log prod r, r = 1 / l = y 2^t with y in (0.7, 1.42]: the
+    // product of a warp's y stays in range, one logarithm for all
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    double prod = 1.0;
+    for (int i = b.tid; i < n; i += FXT) {
+        const double yr = fx_double(fx_ry(F)[i]), ri = fx_shift(yr, fx_rt(F)[i]);
+        prod *= yr;
+        v[0] += fx_rt(F)[i];
+        const int s = fx_slot(i, i, m), z = fx_slot(n, i, m);
+        const double p1 = fx_double(fx_load(F, 1, s)) * ri, p2 = fx_double(fx_load(F, 2, s)) * ri;
+        const double z0 = fx_double(fx_load(F, 0, z)), z1 = fx_double(fx_load(F, 1, z)),
+                     z2 = fx_double(fx_load(F, 2, z));
+        v[1] += p1;                       // (d/dlog d) sum log l
+        v[2] += fma(-p1, p1, p2);
+        v[3] = fma(z0, z0, v[3]);         // psi and its derivatives (scaled)
+        v[4] = fma(2.0 * z0, z1, v[4]);
+        v[5] = fma(2.0 * z1, z1, fma(2.0 * z0, z2, v[5]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) prod *= __shfl_xor_sync(LAGP_FULL_MASK, prod, o);
+    __shared__ double s_prod[FXW];
+    if (b.lane == 0) s_prod[b.warp] = prod;
+    block_sums<6>(v, b);  // (its barriers order s_prod)
+    __shared__ FxEval s_r;
+    if (b.warp == 0) {
+        // the two logarithms side by side, the other scalars on every lane
+        const double arg = b.lane ? scalbn(v[3], 2 * zs) / 2.0 : (s_prod[0] * s_prod[1]) * (s_prod[2] * s_prod[3]);
+        const double lg = log(arg);
+        const double half_logdet = -(__shfl_sync(LAGP_FULL_MASK, lg, 0) + v[0] * CUDART_LN2);
+        const double logpsi = __shfl_sync(LAGP_FULL_MASK, lg, 1);
+        const double hn = 0.5 * n, ipsi = 1.0 / v[3], id = -ninv_d, q1 = v[4] * ipsi;
+        if (b.lane == 0) {
+            s_r.l = lgam - half_logdet - hn * logpsi;
+            s_r.dl = (-v[1] - hn * q1) * id;
+            s_r.d2l = (-v[2] - hn * fma(-q1, q1, v[5] * ipsi)) * id * id;
+        }
+    }
+    __syncthreads();
+    FxEval o = s_r;
+    o.flag = 0;
+    return o;
+}
+
+__global__ void __launch_bounds__(FXT, 4)
+mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int max_iter, MleOut o,
+              unsigned long long *work) {
+    const int nmax = f.cls_hi, p = a.p;
+    double *xd = reinterpret_cast<double *>(fx_smem);  // before the matrices are filled
+    const int y_at = (int)max(3 * f.words * 16, (nmax * p * 8 + 15) & ~15);
+    double *y = reinterpret_cast<double *>(fx_smem + y_at);
+    double *dist = f.dist + (size_t)blockIdx.x * (nmax * (nmax + 1) / 2);
+    __shared__ int s_loc, s_flag, red[FXW];
+    __shared__ double s_lgam;
+    const Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
+    unsigned long long n_llik = 0, n_derivs = 0;  // evaluations x n^3 (thread 0's count)
+    for (;;) {
+        if (b.tid == 0) s_loc = atomicAdd(f.counter, 1);
+        __syncthreads();
+        const int64_t loc = s_loc;
+        __syncthreads();
+        if (loc >= a.M) break;
+        const int nm = a.n ? a.n[loc] : a.nmax;
+        if (!fx_mine(f, nm, a.nmax)) continue;
+        int st = load_design(a, loc, nm, dv, xd, y, &s_flag, b);
+        const unsigned long long n3 = (unsigned long long)nm * nm * nm;
+        FxEval r{CUDART_NAN, CUDART_NAN, CUDART_NAN, 0};
+        int it = 0;
+        double d = dv[loc];
+        if (st == LAGP_OK) {
+            const double g = a.g;
+            d = fmin(fmax(d, dmin), dmax);
+            bool odd = false;
+            for (int e = b.tid; e < nm * (nm + 1) / 2; e += FXT) {
+                int i, k;
+                fx_tri(e, i, k);
+                const double D = sqd(xd + (size_t)i * p, xd + (size_t)k * p, p);
+                odd |= !(D < CUDART_INF);
+                dist[e] = D;  // read back by this thread only
+            }
+            if (b.tid == 0) {
+                const double hn = 0.5 * nm;
+                s_lgam = lgamma(hn) - hn * log(2.0 * CUDART_PI);
+            }
+            const int ey = fx_exponent(y, nm, red, b);
+            odd = __syncthreads_or(odd) || ey == INT32_MAX;
+            const double lgam = s_lgam;
+            const FxFactor F{f.words, nm, nm + 1, y_at, nmax};
+            int zs = ey + FX_Z0;
+            // one evaluation; out of range: once more with a wider z
+            auto eval = [&](double at) {
+                FxEval q = fx_llik(F, dist, at, g, zs, lgam, b);
+                if (q.flag && zs < ey + FX_Z1) {
+                    zs = ey + FX_Z1;
+                    q = fx_llik(F, dist, at, g, zs, lgam, b);
+                }
+                return q;
+            };
+            unsigned long long ll = 0, de = 0;
+            if (odd) {
+                st = FX_REDO;
+            } else {
+                r = eval(d);
+                ll += n3;
+                if (r.flag) {
+                    st = FX_REDO;
+                } else {
+                    de += n3;
+                    while (it < max_iter) {
+                        it++;
+                        double delta;
+                        if (r.d2l < 0.0) delta = -r.dl / r.d2l;
+                        else delta = (r.dl > 0.0) ? d : -0.5 * d;
+                        bool accepted = false;
+                        double dn = d;
+                        FxEval t = r;
+                        // a short Newton step near the maximiser raises l below the
+                        // FP64 resolution of l: taken without comparing l values
+                        const bool short_newton = r.d2l < 0.0 && fabs(delta) <= 1e-3 * d;
+                        for (int h = 0; h <= 20; h++) {
+                            dn = fmin(fmax(d + delta, dmin), dmax);
+                            t = eval(dn);
+                            ll += n3;
+                            if (t.flag) break;
+                            if (short_newton || t.l >= r.l) {
+                                accepted = true;
+                                break;
+                            }
+                            delta *= 0.5;
+                        }
+                        if (t.flag) {
+                            st = FX_REDO;
+                            break;
+                        }
+                        if (!accepted) break;
+                        const double step = fabs(dn - d);
+                        d = dn;
+                        r = t;
+                        de += n3;
+                        if (step < 1e-10 * d) break;
+                    }
+                }
+            }
+            if (st != FX_REDO) {
+                n_llik += ll;
+                n_derivs += de;
+            }
+        }
+        if (b.tid == 0) {
+            const bool ok = st == LAGP_OK;
+            if (st == FX_REDO) atomicAdd(f.redo, 1);
+            if (ok) dv[loc] = d;
+            if (o.llik) o.llik[loc] = ok ? r.l : CUDART_NAN;
+            if (o.dllik) o.dllik[loc] = ok ? r.dl : CUDART_NAN;
+            if (o.d2llik) o.d2llik[loc] = ok ? r.d2l : CUDART_NAN;
+            if (o.iters) o.iters[loc] = it;
+            o.status[loc] = st;
+        }
+        __syncthreads();
+    }
+    if (b.tid == 0 && work) {
+        atomicAdd(work, n_llik);
+        atomicAdd(work + 1, n_derivs);
+    }
+}
+
+size_t fx_predict_smem(int n, int p) {
+    return (size_t)fx_words(n, n + 2) * 16 + ((size_t)n * p + p + 4 * (size_t)n) * 8;
+}
+size_t fx_mle_smem(int n, int p) {
+    const size_t area = std::max((size_t)3 * fx_words(n, n + 1) * 16, (size_t)n * p * 8);
+    return area + (size_t)n * 20 + 64;
+}
+
+// Upper ends of the size classes: one launch a class, so that a location's
+// shared memory (n^2, 48 KB at n = 60 for the MLE) follows its own design size
+// and not the largest one's.
+constexpr int FX_CLASSES[] = {40, 64, 80, 104, 128};
+
+// Calls fn(lo, hi, first) for every class of sizes up to nmax, the largest
+// first (one class when all locations have the same size).
+template <typename Fn>
+lagp_status fx_each_class(const GpArgs &a, Fn fn) {
+    if (!a.n) return fn(0, a.nmax, true);
+    int hi = a.nmax;
+    bool first = true;
+    for (int c = (int)(sizeof FX_CLASSES / sizeof *FX_CLASSES) - 1; c >= 0; c--) {
+        const int lo = c ? FX_CLASSES[c - 1] : 0;
+        if (hi <= lo) continue;
+        LAGP_TRY(fn(lo, hi, first));
+        first = false;
+        hi = lo;
+    }
+    return LAGP_OK;
+}
+
+template <typename Kern>
+int fx_grid(lagp_ctx *ctx, Kern kern, size_t smem, int64_t M) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, FXT, smem);
+    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * std::max(occ, 1), M));
+}
+
+}  // namespace
+
+bool gp_fixed_supported(lagp_ctx *ctx, const GpArgs &a, bool mle) {
+    if (a.nmax > FX_NMAX || !(a.g < 1.0)) return false;
+    return (mle ? fx_mle_smem(a.nmax, a.p) : fx_predict_smem(a.nmax, a.p)) + 2048 <= ctx->smem_optin;
+}
+
+size_t gp_fixed_workspace(lagp_ctx *ctx, const GpArgs &a) {
+    return (size_t)ctx->num_sms * 16 * ((size_t)a.nmax * (a.nmax + 1) / 2) * 8;
+}
+
+lagp_status launch_predict_fixed(lagp_ctx *ctx, const GpArgs &a, const double *d, double *mean, double *s2,
+                                 double *df, int32_t *status, int *counters, int *redo) {
+    return fx_each_class(a, [&](int lo, int hi, bool first) -> lagp_status {
+        const size_t smem = fx_predict_smem(hi, a.p);
+        const int grid = fx_grid(ctx, predict_fx_kernel, smem, a.M);
+        const FxLaunch f{lo, hi, first, fx_words(hi, hi + 2), counters++, redo, nullptr};
+        predict_fx_kernel<<<grid, FXT, smem, ctx->stream>>>(a, f, d, mean, s2, df, status);
+        ctx->launches++;
+        return lagp_cuda_check(ctx, cudaGetLastError(), "predict_fx_kernel");
+    });
+}
+
+lagp_status launch_mle_fixed(lagp_ctx *ctx, const GpArgs &a, double *d, double dmin, double dmax, int32_t max_iter,
+                             const MleOut &o, unsigned long long *work, double *ws, int *counters, int *redo) {
+    return fx_each_class(a, [&](int lo, int hi, bool first) -> lagp_status {
+        const size_t smem = fx_mle_smem(hi, a.p);
+        const int grid = std::min(fx_grid(ctx, mle_fx_kernel, smem, a.M), ctx->num_sms * 16);
+        const FxLaunch f{lo, hi, first, fx_words(hi, hi + 1), counters++, redo, ws};
+        mle_fx_kernel<<<grid, FXT, smem, ctx->stream>>>(a, f, d, dmin, dmax, max_iter, o, work);
+        ctx->launches++;
+        return lagp_cuda_check(ctx, cudaGetLastError(), "mle_fx_kernel");
+    });
+}

@@ -17,18 +17,14 @@
 // live in a per-CTA global workspace (L2-resident), vectors in shared memory.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "device_util.cuh"
 #include "exp64.cuh"
+#include "gp_common.cuh"
 #include "lagp_internal.h"
 
 namespace {
-
-constexpr int GP_THREADS = 128;
-constexpr int GP_WARPS = GP_THREADS / 32;
-
-struct Blk {
-    int tid, lane, warp;
-};
 
 __device__ double block_sum(double v, double *red, const Blk &b) {
     v = warp_sum(v);
@@ -38,28 +34,6 @@ __device__ double block_sum(double v, double *red, const Blk &b) {
     double s = 0.0;
     for (int w = 0; w < GP_WARPS; w++) s += red[w];
     return s;
-}
-
-// Block sums of NV values at once: warp sums, then one warp adds the warps'
-// partials (not every thread); three barriers for all NV.
-template <int NV>
-__device__ void block_sums(double (&v)[NV], const Blk &b) {
-    __shared__ double part[GP_WARPS * NV], tot[NV];
-#pragma unroll
-    for (int i = 0; i < NV; i++) v[i] = warp_sum(v[i]);
-    __syncthreads();  // earlier readers of part / tot are done
-    if (b.lane == 0)
-#pragma unroll
-        for (int i = 0; i < NV; i++) part[b.warp * NV + i] = v[i];
-    __syncthreads();
-    if (b.warp == 0 && b.lane < NV) {
-        double t = 0.0;
-        for (int w = 0; w < GP_WARPS; w++) t += part[w * NV + b.lane];
-        tot[b.lane] = t;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < NV; i++) v[i] = tot[i];
 }
 
 // Lower Cholesky factor L of the symmetric n x n matrix A (lower triangle
@@ -161,42 +135,6 @@ __device__ void warp_backward(const double *L, int ld, const double *rd, const d
 struct GpWork {
     double *D, *K, *L, *Li, *Ki, *A1;  // n x ld each
 };
-
-// Validate a location and load its design; returns the per-location status.
-__device__ int load_design(const GpArgs &a, int64_t loc, int nm, const double *dptr, double *xd,
-                           double *y, int *flag, const Blk &b) {
-    if (b.tid == 0) *flag = LAGP_OK;
-    __syncthreads();
-    const double d = dptr ? dptr[loc] : 1.0;
-    if (b.tid == 0 && (nm < 1 || nm > a.nmax || !(d > 0.0) || !isfinite(d))) *flag = LAGP_EINVAL;
-    __syncthreads();
-    if (*flag != LAGP_OK) return *flag;
-    const int32_t *s = a.sel + loc * a.nmax;
-    for (int t = b.tid; t < nm; t += GP_THREADS) {
-        int32_t r = s[t];
-        if (r < 0 || r >= a.N) *flag = LAGP_EINVAL;
-    }
-    __syncthreads();
-    if (*flag != LAGP_OK) return *flag;
-    for (int e = b.tid; e < nm * a.p; e += GP_THREADS) {
-        int t = e / a.p, i = e - t * a.p;
-        xd[e] = load_coord64(a.X, s[t], a.p, i, a.dtype);
-    }
-    for (int t = b.tid; t < nm; t += GP_THREADS)
-        y[t] = a.dtype == LAGP_F64 ? static_cast<const double *>(a.Y)[s[t]]
-                                   : (double)static_cast<const float *>(a.Y)[s[t]];
-    __syncthreads();
-    return LAGP_OK;
-}
-
-__device__ double sqd(const double *u, const double *v, int p) {
-    double s = 0.0;
-    for (int i = 0; i < p; i++) {
-        double df = u[i] - v[i];
-        s = fma(df, df, s);
-    }
-    return s;
-}
 
 // Row i and column k <= i of the e-th element of a lower triangle stored by rows.
 __device__ __forceinline__ void tri_index(int e, int &i, int &k) {
@@ -494,9 +432,10 @@ __device__ GpWork work_for_block(double *ws, int nmax, int ld) {
 // ------------------------------------------------------------------ predict
 
 __global__ void __launch_bounds__(GP_THREADS)
-predict_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, double *mean,
-               double *s2, double *df, int32_t *status) {
+predict_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, const int *redo,
+               double *mean, double *s2, double *df, int32_t *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (redo && *redo == 0) return;  // (after the fixed-point kernel: the locations it left)
     const int nmax = a.nmax, p = a.p, ld = (nmax + 31) & ~31;
     GpShared S = carve(smem_raw, nmax, p);
     for (int i = threadIdx.x; i < EXP64_TABLE_SIZE; i += GP_THREADS) S.etab[i] = exp64_table_g[i];  // ordered by the loop's first barrier
@@ -509,6 +448,7 @@ predict_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws
         const int64_t loc = s_loc;
         __syncthreads();
         if (loc >= a.M) break;
+        if (redo && status[loc] != FX_REDO) continue;
         const int nm = a.n ? a.n[loc] : nmax;
         int st = load_design(a, loc, nm, dv, S.xd, S.y, &s_flag, b);
         double mu = CUDART_NAN, sv = CUDART_NAN, dfv = CUDART_NAN;
@@ -551,15 +491,11 @@ predict_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws
 
 // ---------------------------------------------------------------------- MLE
 
-struct MleOut {
-    double *llik, *dllik, *d2llik;
-    int32_t *iters, *status;
-};
-
 __global__ void __launch_bounds__(GP_THREADS, 6)
 mle_kernel(GpArgs a, double *dv, double dmin, double dmax, int max_iter, int *counter, double *ws,
-           MleOut o, unsigned long long *work) {
+           const int *redo, MleOut o, unsigned long long *work) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (redo && *redo == 0) return;  // (after the fixed-point kernel: the locations it left)
     const int nmax = a.nmax, p = a.p, ld = (nmax + 31) & ~31;
     GpShared S = carve(smem_raw, nmax, p);
     for (int i = threadIdx.x; i < EXP64_TABLE_SIZE; i += GP_THREADS) S.etab[i] = exp64_table_g[i];  // ordered by the loop's first barrier
@@ -573,6 +509,7 @@ mle_kernel(GpArgs a, double *dv, double dmin, double dmax, int max_iter, int *co
         const int64_t loc = s_loc;
         __syncthreads();
         if (loc >= a.M) break;
+        if (redo && o.status[loc] != FX_REDO) continue;
         const int nm = a.n ? a.n[loc] : nmax;
         int st = load_design(a, loc, nm, dv, S.xd, S.y, &s_flag, b);
         const unsigned long long n3 = (unsigned long long)nm * nm * nm;
@@ -758,10 +695,13 @@ struct GpLaunch {
     size_t smem;
     double *ws;
     int *counter;
+    // the fixed-point kernel's launches before this one: work counters of its
+    // size classes, and the number of locations it leaves (null: none runs)
+    int *fx_counters, *redo;
 };
 
 template <typename Kern>
-lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, GpLaunch &L) {
+lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, bool fixed, GpLaunch &L) {
     const int ld = (a.nmax + 31) & ~31;
     L.smem = ((size_t)a.nmax * a.p + (size_t)a.nmax * 10 + (size_t)a.p + EXP64_TABLE_SIZE + 4) * 8 + 64;
     if (L.smem > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "n_max x p too large");
@@ -773,21 +713,31 @@ lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, GpLaunch &L) {
     if (grid > a.M) grid = a.M;
     if (grid < 1) grid = 1;
     L.grid = (int)grid;
-    L.ws = static_cast<double *>(lagp_ws(ctx, WS_GP_MAT, (size_t)grid * 6 * a.nmax * ld * 8 + 256));
-    L.counter = static_cast<int *>(lagp_ws(ctx, WS_ALC_COUNTER, 256));
-    if (!L.ws || !L.counter) return LAGP_ENOMEM;
-    LAGP_CUDA(ctx, cudaMemsetAsync(L.counter + 1, 0, sizeof(int), ctx->stream));
-    L.counter += 1;  // its own counter word
+    size_t bytes = (size_t)grid * 6 * a.nmax * ld * 8 + 256;
+    if (fixed) bytes = std::max(bytes, gp_fixed_workspace(ctx, a));
+    L.ws = static_cast<double *>(lagp_ws(ctx, WS_GP_MAT, bytes));
+    int *words = static_cast<int *>(lagp_ws(ctx, WS_ALC_COUNTER, 256));
+    if (!L.ws || !words) return LAGP_ENOMEM;
+    // words of its own: the work counter, the fixed-point kernel's, its count
+    // of locations left
+    LAGP_CUDA(ctx, cudaMemsetAsync(words + 1, 0, 10 * sizeof(int), ctx->stream));
+    L.counter = words + 1;
+    L.fx_counters = words + 2;
+    L.redo = fixed ? words + 10 : nullptr;
     return LAGP_OK;
 }
 
 }  // namespace
 
+// Prediction and MLE: in fixed point where that holds (designs of up to 128
+// rows, nugget below 1), then in FP64 what it leaves; else in FP64.
 lagp_status launch_predict(lagp_ctx *ctx, const GpArgs &a, const double *d, double *mean,
                            double *s2, double *df, int32_t *status) {
     GpLaunch L;
-    LAGP_TRY(prepare(ctx, a, predict_kernel, L));
-    predict_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, L.counter, L.ws, mean, s2, df, status);
+    const bool fixed = gp_fixed_supported(ctx, a, false);
+    LAGP_TRY(prepare(ctx, a, predict_kernel, fixed, L));
+    if (fixed) LAGP_TRY(launch_predict_fixed(ctx, a, d, mean, s2, df, status, L.fx_counters, L.redo));
+    predict_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, L.counter, L.ws, L.redo, mean, s2, df, status);
     ctx->launches++;
     LAGP_CUDA(ctx, cudaGetLastError());
     return LAGP_OK;
@@ -797,12 +747,15 @@ lagp_status launch_mle(lagp_ctx *ctx, const GpArgs &a, double *d, double dmin, d
                        int32_t max_iter, double *llik, double *dllik, double *d2llik,
                        int32_t *iters, int32_t *status) {
     GpLaunch L;
-    LAGP_TRY(prepare(ctx, a, mle_kernel, L));
+    const bool fixed = gp_fixed_supported(ctx, a, true);
+    LAGP_TRY(prepare(ctx, a, mle_kernel, fixed, L));
     MleOut o{llik, dllik, d2llik, iters, status};
     int *ac = nullptr;
     unsigned long long *aw = nullptr;
     LAGP_TRY(alc_counters(ctx, &ac, &aw));  // (the MLE's words follow the ALC's)
-    mle_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, dmin, dmax, max_iter, L.counter, L.ws, o,
+    if (fixed)
+        LAGP_TRY(launch_mle_fixed(ctx, a, d, dmin, dmax, max_iter, o, aw + 8, L.ws, L.fx_counters, L.redo));
+    mle_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, dmin, dmax, max_iter, L.counter, L.ws, L.redo, o,
                                                             aw + 8);
     ctx->launches++;
     LAGP_CUDA(ctx, cudaGetLastError());
@@ -814,7 +767,7 @@ lagp_status launch_predict_grad(lagp_ctx *ctx, const GpArgs &a, const double *d,
                                 double *ds2_dg, double *dllik_dd, double *dllik_dg,
                                 int32_t *status) {
     GpLaunch L;
-    LAGP_TRY(prepare(ctx, a, grad_kernel, L));
+    LAGP_TRY(prepare(ctx, a, grad_kernel, false, L));
     GradOut o{dmean_dd, dmean_dg, ds2_dd, ds2_dg, dllik_dd, dllik_dg, status};
     grad_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, L.counter, L.ws, o);
     ctx->launches++;

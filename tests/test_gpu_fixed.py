@@ -1,0 +1,84 @@
+"""Prediction and MLE in fixed point (csrc/gp_fixed.cu) where they can go
+wrong: sizes at the edges of its classes and column pairs in one uneven batch,
+responses and nuggets at the ends of its range, and the locations it leaves to
+the FP64 kernels.  Bars as in test_gpu_parity.py, against the FP64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from test_gpu_parity import L, O, check_pred, dev  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+SIZES = np.array([1, 2, 3, 4, 39, 40, 41, 42, 63, 64, 65, 66, 79, 80, 81, 103, 104, 105, 127, 128], np.int32)
+
+
+def designs(O, seed, g, n_arr, **kw):
+    w = W.borehole(seed=seed, N=4_000, M=len(n_arr), n=int(n_arr.max()), Np=200, g=g, **kw)
+    return w, O.knn(w.X, w.Xref, int(n_arr.max())).astype(np.int32)
+
+
+def check_mle(out, ref):
+    assert np.array_equal(out["status"].cpu().numpy(), ref["status"])
+    assert np.array_equal(out["iters"].cpu().numpy(), ref["iters"])
+    np.testing.assert_allclose(out["d"].cpu().numpy(), ref["d"], rtol=1e-6)
+    np.testing.assert_allclose(out["llik"].cpu().numpy(), ref["llik"], rtol=1e-9, atol=1e-9)
+    scale = np.abs(ref["llik"]) / ref["d"]
+    np.testing.assert_allclose(out["dllik"].cpu().numpy(), ref["dllik"], rtol=1e-5, atol=1e-7 * scale.max())
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_uneven_sizes_at_class_edges(L, O, dtype):
+    g, d = 1e-3, 1.5
+    w, sel = designs(O, 31, g, SIZES, dtype=dtype)
+    ref = O.predict(w.X, w.Y, w.Xref, sel, SIZES, d, g)
+    out = L.lagp_predict(dev(w.X), dev(w.Y), dev(w.Xref), dev(sel), SIZES, d, g)
+    assert (out["status"].cpu().numpy() == 0).all()
+    check_pred(out["mean"].cpu().numpy(), out["s2"].cpu().numpy(), ref, w.X, w.Y, w.Xref, sel, SIZES, d, g)
+    d0 = np.full(w.M, d)
+    check_mle(L.lagp_mle_step(dev(w.X), dev(w.Y), dev(sel), SIZES, d0, g, 1e-3, 20.0, 2),
+              O.mle(w.X, w.Y, sel, SIZES, d0, g, 1e-3, 20.0, 2))
+
+
+@pytest.mark.parametrize("g", [1e-6, 0.5, 0.999, 1.0, 30.0])
+@pytest.mark.parametrize("scale,spike", [(1.0, 0.0), (1e-13, 0.0), (1e13, 0.0), (1.0, 1e4)])
+def test_ranges_of_nugget_and_responses(L, O, g, scale, spike):
+    """spike: one response far from the others (z then exceeds what its scale
+    leaves room for, and the wider scale or FP64 takes over)."""
+    n, d = 24, 2.0
+    n_arr = np.full(12, n, np.int32)
+    w, sel = designs(O, 32, g, n_arr)
+    Y = w.Y * scale
+    Y[sel[3, 5]] += spike
+    ref = O.predict(w.X, Y, w.Xref, sel, n, d, g)
+    out = L.lagp_predict(dev(w.X), dev(Y), dev(w.Xref), dev(sel), n, d, g)
+    assert (out["status"].cpu().numpy() == 0).all()
+    check_pred(out["mean"].cpu().numpy(), out["s2"].cpu().numpy(), ref, w.X, Y, w.Xref, sel, n_arr, d, g)
+    d0 = np.full(w.M, d)
+    check_mle(L.lagp_mle_step(dev(w.X), dev(Y), dev(sel), n, d0, g, 1e-3, 20.0, 1),
+              O.mle(w.X, Y, sel, n, d0, g, 1e-3, 20.0, 1))
+
+
+def test_locations_left_to_fp64(L, O):
+    """Far locations (k_n(x) underflows), zero and non-finite responses,
+    duplicated rows without a nugget: as the FP64 kernels have them."""
+    n, d = 20, 0.5
+    n_arr = np.full(8, n, np.int32)
+    w, sel = designs(O, 33, 0.0, n_arr)
+    Y, Xref = w.Y.copy(), w.Xref.copy()
+    Xref[0] += 40.0                  # exp(-D/d) is zero or subnormal
+    sel[1, 7] = sel[1, 3]            # singular without a nugget: rounding decides what FP64 makes of it
+    rows = np.setdiff1d(np.arange(w.N), sel.ravel())[:n].astype(np.int32)
+    sel[2], Y[rows] = rows, 0.0      # all responses zero
+    ref = O.predict(w.X, Y, Xref, sel, n, d, 0.0)
+    out = {k: v.cpu().numpy() for k, v in L.lagp_predict(dev(w.X), dev(Y), dev(Xref), dev(sel), n, d, 0.0).items()}
+    assert out["status"][1] in (0, 2)
+    ok = np.arange(8) != 1
+    assert (out["status"][ok] == 0).all()
+    check_pred(out["mean"][ok], out["s2"][ok], {k: v[ok] for k, v in ref.items()}, w.X, Y, Xref, sel[ok], n_arr[ok], d, 0.0)
+    m = L.lagp_mle_step(dev(w.X), dev(Y), dev(sel), n, d, 0.0, 1e-3, 20.0, 0)
+    assert (m["status"].cpu().numpy()[ok] == 0).all()
+    Y[sel[4, 2]] = np.nan
+    out = L.lagp_predict(dev(w.X), dev(Y), dev(Xref), dev(sel), n, d, 0.0)
+    assert torch.isnan(out["mean"][4]) and int(out["status"][4]) == 0
