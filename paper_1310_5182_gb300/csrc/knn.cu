@@ -22,10 +22,18 @@
 //               overflowed, is redone by a second launch with stride 1 (the
 //               exact method), where a block with at most four such queries
 //               gives each a team of warps that share its sweep.
-//   knn_sort    one CTA per query: exact FP64 distances of the collected rows
+//   knn_rank    one CTA per query: buckets the collected rows by direct-form
+//               FP32 distance and orders each bucket; exact FP64 distances
 //               (separately rounded subtract/multiply/add in coordinate order,
-//               on the original coordinates), bitonic sort on (d2, row), first
-//               N' rows written out.
+//               on the original coordinates) inside runs of near ties; first N'
+//               rows written out.
+//   knn_sort    the same by a radix selection and a bitonic sort, for what
+//               knn_rank leaves and after the exact retry.
+// Large problems (ORD_MIN_PAIRS) first sort rows and locations by cell
+// (knn_cells, knn_cell_starts, knn_cell_scatter), so that blocks of them have
+// small bounding boxes (knn_boxes) and the tensor-core collection skips the
+// block pairs that are too far apart; candidates are then positions in that
+// order, mapped back to design rows by the sort.
 // The collected set provably contains the exact FP64 top-N', so the result
 // equals an FP64 sort of all N rows bit for bit.
 #include <cuda_runtime.h>
@@ -70,7 +78,6 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 constexpr int CAND_CAP = 8192;        // candidate capacity cap (sort in shared memory)
-constexpr int SORT_SMALL = 1024;      // survivors the first sort launch holds
 // kNN meta area: the tensor-core screen's failure word (offset 0), two block
 // counters (64), the coordinate bounds (256 and 768, 64 keys each), the
 // launch constants (KnnConst, 1280), then per-query candidate counts and
@@ -139,14 +146,15 @@ __global__ void knn_bounds(const void *__restrict__ X, int64_t N, const void *__
     }
 }
 
-// Centred FP32 copy of design row r, (y_0 .. y_{p-1}, |y|^2, 0 padding),
+// Centred FP32 copy of the design row at position r, (y_0 .. y_{p-1}, |y|^2, 0 padding),
 // with y_i = fl32(x_i - c_i) and |y|^2 an FP32 fused multiply-add chain in
 // coordinate order; rows past N are zero.
-__device__ __forceinline__ void centred_row(const void *X, int64_t N, int64_t r, int p, int ps,
-                                            lagp_dtype dt, const double *c, float *out) {
+__device__ __forceinline__ void centred_row(const void *X, int64_t N, int64_t r, const int32_t *perm, int p,
+                                            int ps, lagp_dtype dt, const double *c, float *out) {
     float n2 = 0.f;
+    const int64_t row = r < N && perm ? perm[r] : r;
     for (int i = 0; i < p; i++) {
-        const float y = r < N ? (float)(load_coord64(X, r, p, i, dt) - c[i]) : 0.f;
+        const float y = r < N ? (float)(load_coord64(X, row, p, i, dt) - c[i]) : 0.f;
         out[i] = y;
         n2 = fmaf(y, y, n2);
     }
@@ -159,14 +167,15 @@ __device__ __forceinline__ void centred_row(const void *X, int64_t N, int64_t r,
 // serialise the threads that wait for the margin).
 __device__ __forceinline__ double pow_bound(double u, double n) { return 1.0 / (1.0 - ceil(n) * u); }
 
-// Y: all rows (Npad of them), Ys: rows 0, s, 2s, ... (nsamp_pad of them;
+// In the order of perm (null: as given).  Y: all rows (Npad of them), Ys: positions 0, s, 2s, ... (nsamp_pad of them;
 // null when s = 1, where the sample is the whole design), Yv: the
 // coordinates of Y with a row stride of p rounded up to 4; kc: the launch's
 // constants (block 0).
 __global__ void knn_prep(const void *__restrict__ X, int64_t N, int p, lagp_dtype dt,
                          const unsigned long long *kmax, const unsigned long long *kmin,
-                         float *__restrict__ Y, int64_t Npad, float *__restrict__ Ys,
-                         int64_t nsamp_pad, int64_t sstride, KnnConst *kc, float *__restrict__ Yv) {
+                         const int32_t *__restrict__ perm, float *__restrict__ Y, int64_t Npad,
+                         float *__restrict__ Ys, int64_t nsamp_pad, int64_t sstride, KnnConst *kc,
+                         float *__restrict__ Yv) {
     __shared__ double c[64];
     __shared__ double sB;
     if (threadIdx.x == 0) {
@@ -184,14 +193,121 @@ __global__ void knn_prep(const void *__restrict__ X, int64_t N, int p, lagp_dtyp
     const int ps = row_stride(p);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < Npad; r += stride) {
-        centred_row(X, N, r, p, ps, dt, c, Y + r * ps);
+        centred_row(X, N, r, perm, p, ps, dt, c, Y + r * ps);
         // the same coordinates with a row stride of p rounded up to 4 (vector gathers in the sort)
         const int pv = (p + 3) & ~3;
         for (int i = 0; i < pv; i++) Yv[r * pv + i] = i < p ? Y[r * ps + i] : 0.f;
     }
     if (Ys)
         for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nsamp_pad; r += stride)
-            centred_row(X, N, r * sstride, p, ps, dt, c, Ys + r * ps);
+            centred_row(X, N, r * sstride, perm, p, ps, dt, c, Ys + r * ps);
+}
+
+// ------------------------------------------------------------ spatial order
+// The design rows and the locations sorted by the cell they lie in, so that
+// 128 rows (or 64 locations) in a row have a small bounding box: a counting
+// sort on a 16-bit cell number, the coordinates' leading bits (up to 16 cuts
+// in halves, taken round the coordinates) read as a Gray code, so that
+// neighbouring cells in the order differ in one cut.  The order within a cell
+// is whatever the atomics make it: no result depends on it.
+constexpr int ORD_BITS = 16, ORD_CELLS = 1 << ORD_BITS;
+// From here on: the order costs four launches and 60 to 500 us, the collection
+// of 2^30 pairs 0.55 ms (100,000 x 10,000 in 8 dimensions: 10.55 ms a call
+// without, 10.80 with it; 500,000 x 201,600 in 3: 49.1 without, 19.7 with).
+constexpr int64_t ORD_MIN_ROWS = 1 << 15, ORD_MIN_PAIRS = 1ll << 30;
+
+__global__ void knn_cells(const void *__restrict__ X, int64_t N, const void *__restrict__ Xr, int64_t M, int p,
+                          lagp_dtype dt, const unsigned long long *kmax, const unsigned long long *kmin,
+                          uint16_t *__restrict__ cell, uint32_t *__restrict__ hist) {
+    __shared__ double lo[ORD_BITS], inv[ORD_BITS];
+    const int dims = min(p, ORD_BITS);
+    if (threadIdx.x < dims) {
+        const int i = threadIdx.x;
+        const double a = kmax[i] ? dkey_inv(~kmin[i]) : 0.0, b = kmax[i] ? dkey_inv(kmax[i]) : 0.0;
+        lo[i] = a;
+        inv[i] = b > a ? 1.0 / (b - a) : 0.0;
+    }
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < N + M; r += stride) {
+        const bool des = r < N;
+        uint32_t code = 0;
+        for (int i = 0; i < dims; i++) {
+            const int bits = (ORD_BITS - i + dims - 1) / dims;  // cuts of this coordinate
+            const float t = (float)((load_coord64(des ? X : Xr, des ? r : r - N, p, i, dt) - lo[i]) * inv[i]);
+            const uint32_t v = min((uint32_t)(fmaxf(t, 0.f) * (float)(1 << bits)), (1u << bits) - 1u);  // (NaN: 0)
+            for (int b = 0; b < bits; b++)
+                code |= ((v >> (bits - 1 - b)) & 1u) << (ORD_BITS - 1 - (b * dims + i));
+        }
+        code ^= code >> 1;  // Gray code to its rank
+        code ^= code >> 2;
+        code ^= code >> 4;
+        code ^= code >> 8;
+        cell[r] = (uint16_t)code;
+        atomicAdd(hist + (des ? 0 : ORD_CELLS) + code, 1u);
+    }
+}
+
+// Exclusive prefix sums of the two histograms (block 0: rows, 1: locations).
+__global__ void __launch_bounds__(1024) knn_cell_starts(uint32_t *hist) {
+    constexpr int PER = ORD_CELLS / 1024;
+    __shared__ uint32_t wsum[32];
+    uint32_t *h = hist + (size_t)blockIdx.x * ORD_CELLS + threadIdx.x * PER;
+    uint32_t s = 0;
+    for (int i = 0; i < PER; i += 4) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(h + i);
+        s += v.x + v.y + v.z + v.w;
+    }
+    uint32_t incl = s;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(LAGP_FULL_MASK, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    uint32_t at = incl - s;
+    for (int i = 0; i < w; i++) at += wsum[i];
+    for (int i = 0; i < PER; i += 4) {
+        uint4 v = *reinterpret_cast<uint4 *>(h + i);
+        const uint4 n = v;
+        v.x = at, v.y = v.x + n.x, v.z = v.y + n.y, v.w = v.z + n.z;
+        at = v.w + n.w;
+        *reinterpret_cast<uint4 *>(h + i) = v;
+    }
+}
+
+__global__ void knn_cell_scatter(const uint16_t *__restrict__ cell, int64_t N, int64_t M,
+                                 uint32_t *__restrict__ starts, int32_t *__restrict__ row,
+                                 int32_t *__restrict__ query) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < N + M; r += stride) {
+        const bool des = r < N;
+        const uint32_t at = atomicAdd(starts + (des ? 0 : ORD_CELLS) + cell[r], 1u);
+        (des ? row : query)[at] = (int32_t)(des ? r : r - N);
+    }
+}
+
+// Bounding boxes of the blocks of 128 positions, from the ordered centred
+// copy: one warp a block.
+__global__ void knn_boxes(const float *__restrict__ Y, int64_t N, int p, int nmb, float *__restrict__ box) {
+    const int lane = threadIdx.x & 31, ps = row_stride(p);
+    for (int mb = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); mb < nmb; mb += gridDim.x * (blockDim.x >> 5))
+        for (int i = 0; i < p; i++) {
+            float lo = CUDART_INF_F, hi = -CUDART_INF_F;  // (fminf and fmaxf leave NaN out)
+            for (int64_t r = (int64_t)mb * 128 + lane; r < min(N, (int64_t)mb * 128 + 128); r += 32) {
+                lo = fminf(lo, Y[r * ps + i]);
+                hi = fmaxf(hi, Y[r * ps + i]);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(LAGP_FULL_MASK, lo, o));
+                hi = fmaxf(hi, __shfl_xor_sync(LAGP_FULL_MASK, hi, o));
+            }
+            if (lane == 0) {
+                box[(int64_t)i * nmb + mb] = lo;
+                box[(int64_t)(p + i) * nmb + mb] = hi;
+            }
+        }
 }
 
 // Widened thresholds for the collection pass.  With u = 2^-24 (widened by
@@ -596,8 +712,9 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
     }
 }
 
-// Block-wide exclusive prefix sum of one int per thread (SORT_THREADS
-// threads); returns the thread's offset, *total the sum.
+// Block-wide exclusive prefix sum of one int per thread (NT threads); returns
+// the thread's offset, *total the sum.
+template <int NT>
 __device__ int block_excl_scan(int v, int *wsum, int *total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int incl = v;
@@ -609,7 +726,7 @@ __device__ int block_excl_scan(int v, int *wsum, int *total) {
     if (lane == 31) wsum[w] = incl;
     __syncthreads();
     int off = 0, tot = 0;
-    for (int i = 0; i < SORT_THREADS / 32; i++) {
+    for (int i = 0; i < NT / 32; i++) {
         off += i < w ? wsum[i] : 0;
         tot += wsum[i];
     }
@@ -715,23 +832,16 @@ __device__ void sort1024_registers(unsigned long long *sk, int S, unsigned long 
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(SORT_THREADS)
-knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, int p, lagp_dtype dt,
-         const void *__restrict__ Xref, int64_t M, const int32_t *__restrict__ Np, int32_t Npmax,
-         const unsigned long long *__restrict__ kmax, const unsigned long long *__restrict__ kmin,
-         const int32_t *__restrict__ cand, const int32_t *__restrict__ cand_count, int32_t Cmax,
-         int32_t *__restrict__ idx, const KnnConst *__restrict__ kc, const float *__restrict__ rcol,
-         int32_t *__restrict__ retry, int32_t *__restrict__ bigf, int big) {
+// The general sort, for the queries that knn_rank leaves (bigf) and, after the
+// exact retry, the flagged ones: any number of survivors, any run of ties, in
+// shared memory.  One CTA a query, the grid striding over the queries.
+__device__ void knn_sort_query(const void *__restrict__ X, const float *__restrict__ Yv,
+                               const int32_t *__restrict__ perm, int p, lagp_dtype dt,
+                               const void *__restrict__ Xref, int64_t q, const int32_t *__restrict__ Np,
+                               int32_t Npmax, const int32_t *__restrict__ cand,
+                               const int32_t *__restrict__ cand_count, int32_t Cmax, int32_t *__restrict__ idx,
+                               const KnnConst *__restrict__ kc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t q = blockIdx.x;
-    // Two launches.  The first (big = 0, shared memory for up to 1,024
-    // survivors) sorts every query but those flagged for the exact retry, and
-    // flags (bigf) the ones with more survivors; the second (big = 1, shared
-    // memory for any count) sorts the flagged ones of either kind.
-    const bool flagged = (retry && retry[q] != 0) || (big && bigf[q] != 0);
-    (void)kmax;
-    (void)kmin;
-    if (flagged != (big != 0)) return;
     const int C = cand_count[q];
     const int k = Np ? Np[q] : Npmax;
     int32_t *out = idx + q * Npmax;
@@ -741,20 +851,20 @@ knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, int p, lagp_d
     }
     int Cp = 1;
     while (Cp < Cmax) Cp <<= 1;
-    // region 1 (R1 doubles): FP32 keys and rows for steps 1-3, then FP64 keys;
-    // region 2 (R2 words of 64 bits): the survivors' (s, row) keys
-    const int R1 = big ? Cp : (Cmax + 1) & ~1, R2 = big ? Cp : SORT_SMALL;
+    // region 1 (R1 doubles): FP32 keys and positions for steps 1-3, then FP64
+    // keys; region 2 (R1 words of 64 bits): the survivors' (s, row) keys
+    const int R1 = Cp;
     uint32_t *key32 = reinterpret_cast<uint32_t *>(smem_raw);           // Cmax
     int32_t *rowA = reinterpret_cast<int32_t *>(key32 + R1);            // Cmax
     double *dk = reinterpret_cast<double *>(smem_raw);                  // R1
-    unsigned long long *sk = reinterpret_cast<unsigned long long *>(smem_raw + (size_t)R1 * 8);  // R2
+    unsigned long long *sk = reinterpret_cast<unsigned long long *>(smem_raw + (size_t)R1 * 8);  // R1
     __shared__ double xq[64];
     __shared__ float yq[64];
     __shared__ float s_d2f;
     __shared__ uint32_t hist[256];
     __shared__ int wsum[SORT_THREADS / 32];
     __shared__ uint32_t s_prefix;
-    __shared__ int s_kk, s_big, s_fail;
+    __shared__ int s_kk, s_big;
     __shared__ float s_tauf;
     __shared__ uint32_t tied[CAND_CAP / 32];
     if (threadIdx.x < p) {
@@ -836,36 +946,22 @@ knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, int p, lagp_d
         // the margins with the launch's constants
         const double g = kc->g_half, e2 = kc->e2;
         const float vk = __uint_as_float(s_prefix);
-        const double rk = sqrt((double)vk) * g * (1.0 + 1e-13) + e2;  // >= exact N'-th distance
         const float tauf = __double2float_rd(screen_margin_c(vk, g, e2));
         s_tauf = tauf;
         s_d2f = __double2float_ru(2.0 * tie_bound(tauf, g, kc->g_full, e2));
-        // rows collected on the tensor cores: the N'-th of them must lie
-        // within the radius collected in full, else the query goes to the
-        // exact retry
-        s_fail = rcol ? !(rk <= (double)rcol[q]) : 0;
     }
     __syncthreads();
-    if (s_fail) {
-        if (threadIdx.x == 0) retry[q] = 1;
-        for (int t = threadIdx.x; t < Npmax; t += SORT_THREADS) out[t] = -1;
-        return;
-    }
     const float tauf = s_tauf;
     // (3) survivors, in candidate order, as (s, row) keys
     int mine = 0;
     for (int e = threadIdx.x; e < C; e += SORT_THREADS) mine += __uint_as_float(key32[e]) <= tauf;
     int S = 0;
-    int pos = block_excl_scan(mine, wsum, &S);  // S is block-uniform
+    int pos = block_excl_scan<SORT_THREADS>(mine, wsum, &S);  // S is block-uniform
     int Sp = 1;
     while (Sp < S) Sp <<= 1;
-    if (Sp > R2) {  // more survivors than this launch holds: the second launch sorts it
-        if (threadIdx.x == 0) bigf[q] = 1;
-        return;
-    }
     for (int e = threadIdx.x; e < C; e += SORT_THREADS)
         if (__uint_as_float(key32[e]) <= tauf)
-            sk[pos++] = ((unsigned long long)key32[e] << 32) | (uint32_t)rowA[e];
+            sk[pos++] = ((unsigned long long)key32[e] << 32) | (uint32_t)(perm ? perm[rowA[e]] : rowA[e]);
     for (int e = S + threadIdx.x; e < Sp; e += SORT_THREADS) sk[e] = ~0ull;
     __syncthreads();
     // (4) bitonic sort on (s, row): up to 1,024 keys in registers (four a
@@ -964,6 +1060,257 @@ knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, int p, lagp_d
     for (int t = threadIdx.x; t < Npmax; t += SORT_THREADS) out[t] = t < k ? (int32_t)(uint32_t)sk[t] : -1;
 }
 
+__global__ void __launch_bounds__(SORT_THREADS)
+knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t *__restrict__ perm, int p,
+         lagp_dtype dt, const void *__restrict__ Xref, int64_t M, const int32_t *__restrict__ Np, int32_t Npmax,
+         const int32_t *__restrict__ cand, const int32_t *__restrict__ cand_count, int32_t Cmax,
+         int32_t *__restrict__ idx, const KnnConst *__restrict__ kc, const int32_t *__restrict__ retry,
+         const int32_t *__restrict__ bigf) {
+    for (int64_t q = blockIdx.x; q < M; q += gridDim.x) {
+        if (!(retry && retry[q] != 0) && bigf[q] == 0) continue;
+        knn_sort_query(X, Yv, perm, p, dt, Xref, q, Np, Npmax, cand, cand_count, Cmax, idx, kc);
+        __syncthreads();  // shared memory is free for the next query
+    }
+}
+
+// Rank of the collected rows without a comparison sort, one CTA a query: the
+// rows' direct-form FP32 values (kept in registers, IT a thread) go into `nb`
+// buckets of equal width between the smallest and the largest (a monotone
+// map, so that the buckets are in order), about one row a bucket; a prefix sum
+// of the counts places the rows of the buckets up to the one after the N'-th
+// row's, and each bucket is ordered on (s, row) by one thread.  Then the
+// margins, the collection check and the runs of near ties as in the steps
+// above (3, 5, 6).  Linear in the number of rows, eight barriers, against the
+// bitonic sort's (log^2) with a radix selection before it: N' = 1500 of 2,600
+// rows, 201,600 queries, 32.8 -> 8.7 ms; N' = 2000 of 3,600, 25,000 queries,
+// 14.7 -> 3.9 ms.  Bound: instruction issue and the
+// latency of the gathers.  Left to knn_sort (bigf): distances that are not
+// finite, a bucket of more than RANK_BUCKET rows, runs longer than 32 (many
+// equal distances), survivors past the placed buckets.
+constexpr int RANK_BUCKET = 24;
+
+// Buckets for up to `cap` placed rows (cap FP64 keys reuse their space).
+__host__ __device__ inline int rank_buckets(int cap) { return (2 * cap + 1023) / 1024 * 1024; }
+
+template <int IT, int NT>
+__global__ void __launch_bounds__(NT)
+knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t *__restrict__ perm, int p,
+         lagp_dtype dt, const void *__restrict__ Xref, const int32_t *__restrict__ Np, int32_t Npmax,
+         const int32_t *__restrict__ cand, const int32_t *__restrict__ cand_count, int32_t Cmax, int cap,
+         int32_t *__restrict__ idx, const KnnConst *__restrict__ kc, const float *__restrict__ rcol,
+         int32_t *__restrict__ retry, int32_t *__restrict__ bigf) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int64_t q = blockIdx.x;
+    if (rcol && retry[q] != 0) return;  // (overflowed or not screened: the exact retry)
+    const int C = cand_count[q], k = Np ? Np[q] : Npmax, tid = threadIdx.x, lane = tid & 31;
+    int32_t *out = idx + q * Npmax;
+    if (C < k || C > Cmax || k < 1 || k > Npmax) {  // invalid or overflowed: empty row
+        for (int t = tid; t < Npmax; t += NT) out[t] = -1;
+        return;
+    }
+    const int nb = rank_buckets(cap);
+    uint32_t *start = reinterpret_cast<uint32_t *>(smem_raw);                           // nb: counts, then starts
+    double *dk = reinterpret_cast<double *>(smem_raw);                                  // cap, after the buckets
+    unsigned long long *sk = reinterpret_cast<unsigned long long *>(smem_raw + (size_t)nb * 4);  // cap (s, row) keys
+    uint32_t *tied = reinterpret_cast<uint32_t *>(sk + cap);                            // cap / 32 + 1
+    __shared__ double xq[64];
+    __shared__ float yq[64];
+    __shared__ int wsum[NT / 32];
+    __shared__ uint32_t s_lo, s_hi;
+    __shared__ int s_kb, s_left, s_fail, s_S;
+    __shared__ float s_tauf, s_d2f;
+    if (tid < p) {
+        xq[tid] = load_coord64(Xref, q, p, tid, dt);
+        yq[tid] = (float)(xq[tid] - kc->c[tid]);
+    }
+    if (tid == 0) s_lo = 0xFFFFFFFFu, s_hi = 0u, s_left = 0;
+    for (int b = tid; b < nb; b += NT) start[b] = 0u;
+    __syncthreads();
+    // direct-form FP32 values (non-negative floats order like their bits)
+    uint32_t key[IT];
+    int32_t pos[IT];
+    const int pv = (p + 3) & ~3;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < IT; i++) {
+        const int e = tid + i * NT;
+        pos[i] = e < C ? cand[q * Cmax + e] : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < IT; i++) {
+        if (pos[i] < 0) continue;
+        const float4 *yr = reinterpret_cast<const float4 *>(Yv + (int64_t)pos[i] * pv);
+        float sv = 0.f;
+        for (int i4 = 0; i4 < pv; i4 += 4) {
+            const float4 v = yr[i4 >> 2];
+            const float t[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (i4 + j < p) {  // coordinate order, as the direct form defines
+                    const float df = t[j] - yq[i4 + j];
+                    sv = fmaf(df, df, sv);
+                }
+        }
+        key[i] = __float_as_uint(sv);
+        lo = min(lo, key[i]);
+        hi = max(hi, key[i]);
+    }
+    lo = __reduce_min_sync(LAGP_FULL_MASK, lo);
+    hi = __reduce_max_sync(LAGP_FULL_MASK, hi);
+    if (lane == 0) {
+        atomicMin(&s_lo, lo);
+        atomicMax(&s_hi, hi);
+    }
+    __syncthreads();
+    const float base = __uint_as_float(s_lo), scale = (float)nb / (__uint_as_float(s_hi) - base);
+    if (s_hi >= 0x7f800000u) {  // infinite or NaN
+        if (tid == 0) bigf[q] = 1;
+        return;
+    }
+    // (equal values: 0 * infinity, bucket 0)
+    auto bucket = [&](uint32_t b) { return min(nb - 1, (int)((__uint_as_float(b) - base) * scale)); };
+    uint16_t rank[IT];
+#pragma unroll
+    for (int i = 0; i < IT; i++)
+        if (pos[i] >= 0) rank[i] = (uint16_t)atomicAdd(&start[bucket(key[i])], 1u);
+    __syncthreads();
+    // starts of the buckets (a warp takes consecutive rows of 32); the N'-th
+    // row's bucket
+    {
+        const int rows = nb / NT;  // rows of 32 buckets a warp
+        uint32_t *mine = start + (tid >> 5) * rows * 32 + lane;
+        int sum = 0, most = 0;
+        for (int j = 0; j < rows; j++) {
+            const int n = mine[32 * j];
+            sum += n;
+            most = max(most, n);
+        }
+        if (most > RANK_BUCKET) s_left = 1;
+        int total;
+        const int before = block_excl_scan<NT>(sum, wsum, &total);
+        int at = __shfl_sync(LAGP_FULL_MASK, before, 0);  // rows before this warp's buckets
+        for (int j = 0; j < rows; j++) {
+            const int n = mine[32 * j];
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(LAGP_FULL_MASK, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int from = at + incl - n;
+            mine[32 * j] = from;
+            if (from < k && from + n >= k) s_kb = ((tid >> 5) * rows + j) * 32 + lane;
+            at += __shfl_sync(LAGP_FULL_MASK, incl, 31);
+        }
+    }
+    __syncthreads();
+    const int last = min(s_kb + 1, nb - 1);  // the buckets placed: 0 .. last
+    const int cut = last + 1 < nb ? (int)start[last + 1] : C;
+    if (s_left || cut > cap) {
+        if (tid == 0) bigf[q] = 1;
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < IT; i++)
+        if (pos[i] >= 0) {
+            const int b = bucket(key[i]);
+            if (b <= last)
+                sk[start[b] + rank[i]] = ((unsigned long long)key[i] << 32) | (uint32_t)(perm ? perm[pos[i]] : pos[i]);
+        }
+    __syncthreads();
+    for (int b = tid; b <= last; b += NT) {
+        const int i0 = start[b], i1 = b + 1 < nb ? (int)start[b + 1] : C;
+        for (int t = i0 + 1; t < i1; t++) {  // insertion sort on (s, row)
+            const unsigned long long kv = sk[t];
+            int u = t - 1;
+            while (u >= i0 && kv < sk[u]) {
+                sk[u + 1] = sk[u];
+                u--;
+            }
+            sk[u + 1] = kv;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        // the margins with the launch's constants
+        const double g = kc->g_half, e2 = kc->e2;
+        const float vk = __uint_as_float((uint32_t)(sk[k - 1] >> 32));
+        const double rk = sqrt((double)vk) * g * (1.0 + 1e-13) + e2;  // >= exact N'-th distance
+        const float tauf = __double2float_rd(screen_margin_c(vk, g, e2));
+        s_tauf = tauf;
+        s_d2f = __double2float_ru(2.0 * tie_bound(tauf, g, kc->g_full, e2));
+        // rows collected on the tensor cores: the N'-th of them must lie
+        // within the radius collected in full, else the query goes to the
+        // exact retry
+        s_fail = rcol ? !(rk <= (double)rcol[q]) : 0;
+        // the survivors (s <= tauf) must all be placed
+        if (cut < C && bucket(__float_as_uint(tauf)) > last) s_left = 1;
+        s_S = k;
+    }
+    __syncthreads();
+    if (s_fail || s_left) {
+        if (tid == 0) (s_fail ? retry : bigf)[q] = 1;
+        if (s_fail)
+            for (int t = tid; t < Npmax; t += NT) out[t] = -1;
+        return;
+    }
+    const float tauf = s_tauf, d2f = s_d2f;
+    for (int e = k + tid; e < cut; e += NT)
+        if (__uint_as_float((uint32_t)(sk[e] >> 32)) <= tauf) atomicAdd(&s_S, 1);
+    __syncthreads();
+    const int S = s_S;
+    // tie flags (bit i: rows i and i + 1 need their FP64 order) before any run is re-ordered
+    for (int i0 = tid - lane; i0 < S; i0 += NT) {
+        const int i = i0 + lane;
+        bool t = false;
+        if (i + 1 < S) {
+            // the FP32 difference rounded down never exceeds the true one
+            const float x = __uint_as_float((uint32_t)(sk[i] >> 32)), y = __uint_as_float((uint32_t)(sk[i + 1] >> 32));
+            t = !(__fsub_rd(y, x) > d2f);
+        }
+        const uint32_t m = __ballot_sync(LAGP_FULL_MASK, t);
+        if (lane == 0) tied[i0 >> 5] = m;
+    }
+    __syncthreads();
+    auto is_tied = [&](int i) { return (tied[i >> 5] >> (i & 31)) & 1u; };
+    for (int i = tid; i < S; i += NT) {
+        if (!is_tied(i) || (i > 0 && is_tied(i - 1))) continue;  // not the start of a run
+        int end = i + 1;  // the run is [i, end]
+        while (is_tied(end) && end - i < 32) end++;
+        if (end - i >= 32) {
+            s_left = 1;
+            continue;
+        }
+        for (int t = i; t <= end; t++) {
+            const int32_t r = (int32_t)(uint32_t)sk[t];
+            double sd = 0.0;
+            for (int c = 0; c < p; c++) {
+                const double diff = __dsub_rn(xq[c], load_coord64(X, r, p, c, dt));
+                sd = __dadd_rn(sd, __dmul_rn(diff, diff));
+            }
+            dk[t] = sd;
+        }
+        for (int t = i + 1; t <= end; t++) {  // insertion sort on (d2, row)
+            const double dv = dk[t];
+            const unsigned long long kv = sk[t];
+            int u = t - 1;
+            while (u >= i && pair_less(dv, (uint32_t)kv, dk[u], (uint32_t)sk[u])) {
+                dk[u + 1] = dk[u];
+                sk[u + 1] = sk[u];
+                u--;
+            }
+            dk[u + 1] = dv;
+            sk[u + 1] = kv;
+        }
+    }
+    __syncthreads();
+    if (s_left) {
+        if (tid == 0) bigf[q] = 1;
+        return;
+    }
+    for (int t = tid; t < Npmax; t += NT) out[t] = t < k ? (int32_t)(uint32_t)sk[t] : -1;
+}
+
 // The screen's first launch: the sampled threshold and the collection on the
 // norm expansion (CUDA cores), or with tau0 the sampled threshold only (the
 // collection then runs on the tensor cores); and the exact retry of the
@@ -1036,17 +1383,42 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     const int blocks = ctx->num_sms * 4;
     knn_bounds<<<blocks, 256, 0, st>>>(X, N, Xref, M, p, dtype, kmax, kmin);
     KnnConst *kc = reinterpret_cast<KnnConst *>(meta + META_CONST);
-    knn_prep<<<blocks, 256, 0, st>>>(X, N, p, dtype, kmax, kmin, Y32, Npad, stride > 1 ? Ys : nullptr,
+    // the spatial order, for the tensor-core collection of large problems
+    const bool tc = ctx->tuning.knn_path == 0 && knn_tc_supported(p);
+    KnnOrder order;
+    if (tc && N >= ORD_MIN_ROWS && N * M >= ORD_MIN_PAIRS) {
+        const int nmb = (int)((N + 127) / 128);
+        const size_t oRow = (size_t)ORD_CELLS * 8, oQuery = oRow + (size_t)N * 4, oBox = oQuery + (size_t)M * 4,
+                     oCell = oBox + (size_t)2 * p * nmb * 4;
+        char *w = static_cast<char *>(lagp_ws(ctx, WS_KNN_ORDER, oCell + (size_t)(N + M) * 2 + 16));
+        if (!w) return LAGP_ENOMEM;
+        uint32_t *hist = reinterpret_cast<uint32_t *>(w);
+        int32_t *row = reinterpret_cast<int32_t *>(w + oRow), *query = reinterpret_cast<int32_t *>(w + oQuery);
+        uint16_t *cell = reinterpret_cast<uint16_t *>(w + oCell);
+        LAGP_CUDA(ctx, cudaMemsetAsync(hist, 0, (size_t)ORD_CELLS * 8, st));
+        knn_cells<<<blocks, 256, 0, st>>>(X, N, Xref, M, p, dtype, kmax, kmin, cell, hist);
+        knn_cell_starts<<<2, 1024, 0, st>>>(hist);
+        knn_cell_scatter<<<blocks, 256, 0, st>>>(cell, N, M, hist, row, query);
+        ctx->launches += 3;
+        order.row = row;
+        order.query = query;
+        order.box = reinterpret_cast<float *>(w + oBox);
+    }
+    knn_prep<<<blocks, 256, 0, st>>>(X, N, p, dtype, kmax, kmin, order.row, Y32, Npad, stride > 1 ? Ys : nullptr,
                                      nsamp_pad, stride, kc, Yv);
     ctx->launches += 2;
+    if (order.box) {
+        knn_boxes<<<blocks, 256, 0, st>>>(Y32, N, p, (int)((N + 127) / 128), order.box);
+        ctx->launches++;
+    }
     LAGP_CUDA(ctx, cudaGetLastError());
     // collection on the tensor cores unless the tuning asks for CUDA cores
     void *tc_ws = nullptr;
     float *tau0 = nullptr, *rcol = nullptr;
-    if (ctx->tuning.knn_path == 0 && knn_tc_supported(p)) {
+    if (tc) {
         tc_ws = lagp_ws(ctx, WS_KNN_TC, knn_tc_workspace(N, M, p));
         if (!tc_ws) return LAGP_ENOMEM;
-        LAGP_TRY(launch_knn_tc_prep(ctx, tc_ws, X, N, p, dtype, Xref, M, kmax, kmin, &tau0, &rcol));
+        LAGP_TRY(launch_knn_tc_prep(ctx, tc_ws, X, N, p, dtype, Xref, M, kmax, kmin, order, &tau0, &rcol));
     }
     int *tc_err = reinterpret_cast<int *>(meta);
 
@@ -1056,11 +1428,12 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     dim3 grid((unsigned)std::min<int64_t>(nblk, (int64_t)ctx->num_sms * 2));
     int Cp = 1;
     while (Cp < Cmax) Cp <<= 1;
-    // the first sort launch: up to SORT_SMALL survivors (more CTAs per SM);
-    // the second: any count
-    const size_t smem_small = (size_t)((Cmax + 1) & ~1) * 8 + (size_t)SORT_SMALL * 8;
+    // shared memory of the rank (rows placed: N' and what shares the last
+    // buckets) and of the general sort
+    const int cap = std::min<int>((Npmax + Npmax / 8 + 128 + 31) & ~31, (Cmax + 31) & ~31);
+    const size_t smem_rank = (size_t)rank_buckets(cap) * 4 + (size_t)cap * 8 + (size_t)(cap / 32 + 1) * 4;
     const size_t smem_big = (size_t)Cp * 16;
-    if (smem_big > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: N' too large for the sort");
+    if (std::max(smem_big, smem_rank) > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: N' too large for the sort");
     cudaFuncSetAttribute(knn_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_big);
     auto screen = [&](bool retry_pass) {
         switch (p) {
@@ -1070,9 +1443,21 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
             default: launch_screen<0>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters, tau0); break;
         }
     };
-    auto sort = [&](const float *rc, int32_t *rflags, int big) {
-        knn_sort<<<(unsigned)M, SORT_THREADS, big ? smem_big : smem_small, st>>>(
-            X, Yv, p, dtype, Xref, M, Np, Npmax, kmax, kmin, cand, cc, Cmax, idx, kc, rc, rflags, bigf, big);
+    auto rank = [&]() {
+        auto go = [&](auto kern, unsigned nt) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rank);
+            kern<<<(unsigned)M, nt, smem_rank, st>>>(X, Yv, order.row, p, dtype, Xref, Np, Npmax, cand, cc, Cmax, cap,
+                                                     idx, kc, rcol, retry, bigf);
+        };
+        if (Cmax <= 8 * 256) go(knn_rank<8, 256>, 256);
+        else if (Cmax <= 16 * 256) go(knn_rank<16, 256>, 256);
+        else go(knn_rank<16, 512>, 512);
+        ctx->launches++;
+    };
+    auto sort = [&](int32_t *rflags) {
+        const unsigned g = (unsigned)std::min<int64_t>(M, (int64_t)ctx->num_sms * 3);
+        knn_sort<<<g, SORT_THREADS, smem_big, st>>>(X, Yv, order.row, p, dtype, Xref, M, Np, Npmax, cand, cc, Cmax,
+                                                    idx, kc, rflags, bigf);
         ctx->launches++;
     };
     screen(false);
@@ -1080,15 +1465,15 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     if (tc_ws) {
         // collection on the tensor cores, the sort (which checks each query's
         // collection), the exact retry of the flagged queries and their sort
-        LAGP_TRY(launch_knn_tc_collect(ctx, tc_ws, N, p, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, retry,
-                                       tc_err, rcol, nullptr));
-        sort(rcol, retry, 0);
+        LAGP_TRY(launch_knn_tc_collect(ctx, tc_ws, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, order, cand, Cmax, cc,
+                                       status, retry, tc_err, counters + 2, rcol, nullptr));
+        rank();
         screen(true);
-        sort(nullptr, retry, 1);
+        sort(retry);
     } else {
         screen(true);
-        sort(nullptr, nullptr, 0);
-        sort(nullptr, nullptr, 1);
+        rank();
+        sort(nullptr);
     }
     LAGP_CUDA(ctx, cudaGetLastError());
     return LAGP_OK;
@@ -1112,9 +1497,10 @@ lagp_status launch_knn_tc_dist(lagp_ctx *ctx, const void *X, int64_t N, int p, l
     ctx->launches++;
     LAGP_CUDA(ctx, cudaGetLastError());
     float *tau0 = nullptr, *rcol = nullptr;
-    LAGP_TRY(launch_knn_tc_prep(ctx, tc_ws, X, N, p, dtype, Xref, M, kmax, kmin, &tau0, &rcol));
-    return launch_knn_tc_collect(ctx, tc_ws, N, p, M, nullptr, 1, kmax, kmin, nullptr, 1, cc, nullptr, retry,
-                                 reinterpret_cast<int *>(meta), rcol, out);
+    LAGP_TRY(launch_knn_tc_prep(ctx, tc_ws, X, N, p, dtype, Xref, M, kmax, kmin, KnnOrder{}, &tau0, &rcol));
+    return launch_knn_tc_collect(ctx, tc_ws, N, p, Xref, dtype, M, nullptr, 1, kmax, kmin, KnnOrder{}, nullptr, 1, cc,
+                                 nullptr, retry, reinterpret_cast<int *>(meta), reinterpret_cast<int *>(meta + 72), rcol,
+                                 out);
 }
 
 // Diagnostic: of the last kNN call on the context, the queries that went to

@@ -20,6 +20,15 @@ __device__ __forceinline__ double dkey_inv(unsigned long long k) {
     return __longlong_as_double((long long)((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k));
 }
 
+// The same for floats (no NaN).
+__device__ __forceinline__ uint32_t fkey(float x) {
+    const uint32_t b = __float_as_uint(x);
+    return (b >> 31) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float fkey_inv(uint32_t k) {
+    return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
+}
+
 // Centre c_i (midrange of coordinate i) and B = max_i |x_i - c_i| (with a
 // relative slack of 2^-50 for the rounding of c_i), from the bounds of the
 // finite coordinates (a coordinate with none gets c_i = 0, B unchanged).

@@ -28,6 +28,12 @@
 // times the sum of their magnitudes, several times what a truncating
 // alignment of its seventeen addends can lose.
 //
+// With a spatial order (KnnOrder) the operands' rows are sorted by cell, and a
+// query block meets only the design blocks whose bounding box comes within the
+// largest threshold of its own box: 500,000 rows in 3 dimensions, 201,600
+// queries, 34.6 -> 5.7 ms.  In 8 dimensions few blocks fall away (a ball with
+// 2,000 of 4M uniform rows reaches most of the cube): 40.1 -> 38.1 ms.
+//
 // Kernel layout (one CTA per SM, persistent over blocks of up to 128
 // queries): warp 0 streams the design operand into a ring of shared-memory
 // stages with bulk asynchronous copies, warp 1 owns the tensor memory and
@@ -60,6 +66,7 @@ constexpr int TC_NACC = 4;       // TMEM accumulators (128 columns each)
 constexpr int TC_ACC_COLS = 128;
 constexpr int TC_TMEM_COLS = TC_NACC * TC_ACC_COLS;  // 512: the whole tensor memory of the SM
 constexpr int TC_QMAX = 128;     // queries per block (MMA N <= 128)
+constexpr int TC_CHUNK = 16384;  // design blocks whose survivors are listed at a time
 constexpr int TC_QUE = 32 * (TC_QMAX / 16);  // hit-queue entries of an epilogue warp: one a lane and chunk
 
 // Half offset of element k of operand row r in the no-swizzle K-major
@@ -105,10 +112,11 @@ __device__ __forceinline__ float centred_coords(const void *A, int64_t r, int p,
 }
 
 // Design operand (Npad rows, blocked layout; rows past N are zero) and query
-// operand rows (M x K, row-major), FP16.
+// operand rows (M x K, row-major), FP16, both in the launch's order.
 __global__ void knn_tc_prep(const void *__restrict__ X, int64_t N, int64_t Npad, const void *__restrict__ Xr,
                             int64_t M, int p, lagp_dtype dt, const unsigned long long *kmax,
-                            const unsigned long long *kmin, __half *__restrict__ A, __half *__restrict__ Q) {
+                            const unsigned long long *kmin, KnnOrder order, __half *__restrict__ A,
+                            __half *__restrict__ Q) {
     __shared__ double c[64];
     __shared__ double sB;
     if (threadIdx.x == 0) centre_and_bound(kmax, kmin, p, c, sB);
@@ -124,7 +132,8 @@ __global__ void knn_tc_prep(const void *__restrict__ X, int64_t N, int64_t Npad,
         const int64_t rr = des ? r : r - Npad;
         for (int k = 0; k < K; k++) row[k] = zero;
         if (!des || rr < N) {
-            centred_coords(des ? X : Xr, rr, p, dt, c, y);
+            const int32_t *perm = des ? order.row : order.query;
+            centred_coords(des ? X : Xr, perm ? perm[rr] : rr, p, dt, c, y);
             float n2 = 0.f;  // |y 2^-e|^2: the FP32 chain of the unscaled norm, scaled exactly
             for (int i = 0; i < p; i++) {
                 y[i] *= scale;
@@ -159,6 +168,10 @@ struct TcArgs {
     const __half *Q;  // query operand rows, M x K
     int64_t N, M;
     int p, K, nmb;
+    KnnOrder order;
+    const void *Xref;  // locations (for the blocks' bounding boxes)
+    lagp_dtype dt;
+    int *counter;      // blocks of queries taken
     const float *tau0;  // per query: sampled threshold, NaN = not screened
     float *rcol;        // per query out: the radius collected in full (rounded down; NaN: not collected)
     const int32_t *Np;
@@ -183,11 +196,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
     uint32_t *s_t2h = reinterpret_cast<uint32_t *>(s_tau2 + TC_QMAX);  // TC_QMAX/2: FP16 x 2, rounded up
     int *s_cnt = reinterpret_cast<int *>(s_t2h + TC_QMAX / 2);       // TC_QMAX
     uint2 *s_que = reinterpret_cast<uint2 *>(s_cnt + TC_QMAX);  // per epilogue warp: TC_QUE entries
-    uint64_t *bar = reinterpret_cast<uint64_t *>(s_que + TC_QUE * 4 * TC_EPI_GROUPS);
+    uint16_t *s_list = reinterpret_cast<uint16_t *>(s_que + TC_QUE * 4 * TC_EPI_GROUPS);  // TC_CHUNK design blocks
+    uint64_t *bar = reinterpret_cast<uint64_t *>(s_list + TC_CHUNK);
     uint64_t *full = bar, *empty = bar + S, *tfull = bar + 2 * S, *tempty = bar + 2 * S + TC_NACC;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_err;
+    __shared__ int s_err, s_blk, s_nlist;
+    __shared__ int32_t s_q[TC_QMAX];  // the block's locations
     __shared__ double s_c[64], s_B;
+    __shared__ uint32_t s_qlo[20], s_qhi[20], s_tmax;  // order-preserving keys of floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
@@ -219,7 +235,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
     const float s2 = ldexpf(1.f, -2 * tc_scale_exp(s_B));
 
     long long it0 = 0;  // design blocks processed by this CTA so far (ring positions)
-    for (int blk = blockIdx.x; blk < a.nblocks; blk += gridDim.x) {
+    for (;;) {
+        if (tid == 0) s_blk = atomicAdd(a.counter, 1);
+        if (tid < 20) s_qlo[tid] = 0xFFFFFFFFu, s_qhi[tid] = 0u;
+        if (tid == 20) s_tmax = 0u;
+        __syncthreads();
+        const int blk = s_blk;
+        if (blk >= a.nblocks) break;
         const int64_t q0 = (int64_t)blk * a.nq;
         const int nqb = (int)min((int64_t)a.nq, a.M - q0);
         const int nmma = (nqb + 15) & ~15;  // MMA N: a multiple of 16
@@ -231,7 +253,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
         for (int c = tid; c < TC_QMAX; c += TC_THREADS) {
             float t2 = CUDART_NAN_F;  // NaN: no row ever compares below
             if (c < nqb) {
-                const int64_t q = q0 + c;
+                const int64_t q = a.order.query ? a.order.query[q0 + c] : q0 + c;
                 const int k = a.Np ? a.Np[q] : a.Npmax;
                 const float tq = a.tau0[q];
                 if (k >= 1 && k <= a.Npmax && tq == tq) {
@@ -244,7 +266,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
             }
             s_tau2[c] = t2 * s2;  // an exact scaling
             s_cnt[c] = 0;
+            s_q[c] = c < nqb ? (int32_t)(a.order.query ? a.order.query[q0 + c] : q0 + c) : 0;
+            if (a.order.box && t2 == t2) atomicMax(&s_tmax, fkey(t2));
         }
+        // the bounding box of the block's queries
+        if (a.order.box)
+            for (int e = tid; e < nqb * a.p; e += TC_THREADS) {
+                const int c = e / a.p, i = e - c * a.p;
+                const float y = (float)(load_coord64(a.Xref, a.order.query[q0 + c], a.p, i, a.dt) - s_c[i]);
+                if (y == y) {
+                    atomicMin(&s_qlo[i], fkey(y));
+                    atomicMax(&s_qhi[i], fkey(y));
+                }
+            }
         __syncthreads();
         // the thresholds in FP16, rounded up (so that a value below a threshold
         // stays below it after both roundings), two a word
@@ -254,24 +288,54 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
             s_t2h[c2] = (uint32_t)__half_as_ushort(ha) | ((uint32_t)__half_as_ushort(hb) << 16);
         }
         fence_proxy_async_smem();
+        // Design blocks that may hold a row to collect, a chunk at a time: with
+        // boxes, those whose box lies within the largest threshold of the
+        // queries' box.  Every row of another block is further from every
+        // query than sqrt(tau2) (the FP32 evaluation's relative error is below
+        // 1e-5), outside the radius that tau2 guarantees collected.
+        for (int chunk = 0; chunk < a.nmb; chunk += TC_CHUNK) {
+        // (every role of the chunk before is done: a block-uniform verdict)
+        if (__syncthreads_or(*err != 0)) break;
+        if (tid == 0) s_nlist = 0;
         __syncthreads();
+        for (int m0 = chunk; m0 < min(chunk + TC_CHUNK, a.nmb); m0 += TC_THREADS) {
+            const int mb = m0 + tid;
+            bool take = mb < min(chunk + TC_CHUNK, a.nmb);
+            if (a.order.box && take) {
+                float lb = 0.f;
+                for (int i = 0; i < a.p; i++) {
+                    const float lo = a.order.box[(int64_t)i * a.nmb + mb], hi = a.order.box[(int64_t)(a.p + i) * a.nmb + mb];
+                    const float gap = fmaxf(fmaxf(fkey_inv(s_qlo[i]) - hi, lo - fkey_inv(s_qhi[i])), 0.f);
+                    lb = fmaf(gap, gap, lb);
+                }
+                take = !(lb * (1.f - 1e-5f) > fkey_inv(s_tmax));
+            }
+            const uint32_t vote = __ballot_sync(LAGP_FULL_MASK, take);
+            int at = 0;
+            if (lane == 0 && vote) at = atomicAdd(&s_nlist, __popc(vote));
+            at = __shfl_sync(LAGP_FULL_MASK, at, 0);
+            if (take) s_list[at + __popc(vote & ((1u << lane) - 1u))] = (uint16_t)(mb - chunk);
+        }
+        __syncthreads();
+        const int nlist = s_nlist;
 
         if (warp == 0) {
             if (lane == 0) {  // producer: design blocks into the stage ring
                 int issued = 0;
-                for (int mb = 0; mb < a.nmb && !*err; mb++) {
-                    if (a.stall && mb == 1) break;  // the MMA's wait on this block then runs out
-                    const long long it = it0 + mb;
+                for (int li = 0; li < nlist && !*err; li++) {
+                    if (a.stall && li == 1) break;  // the MMA's wait on this block then runs out
+                    const long long it = it0 + li;
+                    const int mb = chunk + s_list[li];
                     const int s = (int)(it % S);
                     const uint32_t round = (uint32_t)(it / S);
                     if (!mbar_wait(empty + s, (round & 1u) ^ 1u, err, 128)) break;
                     mbar_arrive_expect_tx(full + s, stage_bytes);
                     bulk_g2s(sA + (size_t)s * stage_halves, a.A + (size_t)mb * stage_halves, stage_bytes, full + s);
-                    issued = mb + 1;
+                    issued = li + 1;
                 }
                 if (*err && issued > 0) {  // let the copies in flight land before the CTA moves on
-                    for (int mb = max(0, issued - S); mb < issued; mb++) {
-                        const long long it = it0 + mb;
+                    for (int li = max(0, issued - S); li < issued; li++) {
+                        const long long it = it0 + li;
                         int quiet = 0;
                         mbar_wait(full + (int)(it % S), (uint32_t)(it / S) & 1u, &quiet);
                     }
@@ -282,8 +346,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
                 const uint32_t idesc = idesc_f16_f32(TC_MROWS, nmma);
                 const uint32_t qaddr = smem_u32(sQ);
                 long long last = -1;
-                for (int mb = 0; mb < a.nmb && !*err; mb++) {
-                    const long long it = it0 + mb;
+                for (int li = 0; li < nlist && !*err; li++) {
+                    const long long it = it0 + li;
                     const int s = (int)(it % S);
                     const int ac = (int)(it % TC_NACC);
                     if (!mbar_wait(full + s, (uint32_t)(it / S) & 1u, err, 32)) break;
@@ -308,9 +372,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
             const int g = (warp - 2) >> 2, quarter = warp & 3;
             uint2 *que = s_que + (size_t)(warp - 2) * TC_QUE;
             const uint32_t lt_mask = (1u << lane) - 1u;
-            for (int mb = 0; mb < a.nmb; mb++) {
-                const long long it = it0 + mb;
+            for (int li = 0; li < nlist; li++) {
+                const long long it = it0 + li;
                 if ((int)(it % TC_NACC) != g) continue;
+                const int mb = chunk + s_list[li];
                 // every lane waits; the warp goes on only together (the TMEM
                 // loads are warp-collective)
                 const bool ready = mbar_wait(tfull + g, (uint32_t)(it / TC_NACC) & 1u, err, 64);
@@ -382,11 +447,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
                         const int c = cb0 + (bit < 16 ? 2 * bit : 2 * (bit - 16) + 1);
                         mm &= mm - 1u;
                         const int pos = atomicAdd(&s_cnt[c], 1);
-                        if (pos < a.Cmax) a.cand[(q0 + c) * a.Cmax + pos] = hrow;
+                        if (pos < a.Cmax) a.cand[s_q[c] * (int64_t)a.Cmax + pos] = hrow;
                     }
                 }
                 __syncwarp();
             }
+        }
+        it0 += nlist;
         }
         __syncthreads();
         // per-query results: the collected rows and the threshold they were
@@ -395,7 +462,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
         // unscreened query goes to the exact retry
         const bool failed = *err != 0;
         for (int c = tid; c < nqb; c += TC_THREADS) {
-            const int64_t q = q0 + c;
+            const int64_t q = s_q[c];
             const int k = a.Np ? a.Np[q] : a.Npmax;
             const bool kvalid = k >= 1 && k <= a.Npmax;
             const bool ok = kvalid && s_tau2[c] == s_tau2[c];
@@ -405,13 +472,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
             a.rcol[q] = done ? __double2float_rd(tc_collected_radius(s_tau2[c] / s2, a.p, K, s_B)) : CUDART_NAN_F;
             if (a.status) a.status[q] = kvalid ? LAGP_OK : LAGP_EINVAL;
         }
-        it0 += a.nmb;
         __syncthreads();
         if (failed) {
-            // this and the CTA's remaining blocks go to the exact retry
-            for (int b2 = blk + gridDim.x; b2 < a.nblocks; b2 += gridDim.x)
+            // this CTA's block goes to the exact retry, and whatever blocks it
+            // can still take (the others may be failing too)
+            for (;;) {
+                if (tid == 0) s_blk = atomicAdd(a.counter, 1);
+                __syncthreads();
+                const int b2 = s_blk;
+                __syncthreads();
+                if (b2 >= a.nblocks) break;
                 for (int c = tid; c < a.nq && (int64_t)b2 * a.nq + c < a.M; c += TC_THREADS) {
-                    const int64_t q = (int64_t)b2 * a.nq + c;
+                    const int64_t q = a.order.query ? a.order.query[(int64_t)b2 * a.nq + c] : (int64_t)b2 * a.nq + c;
                     const int k = a.Np ? a.Np[q] : a.Npmax;
                     const bool kvalid = k >= 1 && k <= a.Npmax;
                     a.retry[q] = kvalid ? 1 : 0;
@@ -419,6 +491,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
                     a.rcol[q] = CUDART_NAN_F;
                     if (a.status) a.status[q] = kvalid ? LAGP_OK : LAGP_EINVAL;
                 }
+            }
             break;
         }
     }
@@ -447,22 +520,23 @@ size_t knn_tc_workspace(int64_t N, int64_t M, int p) {
 // collection pass.  ws: knn_tc_workspace(N, M, p) bytes.
 lagp_status launch_knn_tc_prep(lagp_ctx *ctx, void *ws, const void *X, int64_t N, int p, lagp_dtype dtype,
                                const void *Xref, int64_t M, const unsigned long long *kmax,
-                               const unsigned long long *kmin, float **tau0, float **rcol) {
+                               const unsigned long long *kmin, const KnnOrder &order, float **tau0, float **rcol) {
     const int K = tc_k(p);
     const int64_t Npad = round_up(std::max<int64_t>(N, 1), TC_MROWS);
     __half *A = static_cast<__half *>(ws);
     __half *Q = A + Npad * K;
     *tau0 = reinterpret_cast<float *>(Q + M * K);
     *rcol = *tau0 + M;
-    knn_tc_prep<<<ctx->num_sms * 4, 128, 0, ctx->stream>>>(X, N, Npad, Xref, M, p, dtype, kmax, kmin, A, Q);
+    knn_tc_prep<<<ctx->num_sms * 4, 128, 0, ctx->stream>>>(X, N, Npad, Xref, M, p, dtype, kmax, kmin, order, A, Q);
     ctx->launches++;
     return lagp_cuda_check(ctx, cudaGetLastError(), "knn_tc_prep");
 }
 
-lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, int64_t M, const int32_t *Np,
-                                  int32_t Npmax, const unsigned long long *kmax, const unsigned long long *kmin,
-                                  int32_t *cand, int32_t Cmax, int32_t *cand_count, int32_t *status,
-                                  int32_t *retry, int *err, float *rcol, float *dump) {
+lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, const void *Xref, lagp_dtype dtype,
+                                  int64_t M, const int32_t *Np, int32_t Npmax, const unsigned long long *kmax,
+                                  const unsigned long long *kmin, const KnnOrder &order, int32_t *cand, int32_t Cmax,
+                                  int32_t *cand_count, int32_t *status, int32_t *retry, int *err, int *counter,
+                                  float *rcol, float *dump) {
     const int K = tc_k(p);
     const int64_t Npad = round_up(std::max<int64_t>(N, 1), TC_MROWS);
     TcArgs a;
@@ -473,6 +547,10 @@ lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, int
     a.p = p;
     a.K = K;
     a.nmb = (int)(Npad / TC_MROWS);
+    a.order = order;
+    a.Xref = Xref;
+    a.dt = dtype;
+    a.counter = counter;
     a.tau0 = reinterpret_cast<const float *>(a.Q + M * K);
     a.rcol = rcol;
     a.Np = Np;
@@ -488,7 +566,10 @@ lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, int
     a.dump = dump;
     a.stall = ctx->knn_tc_stall;
     ctx->knn_tc_stall = 0;
-    // blocks: a multiple of the SM count (balanced waves), at most TC_QMAX queries each
+    // blocks: a multiple of the SM count (balanced waves), at most TC_QMAX
+    // queries each, taken from a counter (with boxes they cost unevenly;
+    // smaller blocks have smaller boxes, but blocks of 32 and 64 queries were
+    // no faster than 128)
     const int64_t sms = ctx->num_sms;
     const int64_t nb_min = (M + TC_QMAX - 1) / TC_QMAX;
     const int64_t nb = std::min<int64_t>(M, round_up(nb_min, sms));
@@ -496,13 +577,13 @@ lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, int
     a.nblocks = (int)((M + a.nq - 1) / a.nq);
     // as many stages as fit (at most TC_STAGES_MAX): the CTA then has the SM
     // (and its tensor memory) to itself
-    const size_t fixed = (size_t)TC_QMAX * K * 2 + (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS) * 4 +
+    const size_t fixed = (size_t)TC_QMAX * K * 2 + (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS + TC_CHUNK / 2) * 4 +
                          (2 * TC_STAGES_MAX + 2 * TC_NACC) * 8 + 1024;
     const size_t stage_bytes = (size_t)TC_MROWS * K * 2;
     a.stages = (int)std::min<size_t>(TC_STAGES_MAX, (ctx->smem_optin - fixed) / stage_bytes);
     if (a.stages < 2) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: tensor-core screen exceeds shared memory");
     size_t smem = (size_t)a.stages * stage_bytes + (size_t)TC_QMAX * K * 2 +
-                  (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS) * 4 +
+                  (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS + TC_CHUNK / 2) * 4 +
                   (2 * (size_t)a.stages + 2 * TC_NACC) * 8;
     // more than half of the SM's shared memory: one CTA per SM, which then
     // holds the whole tensor memory

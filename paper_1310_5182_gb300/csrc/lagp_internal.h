@@ -15,6 +15,7 @@ enum WsSlot {
     WS_KNN_CAND,      // kNN per-query candidate rows
     WS_KNN_META,      // kNN per-query counters / thresholds / flags
     WS_KNN_TC,        // kNN tensor-core operands and sampled thresholds
+    WS_KNN_ORDER,     // kNN spatial order of the design and the locations, bounding boxes
     WS_ALC_PANEL,     // ALC per-CTA candidate panel (F64 kernel values or F32 whitened U)
     WS_ALC_STATE,     // ALC per-CTA FP64 state (K^{-1}, vectors)
     WS_ALC_COUNTER,   // persistent-grid work counters
@@ -82,16 +83,26 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
                        const void *Xref, int64_t M, const int32_t *Np, int32_t Npmax,
                        int32_t *idx, int32_t *status);
 
+// Spatial order of a kNN launch: design rows and locations sorted by the cell
+// they lie in.  Null pointers: the given order, and every block is screened.
+struct KnnOrder {
+    const int32_t *row = nullptr;    // N: design row at each position
+    const int32_t *query = nullptr;  // M: location at each position
+    float *box = nullptr;            // bounding boxes of the blocks of 128 positions (centred
+                                     // coordinates): p x blocks lows, then p x blocks highs
+};
+
 // kNN collection pass on the tensor cores (knn_tc.cu)
 bool knn_tc_supported(int p);
 size_t knn_tc_workspace(int64_t N, int64_t M, int p);
 lagp_status launch_knn_tc_prep(lagp_ctx *ctx, void *ws, const void *X, int64_t N, int p, lagp_dtype dtype,
                                const void *Xref, int64_t M, const unsigned long long *kmax,
-                               const unsigned long long *kmin, float **tau0, float **rcol);
-lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, int64_t M, const int32_t *Np,
-                                  int32_t Npmax, const unsigned long long *kmax, const unsigned long long *kmin,
-                                  int32_t *cand, int32_t Cmax, int32_t *cand_count, int32_t *status,
-                                  int32_t *retry, int *err, float *rcol, float *dump);
+                               const unsigned long long *kmin, const KnnOrder &order, float **tau0, float **rcol);
+lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, const void *Xref, lagp_dtype dtype,
+                                  int64_t M, const int32_t *Np, int32_t Npmax, const unsigned long long *kmax,
+                                  const unsigned long long *kmin, const KnnOrder &order, int32_t *cand, int32_t Cmax,
+                                  int32_t *cand_count, int32_t *status, int32_t *retry, int *err, int *counter,
+                                  float *rcol, float *dump);
 lagp_status launch_knn_tc_dist(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtype dtype,
                                const void *Xref, int64_t M, float *out);
 lagp_status knn_last_stats(lagp_ctx *ctx, int64_t *n_retry, int32_t *tc_failed);
