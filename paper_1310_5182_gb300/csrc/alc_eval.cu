@@ -10,15 +10,30 @@
 //          q_c = z^T u_c = k_n(x)^T K_n^{-1} k_c, and
 //          Delta_c = (K(x_c, x) - q_c)^2 / (1 + g - s_c)
 //          (Eq. (dxy) with Eq. (piedef) after simplification).
-// The candidate kernel is one thread per candidate, 32-row blocks: the
+// In FP64 the candidate kernel is one thread per candidate, 32-row blocks: the
 // off-diagonal blocks L_IJ are staged in shared memory (read as broadcasts),
 // the current block's 32 values live in registers, earlier solved blocks
 // stream from a global panel W[i][c] (coalesced across the candidates).  Per
 // candidate n^2/2 FP64 FMAs with every lane busy: the FP64 unit bounds it.
+//
+// For nuggets below 1 the substitution runs in 59-bit fixed point on the
+// integer pipe instead (fx59.cuh): rows of L have norm < sqrt(2) and u_c is
+// bounded by the same, so a product costs three multiply-adds, 12 cycles a
+// warp instead of 64; the n exponentials of a candidate stay in FP64 and run
+// beside them.  A candidate's covariances are scaled by the power of two that
+// brings the largest near 1/8, so that far candidates keep their relative
+// precision.  L comes from the fixed-point factorisation for n <= 128 (one
+// CTA, 0.80 -> 0.23 ms at n = 128),
+// else from the FP64 one.  What leaves the range is redone in FP64 by the
+// conditional launches behind (one flag a candidate).  60,000 candidates,
+// n = 128: 1.36 -> 0.48 ms, 2.16 -> 0.70 ms a call.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "device_util.cuh"
 #include "exp64.cuh"
+#include "fx_chol.cuh"
 #include "lagp_internal.h"
 
 namespace {
@@ -30,8 +45,10 @@ constexpr int PREP_THREADS = 256;
 // One CTA: L (np x np, np = n rounded up to 32, identity padding), rd, z.
 __global__ void __launch_bounds__(PREP_THREADS)
 eval_prep_kernel(const void *X, int p, lagp_dtype dt, const double *x, const int32_t *design, int n,
-                 int np, double d, double g, double *L, double *rd, double *z, int32_t *status) {
+                 int np, double d, double g, double *L, double *rd, double *z, int32_t *status,
+                 const int *redo) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (redo && *redo == 0) return;  // (after the fixed-point kernels: nothing was left)
     double *xd = reinterpret_cast<double *>(smem_raw);  // n x p design coordinates
     double *kx = xd + (size_t)n * p;                    // np
     __shared__ int s_ok;
@@ -111,7 +128,8 @@ eval_prep_kernel(const void *X, int p, lagp_dtype dt, const double *x, const int
 __global__ void __launch_bounds__(EV_THREADS)
 eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const int32_t *design, int n,
                   int np, const int32_t *cands, int64_t Nc, double d, double g, const double *L,
-                  const double *rd, const double *z, double *W, double *delta, const int32_t *status) {
+                  const double *rd, const double *z, double *W, double *delta, const int32_t *status,
+                  const int *redo, const int32_t *left) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *blk = reinterpret_cast<double *>(smem_raw);  // EV_B x EV_B block of L
     double *xd = blk + EV_B * EV_B;                       // n x p design coordinates
@@ -119,6 +137,11 @@ eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const in
     __shared__ double etab[EXP64_TABLE_SIZE];
     const int tid = threadIdx.x;
     const int64_t c = (int64_t)blockIdx.x * EV_THREADS + tid;
+    if (redo && *redo == 0) return;
+    // after the fixed-point kernels: the candidates they left (all when the
+    // factorisation itself left the range)
+    const bool write = c < Nc && (!left || left[c] != 0);
+    if (left && !__syncthreads_or(write)) return;
     const bool live = c < Nc;
     for (int i = tid; i < EXP64_TABLE_SIZE; i += EV_THREADS) etab[i] = exp64_table_g[i];
     for (int e = tid; e < n * p; e += EV_THREADS) xd[e] = load_coord64(X, design[e / p], p, e % p, dt);
@@ -126,7 +149,7 @@ eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const in
     for (int i = 0; i < p; i++) xc[(size_t)tid * p + i] = load_coord64(X, crow, p, i, dt);
     __syncthreads();
     if (*status != LAGP_OK) {  // the design's K_n was not positive definite
-        if (live) delta[c] = CUDART_NAN;
+        if (write) delta[c] = CUDART_NAN;
         return;
     }
     const double ninv_d = -1.0 / d;
@@ -178,7 +201,7 @@ eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const in
             for (int r = 0; r < EV_B; r++) Wi[(size_t)r * Nc] = acc[r];
         }
     }
-    if (live) {
+    if (write) {
         double sk = 0.0;
         for (int t = 0; t < p; t++) {
             const double df = mx[t] - x[t];
@@ -188,6 +211,242 @@ eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const in
         const double minv = (1.0 + g) - s;                  // m^{-1}(x_c), Eq. (piedef)
         const double r = kap - q;
         delta[c] = minv > 0.0 ? r * r / minv : CUDART_NAN;
+    }
+}
+
+// ---------------------------------------------------------- fixed point
+
+constexpr int EF_THREADS = 64;   // candidates per CTA
+constexpr int EF_B = 16;         // rows per block of the substitution
+constexpr int EF_K = 64;         // earlier rows staged at a time
+constexpr int EF_HEAD = 3;       // covariances scaled to at most 2^-EF_HEAD: |u| up to 16 of them
+
+// Shared memory of the fixed-point prep: the matrix, then y_at as fx_chol.cuh
+// has it, then the design.
+__host__ __device__ inline size_t ef_prep_smem(int n, int p) {
+    return (size_t)fx_words(n, n + 1) * 16 + ((size_t)3 * n + (size_t)n * p) * 8;
+}
+
+// L (limbs, np x np row-major), 1 / diag (ry 2^(rt - 59)) and z = L^{-1} k_n(x)
+// 2^-ws (limbs), np = n rounded up to EF_B with identity rows.  One CTA, n <=
+// 128.  Out of range: *status = FX_REDO and *redo counts.
+__global__ void __launch_bounds__(FXT)
+eval_prep_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const int32_t *design, int n, int np,
+                    double d, double g, int2 *L, long long *ry, int *rt, int2 *z, int *ws, int32_t *status,
+                    int *redo) {
+    const int words = fx_words(n, n + 1), m = n + 1;
+    const FxFactor F{words, n, m, words * 16, n};
+    double *kx = fx_y(F), *xd = kx + 3 * n;  // (after the pivots)
+    __shared__ int red[FXW];
+    const Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
+    for (int e = b.tid; e < n * p; e += FXT) xd[e] = load_coord64(X, design[e / p], p, e % p, dt);
+    __syncthreads();
+    const double ninv_d = -1.0 / d;
+    bool odd = false;  // a distance that is not finite
+    for (int e = b.tid; e < n * (n + 1) / 2 + n; e += FXT) {
+        int i, k;
+        fx_tri(e, i, k);
+        const bool cross = i >= n;
+        const double D = sqd(cross ? x : xd + (size_t)i * p, xd + (size_t)k * p, p);
+        odd |= !(D < CUDART_INF);
+        const double E = exp64_tang(D * ninv_d, exp64_table_g);
+        if (cross) kx[k] = E;
+        else *fx_raw(F, 0, fx_slot(i, k, m)) = fx_from(i == k ? E + g : E);
+    }
+    const int ex = fx_exponent(kx, n, red, b);
+    bool ok = !(__syncthreads_or(odd) || ex == INT32_MAX);
+    if (ok) {
+        for (int k = b.tid; k < n; k += FXT) *fx_raw(F, 0, fx_slot(n, k, m)) = fx_from(fx_shift(kx[k], -(ex + 2)));
+        ok = !fx_factorise<1>(F, b);
+    }
+    if (!ok) {
+        if (b.tid == 0) {
+            *status = FX_REDO;
+            *redo = 1;
+        }
+        return;
+    }
+    for (int e = b.tid; e < np * np; e += FXT) {
+        const int i = e / np, k = e - i * np;
+        Fx f{i == k ? 1 << 29 : 0, 0};
+        if (i < n && k < n) f = k <= i ? fx_split(fx_load(F, 0, fx_slot(i, k, m))) : Fx{0, 0};
+        L[e] = make_int2(f.h, f.l);
+    }
+    for (int i = b.tid; i < np; i += FXT) {
+        ry[i] = i < n ? fx_ry(F)[i] : FX_ONE;
+        rt[i] = i < n ? fx_rt(F)[i] : 0;
+        const Fx f = i < n ? fx_split(fx_load(F, 0, fx_slot(n, i, m))) : Fx{0, 0};
+        z[i] = make_int2(f.h, f.l);
+    }
+    if (b.tid == 0) {
+        *ws = ex + 2;
+        *status = LAGP_OK;
+    }
+}
+
+// The same from the FP64 factor (n > 128): the limbs of its entries.
+__global__ void eval_limbs_kernel(const double *L64, const double *rd, const double *z64, int np64, int n, int np,
+                                  int2 *L, long long *ry, int *rt, int2 *z, int *ws, const int32_t *status,
+                                  int *redo) {
+    if (*status != LAGP_OK) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int e = tid; e < np * np; e += gridDim.x * blockDim.x) {
+        const int i = e / np, k = e - i * np;
+        const double v = i < n && k <= i ? L64[(size_t)i * np64 + k] : (i == k ? 1.0 : 0.0);
+        const Fx f = fx_split(fx_from(v));
+        L[e] = make_int2(f.h, f.l);
+    }
+    for (int i = tid; i < np; i += gridDim.x * blockDim.x) {
+        // rd = y 2^t with y in [0.5, 1)
+        const double r = i < n ? rd[i] : 1.0;
+        const int ex = ((__double2hiint(r) >> 20) & 0x7ff) - 1022;
+        if (ex < 0 || ex > 24) redo[0] = redo[1] = 1;  // (as fx_rsqrt's range)
+        rt[i] = ex;
+        ry[i] = fx_from(fx_shift(r, -ex));
+        const Fx f = fx_split(fx_from(i < n ? z64[i] : 0.0));
+        z[i] = make_int2(f.h, f.l);
+    }
+    if (tid == 0) *ws = 0;
+}
+
+__global__ void __launch_bounds__(EF_THREADS, 8)
+eval_cands_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const int32_t *design, int n, int np,
+                     const int32_t *cands, int64_t Nc, double d, double g, const int2 *__restrict__ L,
+                     const long long *__restrict__ ry, const int *__restrict__ rt, const int2 *__restrict__ z,
+                     const int *__restrict__ wsp, int2 *W, double *delta, const int32_t *status, int *redo,
+                     int32_t *left) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int4 *blk = reinterpret_cast<int4 *>(smem_raw);           // EF_K columns of EF_B rows (two rows a word)
+    double *xd = reinterpret_cast<double *>(blk + EF_K * EF_B / 2);  // n x p design coordinates
+    double *xc = xd + (size_t)n * p;                          // EF_THREADS x p candidate coordinates
+    float *xf = reinterpret_cast<float *>(xc + (size_t)EF_THREADS * p);  // both in FP32, relative to x
+    float *cf = xf + (size_t)n * p + (size_t)threadIdx.x * p;
+    __shared__ int2 s_y[EF_B], s_z[EF_B];
+    __shared__ int s_t[EF_B];
+    const int tid = threadIdx.x;
+    const int64_t c = (int64_t)blockIdx.x * EF_THREADS + tid;
+    const bool live = c < Nc;
+    const int32_t st = *status;
+    if (st != LAGP_OK || redo[1] != 0) {  // (redo[1]: limbs out of range)
+        if (live) {
+            left[c] = st == LAGP_ENOTPD ? 0 : 1;
+            if (st == LAGP_ENOTPD) delta[c] = CUDART_NAN;
+        }
+        return;
+    }
+    for (int e = tid; e < n * p; e += EF_THREADS) {
+        xd[e] = load_coord64(X, design[e / p], p, e % p, dt);
+        xf[e] = (float)(xd[e] - x[e % p]);
+    }
+    const int32_t crow = live ? cands[c] : cands[0];
+    double *mx = xc + (size_t)tid * p;
+    for (int i = 0; i < p; i++) {
+        mx[i] = load_coord64(X, crow, p, i, dt);
+        cf[i] = (float)(mx[i] - x[i]);
+    }
+    __syncthreads();
+    const double ninv_d = -1.0 / d;
+    // the scale: 2^e with max_i k_i 2^e near 2^-EF_HEAD, from the nearest design row in FP32
+    float near = CUDART_INF_F;
+    for (int r = 0; r < n; r++) {
+        float s = 0.f;
+        for (int t = 0; t < p; t++) {
+            const float df = cf[t] - xf[r * p + t];
+            s = fmaf(df, df, s);
+        }
+        near = fminf(near, s);
+    }
+    const int e2 = (int)fminf(near / (float)d * 1.4426950f, 900.f) - EF_HEAD;
+    unsigned bad = !(near < CUDART_INF_F);
+    long long sh = 0, sm = FX_HALF, qh = 0, qm = FX_HALF;  // |u|^2 and z^T u
+    const int nb = np / EF_B;
+    for (int I = 0; I < nb; I++) {
+        long long hi[EF_B], mid[EF_B];
+#pragma unroll
+        for (int r = 0; r < EF_B; r++) hi[r] = 0, mid[r] = FX_HALF;
+        for (int k0 = 0; k0 < I * EF_B; k0 += EF_K) {
+            const int kk = min(EF_K, I * EF_B - k0);
+            __syncthreads();
+            for (int e = tid; e < EF_B * kk; e += EF_THREADS) {
+                const int r = e / kk, k = e - r * kk;
+                reinterpret_cast<int2 *>(blk)[k * EF_B + r] = L[(size_t)(I * EF_B + r) * np + k0 + k];
+            }
+            __syncthreads();
+            const int2 *Wk = W + (size_t)k0 * Nc + (live ? c : 0);
+#pragma unroll 2
+            for (int k = 0; k < kk; k++) {
+                const int2 u = Wk[(size_t)k * Nc];
+                const int4 *row = blk + k * (EF_B / 2);
+#pragma unroll
+                for (int r = 0; r < EF_B; r += 2) {
+                    const int4 l = row[r / 2];
+                    hi[r] = fx_mad(u.x, l.x, hi[r]);
+                    mid[r] = fx_mad(u.y, l.x, fx_mad(u.x, l.y, mid[r]));
+                    hi[r + 1] = fx_mad(u.x, l.z, hi[r + 1]);
+                    mid[r + 1] = fx_mad(u.y, l.z, fx_mad(u.x, l.w, mid[r + 1]));
+                }
+            }
+        }
+        __syncthreads();
+        for (int e = tid; e < EF_B * EF_B; e += EF_THREADS) {
+            const int r = e / EF_B, k = e - r * EF_B;
+            reinterpret_cast<int2 *>(blk)[k * EF_B + r] = L[(size_t)(I * EF_B + r) * np + I * EF_B + k];
+        }
+        if (tid < EF_B) {
+            const Fx y = fx_split(ry[I * EF_B + tid]);
+            s_y[tid] = make_int2(y.h, y.l);
+            s_t[tid] = rt[I * EF_B + tid];
+            s_z[tid] = z[I * EF_B + tid];
+        }
+        __syncthreads();
+        int2 *Wi = W + (size_t)I * EF_B * Nc + c;
+#pragma unroll
+        for (int r = 0; r < EF_B; r++) {  // the diagonal block, in place
+            const int row = I * EF_B + r;
+            double kv = 0.0;
+            if (row < n) {
+                double sd = 0.0;
+                for (int t = 0; t < p; t++) {
+                    const double df = mx[t] - xd[(size_t)row * p + t];
+                    sd = fma(df, df, sd);
+                }
+                kv = fx_shift(exp64_tang(sd * ninv_d, exp64_table_g), e2);
+            }
+            const int2 y2 = s_y[r], z2 = s_z[r];
+            bad |= kv >= 1.0;
+            const long long S = fx_from(kv >= 1.0 ? 0.0 : kv) - (hi[r] << 1) - (mid[r] >> 29);
+            const Fx u = fx_split(fx_scaled(S, s_t[r], Fx{y2.x, y2.y}, bad));
+            bad |= fx_beyond_h(u);
+            sh = fx_mad(u.h, 2 * u.h, sh);
+            sm = fx_mid(sm, u, u);
+            qh = fx_mad(u.h, 2 * z2.x, qh);
+            qm = fx_mid(qm, u, Fx{z2.x, z2.y});
+#pragma unroll
+            for (int r2 = r + 1; r2 < EF_B; r2++) {
+                const int2 l = reinterpret_cast<const int2 *>(blk)[r * EF_B + r2];
+                hi[r2] = fx_mad(u.h, l.x, hi[r2]);
+                mid[r2] = fx_mad(u.l, l.x, fx_mad(u.h, l.y, mid[r2]));
+            }
+            if (live && I + 1 < nb) Wi[(size_t)r * Nc] = make_int2(u.h, u.l);
+        }
+    }
+    if (live) {
+        double sk = 0.0;
+        for (int t = 0; t < p; t++) {
+            const double df = mx[t] - x[t];
+            sk = fma(df, df, sk);
+        }
+        const double kap = exp64_tang(sk * ninv_d, exp64_table_g);  // K(x_c, x)
+        // |u|^2 < 4 in its scale, so that neither sum has wrapped
+        const long long sv = fx_sum(sh, sm), qv = fx_sum(qh, qm);
+        bad |= (unsigned long long)sv >= (1ull << 61);
+        const double s = scalbn(fx_double(sv), -2 * e2), q = scalbn(fx_double(qv), *wsp - e2);
+        const double minv = (1.0 + g) - s;  // m^{-1}(x_c), Eq. (piedef)
+        const double r = kap - q;
+        delta[c] = minv > 0.0 ? r * r / minv : CUDART_NAN;
+        bad |= !(minv > 0.0);  // (for FP64 to judge)
+        left[c] = bad ? 1 : 0;
+        if (bad) atomicExch(redo, 1);
     }
 }
 
@@ -207,26 +466,71 @@ extern "C" lagp_status lagp_alc_eval(lagp_ctx *ctx, const void *X, int64_t N, in
         return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_eval: need 1 <= n <= 1024, Nc >= 0, d > 0, g >= 0");
     LAGP_CUDA(ctx, cudaSetDevice(ctx->device));
     const int np = (n + EV_B - 1) / EV_B * EV_B;
-    const size_t wbytes = (size_t)np * np * 8 + 2 * (size_t)np * 8 + (size_t)np * (Nc > 0 ? Nc : 1) * 8;
-    double *Lm = static_cast<double *>(lagp_ws(ctx, WS_ALC_STATE, wbytes + 256));
-    if (!Lm) return LAGP_ENOMEM;
+    const int64_t nw = Nc > 0 ? Nc : 1;
+    // FP64: L, 1 / diag, z, the panel of solved rows; fixed point: the same in
+    // limbs (its panel in the same place), the exponents, the flags
+    const size_t wbytes = (size_t)np * np * 8 + 2 * (size_t)np * 8 + (size_t)np * nw * 8;
+    const size_t fbytes = (size_t)np * np * 8 + (size_t)np * 24 + (size_t)nw * 4 + 64;
+    const bool fixed = g < 1.0;
+    char *base = static_cast<char *>(lagp_ws(ctx, WS_ALC_STATE, wbytes + (fixed ? fbytes : 0) + 256));
+    if (!base) return LAGP_ENOMEM;
+    double *Lm = reinterpret_cast<double *>(base);
     double *rd = Lm + (size_t)np * np, *z = rd + np, *W = z + np;
+    int2 *fL = reinterpret_cast<int2 *>(base + wbytes);
+    long long *fry = reinterpret_cast<long long *>(fL + (size_t)np * np);
+    int2 *fz = reinterpret_cast<int2 *>(fry + np);
+    int *frt = reinterpret_cast<int *>(fz + np);
+    int *words = frt + np;  // [0] the scale of z, [1] work is left to FP64, [2] all of it
+    int32_t *left = words + 3;
     const size_t smem_prep = ((size_t)n * p + np) * 8;
-    if (smem_prep > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_eval: n x p too large");
-    cudaFuncSetAttribute(eval_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_prep);
-    eval_prep_kernel<<<1, PREP_THREADS, smem_prep, ctx->stream>>>(X, p, dtype, x, design, n, np, d, g, Lm,
-                                                                   rd, z, status);
-    ctx->launches++;
-    LAGP_CUDA(ctx, cudaGetLastError());
-    if (Nc == 0) return LAGP_OK;
     const size_t smem = ((size_t)EV_B * EV_B + (size_t)n * p + (size_t)EV_THREADS * p) * 8;
-    if (smem > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_eval: n x p too large");
-    cudaFuncSetAttribute(eval_cands_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int64_t grid = (Nc + EV_THREADS - 1) / EV_THREADS;
-    eval_cands_kernel<<<(unsigned)grid, EV_THREADS, smem, ctx->stream>>>(X, p, dtype, x, design, n, np, cands,
-                                                                         Nc, d, g, Lm, rd, z, W, delta,
-                                                                         status);
-    ctx->launches++;
+    if (smem_prep > ctx->smem_optin || (Nc > 0 && smem > ctx->smem_optin))
+        return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_eval: n x p too large");
+    cudaStream_t st = ctx->stream;
+    const int nf = (n + EF_B - 1) / EF_B * EF_B;
+    const size_t smem_fx = (size_t)EF_K * EF_B * 8 + ((size_t)n * p + (size_t)EF_THREADS * p) * 8 +
+                           ((size_t)n + EF_THREADS) * p * 4;
+    const bool fx = fixed && smem_fx <= ctx->smem_optin;
+    const bool fx_prep = fx && n <= FX_NMAX && ef_prep_smem(n, p) <= ctx->smem_optin;
+    auto prep64 = [&](const int *redo) {
+        cudaFuncSetAttribute(eval_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_prep);
+        eval_prep_kernel<<<1, PREP_THREADS, smem_prep, st>>>(X, p, dtype, x, design, n, np, d, g, Lm, rd, z, status,
+                                                             redo);
+        ctx->launches++;
+    };
+    if (fx) LAGP_CUDA(ctx, cudaMemsetAsync(words, 0, 12, st));
+    if (fx_prep) {
+        cudaFuncSetAttribute(eval_prep_fx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ef_prep_smem(n, p));
+        eval_prep_fx_kernel<<<1, FXT, ef_prep_smem(n, p), st>>>(X, p, dtype, x, design, n, nf, d, g, fL, fry, frt, fz,
+                                                                words, status, words + 1);
+        ctx->launches++;
+    } else {
+        prep64(nullptr);
+        if (fx && Nc > 0) {
+            eval_limbs_kernel<<<ctx->num_sms, 256, 0, st>>>(Lm, rd, z, np, n, nf, fL, fry, frt, fz, words, status,
+                                                            words + 1);
+            ctx->launches++;
+        }
+    }
+    LAGP_CUDA(ctx, cudaGetLastError());
+    if (fx && Nc > 0) {
+        cudaFuncSetAttribute(eval_cands_fx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fx);
+        eval_cands_fx_kernel<<<(unsigned)((Nc + EF_THREADS - 1) / EF_THREADS), EF_THREADS, smem_fx, st>>>(
+            X, p, dtype, x, design, n, nf, cands, Nc, d, g, fL, fry, frt, fz, words, reinterpret_cast<int2 *>(W), delta,
+            status, words + 1, left);
+        ctx->launches++;
+        LAGP_CUDA(ctx, cudaGetLastError());
+    }
+    // in FP64: everything, or what the fixed-point kernels left
+    if (fx_prep) prep64(words + 1);
+    if (Nc > 0) {
+        cudaFuncSetAttribute(eval_cands_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const int64_t grid = (Nc + EV_THREADS - 1) / EV_THREADS;
+        eval_cands_kernel<<<(unsigned)grid, EV_THREADS, smem, st>>>(X, p, dtype, x, design, n, np, cands, Nc, d, g, Lm,
+                                                                    rd, z, W, delta, status, fx ? words + 1 : nullptr,
+                                                                    fx ? left : nullptr);
+        ctx->launches++;
+    }
     LAGP_CUDA(ctx, cudaGetLastError());
     return LAGP_OK;
 }

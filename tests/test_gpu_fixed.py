@@ -82,3 +82,24 @@ def test_locations_left_to_fp64(L, O):
     Y[sel[4, 2]] = np.nan
     out = L.lagp_predict(dev(w.X), dev(Y), dev(Xref), dev(sel), n, d, 0.0)
     assert torch.isnan(out["mean"][4]) and int(out["status"][4]) == 0
+
+
+@pytest.mark.parametrize("n,g,d", [(1, 1e-4, 0.5), (2, 0.9, 0.5), (15, 1e-4, 0.05), (16, 1e-6, 0.5), (17, 1e-2, 2.0),
+                                   (33, 1.0, 0.5), (64, 1e-4, 0.02), (65, 1e-3, 0.5), (127, 1e-4, 0.5),
+                                   (128, 1e-2, 0.1), (129, 1e-4, 0.5), (200, 1e-3, 0.1)])
+def test_alc_eval_sizes_and_far_candidates(L, O, n, g, d):
+    """Edges of the 16-row blocks, both factorisations (n <= 128 and above),
+    the FP64 path (g = 1), candidates near and across the whole square (tiny
+    covariances); the bar of test_alc_eval_matches_oracle."""
+    w = W.toy2d(seed=52, N=6_000, M=1)
+    idx = O.knn(w.X, w.Xref, n + 200)[0]
+    design = idx[:n]
+    far = np.setdiff1d(np.arange(w.N), idx)[::8]
+    cands = np.concatenate([idx[n:], far]).astype(np.int32)
+    delta, st = L.lagp_alc_eval(dev(w.X), w.Xref[0], dev(design), dev(cands), d, g)
+    assert int(st.cpu()[0]) == 0
+    _, ds = O.alc_scores(w.X, w.Xref[0], design, cands, d, g)
+    A = w.X[design]
+    K = np.exp(-((A[:, None] - A[None]) ** 2).sum(-1) / d) + g * np.eye(n)
+    atol = 16 * np.finfo(np.float64).eps / g * max(1.0, np.linalg.cond(K) * g)
+    assert np.all(np.abs(delta.cpu().numpy() - ds) <= np.maximum(1e-6 * np.abs(ds), atol))
