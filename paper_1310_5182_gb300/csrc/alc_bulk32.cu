@@ -44,7 +44,7 @@
 // atomic work counter):
 //   FP32 group (warps 0-3): owns the candidates (slot c in thread c / CPT);
 //     lists the contenders, and runs the Schur pass of each step;
-//   double-float group (warps 4-7): re-scores the contenders
+//   double-float group (warps 4 and up): re-scores the contenders
 //     (R1 k_j(x_c), K(x_c,x): squared distances and Tang's exponential;
 //      R2 u_c = L^{-1} k_j(x_c); R3 |u_c|^2, w^T u_c, z^T u_c -> Delta;
 //      the argmax, ties to the lower design row), then grows L^{-1}, w, z
@@ -52,9 +52,9 @@
 // In a step with a single contender (the common case) the winner is known
 // as soon as the list is, so the FP32 group's Schur pass and the
 // double-float group's work on the winner run at the same time; with two or
-// more contenders the Schur pass waits for the argmax.  The groups meet at
-// two CTA barriers a step (three with several contenders); inside the
-// double-float group a named barrier orders its phases.
+// more contenders the Schur pass waits for the argmax, and until then the
+// whole CTA re-scores.  The groups meet at two CTA barriers a step; a named
+// barrier (or the CTA's, when all re-score) orders the phases between.
 //
 // Shared memory holds L^{-1} (transposed, an odd leading dimension so that
 // both its row and its column reads are free of bank conflicts, zero below
@@ -76,6 +76,7 @@
 #include <float.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "alc_common.cuh"
 #include "df64.cuh"
@@ -88,12 +89,17 @@ namespace {
 using alc::load_vec;
 using alc::store_vec;
 
-constexpr int THREADS = 256;
-constexpr int WARPS = THREADS / 32;
 constexpr int FTHREADS = 128;              // FP32 group: warps 0..3
 constexpr int FWARPS = FTHREADS / 32;
-constexpr int DTHREADS = THREADS - FTHREADS;  // double-float group: warps 4..7
-constexpr int DWARPS = DTHREADS / 32;
+// The double-float group has DT threads (warps 4 and up).  Its arithmetic is
+// laid out for DBASE of them, so that no result depends on DT.  DT = DBASE
+// where CTAs share an SM; with no more locations than SMs a CTA has one to
+// itself, and DWIDE threads take a step's contenders and exponentials in fewer
+// rounds: 100 locations of the 2-d toy 2.22 -> 1.53 ms, 152 locations with n =
+// 80, N' = 2000 4.34 -> 3.34 ms (640 threads: 1.65, 3.30; 256: 1.83, 3.66; at
+// 300 locations, two CTAs an SM, 128 threads are the faster: 1.08 against 1.31).
+constexpr int DBASE = 128, DWIDE = 384;
+constexpr int DPARTS = DBASE / 32;         // partial sums of the winner's b
 // Adaptive contender margin: FP32 scores within `margin` (relative) of the
 // FP32 maximum are re-scored, margin = min(rescore_rel, max(MARGIN_MIN,
 // MARGIN_KAPPA * err)), err = the largest FP32-vs-double-float score error
@@ -112,7 +118,7 @@ constexpr int LCAP = 32;
 // 2-d toy's search 1.59 -> 1.41 ms and the 1M-point workload's 203 -> 192 ms)
 constexpr int TMAX_CAP = 16;
 // rows of the partial contractions: a warp's, or a batch contender's
-__host__ __device__ __forceinline__ int b32_cprows(int tmax) { return tmax > WARPS ? tmax : WARPS; }
+__host__ __device__ __forceinline__ int b32_cprows(int tmax) { return tmax > 8 ? tmax : 8; }
 
 struct B32Params {
     AlcArgs a;
@@ -134,9 +140,10 @@ __host__ __device__ __forceinline__ int b32_ldl(int nmax) { return nmax | 1; }  
 __host__ __device__ __forceinline__ int b32_ldc(int nmax) { return (nmax + 2) & ~1; }  // >= nmax + 1
 __host__ __device__ __forceinline__ int b32_ldx(int nmax) { return (nmax + 1) & ~1; }  // >= nmax
 
-// the double-float group's barrier (named barrier 1, its 128 threads) and the
+// the double-float group's barrier (named barrier 1, its DT threads) and the
 // FP32 group's (named barrier 2)
-__device__ __forceinline__ void dsync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+template <int DT>
+__device__ __forceinline__ void dbar() { asm volatile("bar.sync 1, %0;" ::"n"(DT) : "memory"); }
 __device__ __forceinline__ void fsync() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
 
 __device__ __forceinline__ float f32_score(float cov, float v, float gf) {
@@ -229,14 +236,15 @@ __device__ __noinline__ void winner_scalars(dfl vs, dfl rs, dfl rys, int j, bool
 
 // resident CTAs per SM the register allocation is sized for (64 registers a
 // thread at four)
-template <int CPT>
+template <int CPT, int DT>
 constexpr int b32_min_blocks() {
-    return CPT >= 32 ? 2 : (CPT >= 16 ? 3 : 4);
+    return DT > DBASE ? 1 : (CPT >= 16 ? 2 : 4);
 }
 
-template <int CPT>
-__global__ void __launch_bounds__(THREADS, b32_min_blocks<CPT>())
+template <int CPT, int DT>
+__global__ void __launch_bounds__(FTHREADS + DT, b32_min_blocks<CPT, DT>())
 alc_bulk32_kernel(B32Params P) {
+    constexpr int THREADS = FTHREADS + DT;
     constexpr int NPAD = FTHREADS * CPT;
     // candidates of an FP32 thread per pass of the Schur recurrence
     constexpr int CH = CPT < 8 ? CPT : 8;
@@ -480,10 +488,267 @@ alc_bulk32_kernel(B32Params P) {
             }
             const bool lone = total == 1;  // the common case: no comparison to make
             const bool last = j + 1 >= nm;
-            // ---------------- the FP32 group: with a single contender the
-            // Schur pass starts now; with several it waits for the argmax
+            // ---------------- the re-score: the double-float group's while the
+            // FP32 group runs the Schur pass of a single contender's step; with
+            // several contenders that pass waits for the argmax, and the whole
+            // CTA re-scores (thread rt of RT, warp rw of RW).
+            // First, the previous winner's new row of L^{-1}, -b^T / lambda, from
+            // the warps' partials (deferred to here, where it overlaps the
+            // staging; the next R2 reads it after two barriers)
+            if (!fgroup && j > 1 && dt < j - 1) {
+                dfl b = ld2(cpart + dt);
+#pragma unroll
+                for (int q = 1; q < DPARTS; q++) b = df_add_sloppy(b, ld2(cpart + q * ldc + dt));
+                st2(LT + dt * ldl + j - 1, df_neg(df_mul(df_normalize(b), ld2(&s_il))));
+            }
+            auto rescore = [&](auto single) {
+                // (two bodies: a lone contender's step has no batches and no comparison left in it)
+                constexpr bool LONE = decltype(single)::value;
+                constexpr int RT = LONE ? DT : THREADS, RW = RT / 32;
+                const int tot = LONE ? 1 : total;
+                const int rt = fgroup ? DT + tid : dt, rw = rt >> 5;
+                const auto rsync = [] {
+                    if constexpr (LONE) dbar<DT>();
+                    else __syncthreads();
+                };
+                // Re-score in batches of at most tmax contenders, the consecutive
+                // chunks of the list (one batch holding every contender when there
+                // are at most tmax of them, the rule); when the running best
+                // improves in a batch that others follow, its vectors are kept
+                // (win_*) for the winner's phase
+                for (int b0 = 0; b0 < tot; b0 += tmax) {
+                    const int ncon = min(tmax, tot - b0), remaining = tot - b0 - ncon;
+                    // ---- the batch: its list entries, coordinates and responses
+                    if (rt < ncon) {
+                        const int e = b0 + rt, slot = e < LCAP ? lst_slot[e] : ov_slot[e];
+                        bat_slot[rt] = slot;
+                        bat_row[rt] = cands[slot];
+                        bat_s[rt] = e < LCAP ? lst_s[e] : ov_s[e];
+                        bat_v[rt] = e < LCAP ? lst_v[e] : ov_v[e];
+                        bat_r[rt] = e < LCAP ? lst_r[e] : ov_r[e];
+                        if (fused) con_y[rt] = Yc[slot];
+                    }
+                    #pragma unroll 1
+                    for (int e2 = rt; e2 < ncon * p; e2 += RT) {
+                        const int w = e2 / p, i = e2 - w * p, e = b0 + w;
+                        const int slot = e < LCAP ? lst_slot[e] : ov_slot[e];
+                        con_x[e2] = make_float2(Cg[i * NPAD + slot], x64 ? Clo[i * NPAD + slot] : 0.f);
+                    }
+                    rsync();
+                    // ---- R1: k_j(x_c) (t < j) and K(x_c, x) (t = j) in double-float;
+                    // each squared distance split over G lanes (G in 1, 2, 4).  G,
+                    // and R2's layout below, follow the step's contender count, not
+                    // the batch's, so that a contender's arithmetic (and every
+                    // result) is the same for any batch size
+                    {
+                        const int jp = j + 1, pairs = ncon * jp, tpairs = min(tot, TMAX_CAP) * jp;
+                        const int G = tpairs * 4 <= DBASE ? 4 : (tpairs * 2 <= DBASE ? 2 : 1);
+                        const int gi = rt & (G - 1), per = RT / G;
+                        for (int base = 0; base < pairs; base += per) {
+                            const int pr = base + rt / G;
+                            const bool ok = pr < pairs;
+                            const int w = ok ? pr / jp : 0, t = ok ? pr - w * jp : 0;
+                            const float2 *cx = con_x + w * p;
+                            dfl s = df_zero();
+                            for (int i = gi; i < p; i += G) {
+                                const float2 xt = t < j ? xdd[i * ldx + t] : xqd[i];
+                                const float2 xc = cx[i];
+                                dfl df = two_sum(xc.x, -xt.x);
+                                df.lo = __fadd_rn(df.lo, __fsub_rn(xc.y, xt.y));
+                                // (df.hi + df.lo)^2 with the exact leading product
+                                const dfl sq = two_prod(df.hi, df.hi);
+                                const float sql = __fmaf_rn(df.hi + df.hi, df.lo, sq.lo);
+                                const dfl ss = two_sum(s.hi, sq.hi);
+                                s.hi = ss.hi;
+                                s.lo = __fadd_rn(s.lo, __fadd_rn(ss.lo, sql));
+                            }
+                            s = df_normalize(s);
+                            for (int o = 1; o < G; o <<= 1)
+                                s = df_add_sloppy(s, dfl{__shfl_xor_sync(LAGP_FULL_MASK, s.hi, o),
+                                                         __shfl_xor_sync(LAGP_FULL_MASK, s.lo, o)});
+                            const dfl kv = df_exp(df_neg(df_mul(s, inv_d)), etab);
+                            if (ok && gi == 0) st2(con_k + w * ldc + t, kv);
+                        }
+                    }
+                    rsync();
+                    // ---- R2: u_c = L^{-1} k_j(x_c): with one or two contenders
+                    // each contender's rows split over wpc warps; with more, one
+                    // thread per (contender, t) over the whole group (two
+                    // accumulation chains), so that the chains are j/2 long
+                    const int wpc = tot == 1 ? 4 : (tot == 2 ? 2 : 1);
+                    if (j > 0) {
+                        if (tot >= 3) {
+                            for (int e = rt; e < ncon * j; e += RT) {
+                                const int w = e / j, t = e - w * j;
+                                const float2 *kc = con_k + w * ldc;
+                                dfl a0 = df_zero(), a1 = df_zero();
+                                int s = 0;
+                                for (; s < t; s += 2) {
+                                    df_fma_acc(a0, ld2(LT + s * ldl + t), ld2(kc + s));
+                                    df_fma_acc(a1, ld2(LT + (s + 1) * ldl + t), ld2(kc + s + 1));
+                                }
+                                if (s == t) df_fma_acc(a0, ld2(LT + s * ldl + t), ld2(kc + s));
+                                st2(cpart + w * ldc + t, df_add(df_normalize(a0), df_normalize(a1)));
+                            }
+                        } else {
+                            for (int item = rw; item < ncon * wpc; item += RW) {
+                                const int w = item / wpc, part = item - w * wpc;
+                                df_tri_lower(con_k + w * ldc, LT, ldl, part * j / wpc, (part + 1) * j / wpc, j, lane,
+                                             cpart + item * ldc);
+                            }
+                        }
+                    }
+                    rsync();
+                    // ---- R3: u_c from the partials; |u_c|^2, w^T u_c, z^T u_c by
+                    // one warp per contender -> v_c, r_c and (fused) y_c - z^T u_c.
+                    // The step's only contender is decided here, and its warp goes
+                    // on to the winner's scalars.
+                    #pragma unroll 1
+                    for (int w = rw; w < ncon; w += RW) {
+                        dfl uu = df_zero(), uw = df_zero(), uz = df_zero();
+                        float2 *uc = con_u + w * ldc;
+                        #pragma unroll 1
+                        for (int t = lane; t < j; t += 32) {
+                            const float2 *P0 = cpart + w * wpc * ldc + t;
+                            dfl ut = ld2(P0);
+                            #pragma unroll 1
+                            for (int q = 1; q < wpc; q++) ut = df_add_sloppy(ut, ld2(P0 + q * ldc));
+                            ut = df_normalize(ut);
+                            st2(uc + t, ut);
+                            df_fma_acc(uu, ut, ut);
+                            df_fma_acc(uw, ut, ld2(wv + t));
+                            if (fused) df_fma_acc(uz, ut, ld2(zv + t));
+                        }
+                        uu = df_normalize(uu);
+                        uw = df_normalize(uw);
+                        uz = df_normalize(uz);
+#pragma unroll 1
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const dfl ou{__shfl_xor_sync(LAGP_FULL_MASK, uu.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uu.lo, o)};
+                            const dfl ow{__shfl_xor_sync(LAGP_FULL_MASK, uw.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uw.lo, o)};
+                            const dfl oz{__shfl_xor_sync(LAGP_FULL_MASK, uz.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uz.lo, o)};
+                            uu = df_add_sloppy(uu, ou);
+                            uw = df_add_sloppy(uw, ow);
+                            uz = df_add_sloppy(uz, oz);
+                        }
+                        const dfl vc = df_sub(onepg, uu);                       // m_j^{-1}(x_c)
+                        const dfl rc = df_sub(ld2(con_k + w * ldc + j), uw);     // K(x_c,x) - w^T u_c
+                        const dfl ryc = fused ? df_sub(ld2(con_y + w), uz) : df_zero();
+                        if (lane == 0) {
+                            st2(con_v + w, vc);
+                            st2(con_r + w, rc);
+                            st2(con_ry + w, ryc);
+                        }
+                        if (LONE) {
+                            // the only contender is the winner when v > 0 (its
+                            // Delta is computed in the winner phase, off this chain)
+                            if (vc.hi > 0.f && rc.hi == rc.hi) {
+                                if (lane == 0) {
+                                    best_row = bat_row[0];
+                                    best_slot = bat_slot[0];
+                                    best_v = bat_v[0];
+                                    best_r = bat_r[0];
+                                    best_dl = make_float2(0.f, 0.f);  // (computed below)
+                                    s_wl = 0;
+                                    s_work[1] += 1ull;
+                                    s_work[2] += (unsigned long long)j;
+                                    s_work[3] += (unsigned long long)j * j;
+                                }
+                                winner_scalars(vc, rc, ryc, j, fused, sel, bat_row[0], lane, wv, zv, LT, ldl, s_il, s_qx,
+                                               s_psi, s_mean, s_total);
+                            }
+                        }
+                    }
+                    rsync();
+                    if (LONE) break;
+                    // ---- R4: Delta = r^2 / v in the lanes of one warp; the batch's
+                    // best against the running best
+                    if (rw == 0) {
+                        dfl dl = dfl{-FLT_MAX, 0.f};
+                        int row = INT32_MAX, slot = -1;
+                        float err = 0.f, bv = 0.f, bc = 0.f;
+                        if (lane < ncon) {
+                            const dfl vc = ld2(con_v + lane);
+                            if (vc.hi > 0.f) {
+                                dl = df_div(df_sqr(ld2(con_r + lane)), vc);
+                                if (!(dl.hi == dl.hi)) {
+                                    dl = dfl{-FLT_MAX, 0.f};
+                                } else {
+                                    row = bat_row[lane];
+                                    slot = bat_slot[lane];
+                                    bv = bat_v[lane];
+                                    bc = bat_r[lane];
+                                }
+                                // (the error against the step's best score below:
+                                // a low contender's error cannot displace the best)
+                                if (j >= a.n0 && dl.hi > 0.f) err = fabsf(bat_s[lane] - dl.hi);
+                            }
+                        }
+                        int wl = lane;
+#pragma unroll 1
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const float oh = __shfl_xor_sync(LAGP_FULL_MASK, dl.hi, o);
+                            const float ol = __shfl_xor_sync(LAGP_FULL_MASK, dl.lo, o);
+                            const int orow = __shfl_xor_sync(LAGP_FULL_MASK, row, o);
+                            const int oslot = __shfl_xor_sync(LAGP_FULL_MASK, slot, o);
+                            const int owl = __shfl_xor_sync(LAGP_FULL_MASK, wl, o);
+                            const float obv = __shfl_xor_sync(LAGP_FULL_MASK, bv, o);
+                            const float obc = __shfl_xor_sync(LAGP_FULL_MASK, bc, o);
+                            const dfl od{oh, ol};
+                            if (df_gt(od, dl) || (!df_gt(dl, od) && orow < row)) {
+                                dl = od;
+                                row = orow;
+                                slot = oslot;
+                                wl = owl;
+                                bv = obv;
+                                bc = obc;
+                            }
+                            err = fmaxf(err, __shfl_xor_sync(LAGP_FULL_MASK, err, o));
+                        }
+                        if (lane == 0) {
+                            const dfl bd = ld2(&best_dl);
+                            s_steperr = fmaxf(s_steperr, err);  // (absolute: divided by the step's best below)
+                            const bool improved = slot >= 0 && (df_gt(dl, bd) || (!df_gt(bd, dl) && row < best_row));
+                            if (improved) {
+                                st2(&best_dl, dl);
+                                best_row = row;
+                                best_slot = slot;
+                                best_v = bv;
+                                best_r = bc;
+                                s_wl = wl;
+                                s_win_saved = remaining > 0;  // (copied below: later batches overwrite)
+                            }
+                            s_save = improved && remaining > 0;
+                            s_work[1] += (unsigned long long)ncon;
+                            s_work[2] += (unsigned long long)ncon * j;
+                            s_work[3] += (unsigned long long)ncon * j * j;
+                        }
+                    }
+                    rsync();
+                    // (s_save is written again only after the next batch has passed
+                    // four more barriers, so every thread reads this value)
+                    if (s_save) {
+                        // the new running best's vectors, before the next batch
+                        // overwrites the batch arrays
+                        const int wl = s_wl;
+                        #pragma unroll 1
+                        for (int t = rt; t < j; t += RT) win_u[t] = con_u[wl * ldc + t];
+                        #pragma unroll 1
+                        for (int i = rt; i < p; i += RT) win_x[i] = con_x[wl * p + i];
+                        if (rt == 0) {
+                            win_s[0] = con_v[wl];
+                            win_s[1] = con_r[wl];
+                            win_s[2] = con_ry[wl];
+                        }
+                        rsync();
+                    }
+                }
+            };
+            if (!lone) rescore(std::false_type{});
+            else if (!fgroup) rescore(std::true_type{});
+            // ---------------- the FP32 group's Schur pass (a single contender:
+            // beside the re-score; several: from the argmax on)
             if (fgroup) {
-                if (!lone) __syncthreads();  // (matched by the double-float group after its argmax)
                 int cstar;
                 float pv, pr;
                 if (lone) {
@@ -498,7 +763,7 @@ alc_bulk32_kernel(B32Params P) {
 #pragma unroll
                 for (int r = 0; r < CPT; r++)
                     if (c0 + r == cstar) chosen |= 1u << r;
-                if (!last) {
+                if (!last && cstar >= 0) {  // (no valid contender: the step's end)
                     // ---------------- FP32 Schur recurrence with pivot x* (new
                     // column j of U), from the pivot's own FP32 state
                     const float inv_lam = rsqrtf(fmaxf(pv, gf));
@@ -567,250 +832,7 @@ alc_bulk32_kernel(B32Params P) {
                 }
                 continue;  // to the next step's barrier
             }
-            // ---------------- the double-float group.  First the previous
-            // winner's new row of L^{-1}, -b^T / lambda, from the warps' partials
-            // (deferred to here, where it overlaps the staging; the next R2
-            // reads it after two barriers)
-            if (j > 1 && dt < j - 1) {
-                dfl b = ld2(cpart + dt);
-#pragma unroll
-                for (int q = 1; q < DWARPS; q++) b = df_add_sloppy(b, ld2(cpart + q * ldc + dt));
-                st2(LT + dt * ldl + j - 1, df_neg(df_mul(df_normalize(b), ld2(&s_il))));
-            }
-            // Re-score in batches of at most tmax contenders, the consecutive
-            // chunks of the list (one batch holding every contender when there
-            // are at most tmax of them, the rule); when the running best
-            // improves in a batch that others follow, its vectors are kept
-            // (win_*) for the winner's phase
-            for (int b0 = 0; b0 < total; b0 += tmax) {
-                const int ncon = min(tmax, total - b0), remaining = total - b0 - ncon;
-                // ---- the batch: its list entries, coordinates and responses
-                if (dt < ncon) {
-                    const int e = b0 + dt, slot = e < LCAP ? lst_slot[e] : ov_slot[e];
-                    bat_slot[dt] = slot;
-                    bat_row[dt] = cands[slot];
-                    bat_s[dt] = e < LCAP ? lst_s[e] : ov_s[e];
-                    bat_v[dt] = e < LCAP ? lst_v[e] : ov_v[e];
-                    bat_r[dt] = e < LCAP ? lst_r[e] : ov_r[e];
-                    if (fused) con_y[dt] = Yc[slot];
-                }
-                #pragma unroll 1
-                for (int e2 = dt; e2 < ncon * p; e2 += DTHREADS) {
-                    const int w = e2 / p, i = e2 - w * p, e = b0 + w;
-                    const int slot = e < LCAP ? lst_slot[e] : ov_slot[e];
-                    con_x[e2] = make_float2(Cg[i * NPAD + slot], x64 ? Clo[i * NPAD + slot] : 0.f);
-                }
-                dsync();
-                // ---- R1: k_j(x_c) (t < j) and K(x_c, x) (t = j) in double-float;
-                // each squared distance split over G lanes (G in 1, 2, 4).  G,
-                // and R2's layout below, follow the step's contender count, not
-                // the batch's, so that a contender's arithmetic (and every
-                // result) is the same for any batch size
-                {
-                    const int jp = j + 1, pairs = ncon * jp, tpairs = min(total, TMAX_CAP) * jp;
-                    const int G = tpairs * 4 <= DTHREADS ? 4 : (tpairs * 2 <= DTHREADS ? 2 : 1);
-                    const int gi = dt & (G - 1), per = DTHREADS / G;
-                    for (int base = 0; base < pairs; base += per) {
-                        const int pr = base + dt / G;
-                        const bool ok = pr < pairs;
-                        const int w = ok ? pr / jp : 0, t = ok ? pr - w * jp : 0;
-                        const float2 *cx = con_x + w * p;
-                        dfl s = df_zero();
-                        for (int i = gi; i < p; i += G) {
-                            const float2 xt = t < j ? xdd[i * ldx + t] : xqd[i];
-                            const float2 xc = cx[i];
-                            dfl df = two_sum(xc.x, -xt.x);
-                            df.lo = __fadd_rn(df.lo, __fsub_rn(xc.y, xt.y));
-                            // (df.hi + df.lo)^2 with the exact leading product
-                            const dfl sq = two_prod(df.hi, df.hi);
-                            const float sql = __fmaf_rn(df.hi + df.hi, df.lo, sq.lo);
-                            const dfl ss = two_sum(s.hi, sq.hi);
-                            s.hi = ss.hi;
-                            s.lo = __fadd_rn(s.lo, __fadd_rn(ss.lo, sql));
-                        }
-                        s = df_normalize(s);
-                        for (int o = 1; o < G; o <<= 1)
-                            s = df_add_sloppy(s, dfl{__shfl_xor_sync(LAGP_FULL_MASK, s.hi, o),
-                                                     __shfl_xor_sync(LAGP_FULL_MASK, s.lo, o)});
-                        const dfl kv = df_exp(df_neg(df_mul(s, inv_d)), etab);
-                        if (ok && gi == 0) st2(con_k + w * ldc + t, kv);
-                    }
-                }
-                dsync();
-                // ---- R2: u_c = L^{-1} k_j(x_c): with one or two contenders
-                // each contender's rows split over wpc warps; with more, one
-                // thread per (contender, t) over the whole group (two
-                // accumulation chains), so that the chains are j/2 long
-                const int wpc = total == 1 ? 4 : (total == 2 ? 2 : 1);
-                if (j > 0) {
-                    if (total >= 3) {
-                        for (int e = dt; e < ncon * j; e += DTHREADS) {
-                            const int w = e / j, t = e - w * j;
-                            const float2 *kc = con_k + w * ldc;
-                            dfl a0 = df_zero(), a1 = df_zero();
-                            int s = 0;
-                            for (; s < t; s += 2) {
-                                df_fma_acc(a0, ld2(LT + s * ldl + t), ld2(kc + s));
-                                df_fma_acc(a1, ld2(LT + (s + 1) * ldl + t), ld2(kc + s + 1));
-                            }
-                            if (s == t) df_fma_acc(a0, ld2(LT + s * ldl + t), ld2(kc + s));
-                            st2(cpart + w * ldc + t, df_add(df_normalize(a0), df_normalize(a1)));
-                        }
-                    } else {
-                        for (int item = dw; item < ncon * wpc; item += DWARPS) {
-                            const int w = item / wpc, part = item - w * wpc;
-                            df_tri_lower(con_k + w * ldc, LT, ldl, part * j / wpc, (part + 1) * j / wpc, j, lane,
-                                         cpart + item * ldc);
-                        }
-                    }
-                }
-                dsync();
-                // ---- R3: u_c from the partials; |u_c|^2, w^T u_c, z^T u_c by
-                // one warp per contender -> v_c, r_c and (fused) y_c - z^T u_c.
-                // The step's only contender is decided here, and its warp goes
-                // on to the winner's scalars.
-                #pragma unroll 1
-                for (int w = dw; w < ncon; w += DWARPS) {
-                    dfl uu = df_zero(), uw = df_zero(), uz = df_zero();
-                    float2 *uc = con_u + w * ldc;
-                    #pragma unroll 1
-                    for (int t = lane; t < j; t += 32) {
-                        const float2 *P0 = cpart + w * wpc * ldc + t;
-                        dfl ut = ld2(P0);
-                        #pragma unroll 1
-                        for (int q = 1; q < wpc; q++) ut = df_add_sloppy(ut, ld2(P0 + q * ldc));
-                        ut = df_normalize(ut);
-                        st2(uc + t, ut);
-                        df_fma_acc(uu, ut, ut);
-                        df_fma_acc(uw, ut, ld2(wv + t));
-                        if (fused) df_fma_acc(uz, ut, ld2(zv + t));
-                    }
-                    uu = df_normalize(uu);
-                    uw = df_normalize(uw);
-                    uz = df_normalize(uz);
-#pragma unroll 1
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const dfl ou{__shfl_xor_sync(LAGP_FULL_MASK, uu.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uu.lo, o)};
-                        const dfl ow{__shfl_xor_sync(LAGP_FULL_MASK, uw.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uw.lo, o)};
-                        const dfl oz{__shfl_xor_sync(LAGP_FULL_MASK, uz.hi, o), __shfl_xor_sync(LAGP_FULL_MASK, uz.lo, o)};
-                        uu = df_add_sloppy(uu, ou);
-                        uw = df_add_sloppy(uw, ow);
-                        uz = df_add_sloppy(uz, oz);
-                    }
-                    const dfl vc = df_sub(onepg, uu);                       // m_j^{-1}(x_c)
-                    const dfl rc = df_sub(ld2(con_k + w * ldc + j), uw);     // K(x_c,x) - w^T u_c
-                    const dfl ryc = fused ? df_sub(ld2(con_y + w), uz) : df_zero();
-                    if (lane == 0) {
-                        st2(con_v + w, vc);
-                        st2(con_r + w, rc);
-                        st2(con_ry + w, ryc);
-                    }
-                    if (lone) {
-                        // the only contender is the winner when v > 0 (its
-                        // Delta is computed in the winner phase, off this chain)
-                        if (vc.hi > 0.f && rc.hi == rc.hi) {
-                            if (lane == 0) {
-                                best_row = bat_row[0];
-                                best_slot = bat_slot[0];
-                                best_v = bat_v[0];
-                                best_r = bat_r[0];
-                                best_dl = make_float2(0.f, 0.f);  // (computed below)
-                                s_wl = 0;
-                                s_work[1] += 1ull;
-                                s_work[2] += (unsigned long long)j;
-                                s_work[3] += (unsigned long long)j * j;
-                            }
-                            winner_scalars(vc, rc, ryc, j, fused, sel, bat_row[0], lane, wv, zv, LT, ldl, s_il, s_qx,
-                                           s_psi, s_mean, s_total);
-                        }
-                    }
-                }
-                dsync();
-                if (lone) break;
-                // ---- R4: Delta = r^2 / v in the lanes of one warp; the batch's
-                // best against the running best
-                if (dw == 0) {
-                    dfl dl = dfl{-FLT_MAX, 0.f};
-                    int row = INT32_MAX, slot = -1;
-                    float err = 0.f, bv = 0.f, bc = 0.f;
-                    if (lane < ncon) {
-                        const dfl vc = ld2(con_v + lane);
-                        if (vc.hi > 0.f) {
-                            dl = df_div(df_sqr(ld2(con_r + lane)), vc);
-                            if (!(dl.hi == dl.hi)) {
-                                dl = dfl{-FLT_MAX, 0.f};
-                            } else {
-                                row = bat_row[lane];
-                                slot = bat_slot[lane];
-                                bv = bat_v[lane];
-                                bc = bat_r[lane];
-                            }
-                            // (the error against the step's best score below:
-                            // a low contender's error cannot displace the best)
-                            if (j >= a.n0 && dl.hi > 0.f) err = fabsf(bat_s[lane] - dl.hi);
-                        }
-                    }
-                    int wl = lane;
-#pragma unroll 1
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float oh = __shfl_xor_sync(LAGP_FULL_MASK, dl.hi, o);
-                        const float ol = __shfl_xor_sync(LAGP_FULL_MASK, dl.lo, o);
-                        const int orow = __shfl_xor_sync(LAGP_FULL_MASK, row, o);
-                        const int oslot = __shfl_xor_sync(LAGP_FULL_MASK, slot, o);
-                        const int owl = __shfl_xor_sync(LAGP_FULL_MASK, wl, o);
-                        const float obv = __shfl_xor_sync(LAGP_FULL_MASK, bv, o);
-                        const float obc = __shfl_xor_sync(LAGP_FULL_MASK, bc, o);
-                        const dfl od{oh, ol};
-                        if (df_gt(od, dl) || (!df_gt(dl, od) && orow < row)) {
-                            dl = od;
-                            row = orow;
-                            slot = oslot;
-                            wl = owl;
-                            bv = obv;
-                            bc = obc;
-                        }
-                        err = fmaxf(err, __shfl_xor_sync(LAGP_FULL_MASK, err, o));
-                    }
-                    if (lane == 0) {
-                        const dfl bd = ld2(&best_dl);
-                        s_steperr = fmaxf(s_steperr, err);  // (absolute: divided by the step's best below)
-                        const bool improved = slot >= 0 && (df_gt(dl, bd) || (!df_gt(bd, dl) && row < best_row));
-                        if (improved) {
-                            st2(&best_dl, dl);
-                            best_row = row;
-                            best_slot = slot;
-                            best_v = bv;
-                            best_r = bc;
-                            s_wl = wl;
-                            s_win_saved = remaining > 0;  // (copied below: later batches overwrite)
-                        }
-                        s_save = improved && remaining > 0;
-                        s_work[1] += (unsigned long long)ncon;
-                        s_work[2] += (unsigned long long)ncon * j;
-                        s_work[3] += (unsigned long long)ncon * j * j;
-                    }
-                }
-                dsync();
-                // (s_save is written again only after the next batch has passed
-                // four more barriers, so every thread reads this value)
-                if (s_save) {
-                    // the new running best's vectors, before the next batch
-                    // overwrites the batch arrays
-                    const int wl = s_wl;
-                    #pragma unroll 1
-                    for (int t = dt; t < j; t += DTHREADS) win_u[t] = con_u[wl * ldc + t];
-                    #pragma unroll 1
-                    for (int i = dt; i < p; i += DTHREADS) win_x[i] = con_x[wl * p + i];
-                    if (dt == 0) {
-                        win_s[0] = con_v[wl];
-                        win_s[1] = con_r[wl];
-                        win_s[2] = con_ry[wl];
-                    }
-                    dsync();
-                }
-            }
-            // several contenders: release the FP32 group with the winner
-            if (!lone) __syncthreads();
+            // ---------------- the double-float group: the winner
             if (best_slot < 0) {
                 // no valid contender (for a lone contender: v <= 0 in
                 // double-float, while the FP32 group went ahead with it)
@@ -841,17 +863,17 @@ alc_bulk32_kernel(B32Params P) {
                 if (alc && j >= a.n0) alc[j] = df_to_double(dl);
                 if (j >= a.n0) s_err = fmaxf(ERR_DECAY * s_err, err);
             }
-            if (!last && j > 0) {
+            if (!last && j > 0 && dw < DPARTS) {
                 // warp dw takes t in [t0, t1): equal lengths, so that the
-                // longest chain is j / DWARPS; its partial covers s < t1
-                const int t0 = dw * j / DWARPS, t1 = (dw + 1) * j / DWARPS;
+                // longest chain is j / DPARTS; its partial covers s < t1
+                const int t0 = dw * j / DPARTS, t1 = (dw + 1) * j / DPARTS;
                 float2 *part = cpart + dw * ldc;
                 df_tri_upper(wu, LT, ldl, t0, t1, lane, part);
                 #pragma unroll 1
                 for (int s = t1 + lane; s < j; s += 32) part[s] = make_float2(0.f, 0.f);
             }
             #pragma unroll 1
-            for (int i = dt; i < p; i += DTHREADS) xdd[i * ldx + j] = wx[i];
+            for (int i = dt; i < p; i += DT) xdd[i * ldx + j] = wx[i];
         }
         // (a double-float failure in the last step is seen here)
         __syncthreads();
@@ -891,23 +913,27 @@ size_t b32_smem_bytes(int nmax, int p, int tmax, int npad) {
            4 * 2 * (size_t)npad + 16;
 }
 
-template <int CPT>
+template <int CPT, int DT>
 lagp_status launch_b32(lagp_ctx *ctx, const AlcArgs &a) {
     constexpr int NPAD = FTHREADS * CPT;
     cudaStream_t st = ctx->stream;
     const std::string key = alc_shape_key("alc_f32", CPT, a.nmax, a.p, a.mean != nullptr);
-    int tmax = std::max(1, std::min(alc_rescore_batch(ctx, key), TMAX_CAP));
+    // (a CTA alone on its SM has shared memory for the largest batch: the 2-d
+    // toy 1.53 -> 1.31 ms.  The wide candidate sets re-score many contenders a
+    // step: the slab 51.4 -> 49.1 ms, the uneven borehole 348 -> 326 ms at two
+    // CTAs an SM.  Four CTAs of narrower sets keep 8: 10.6 against 11.2 ms.)
+    int tmax = std::max(1, std::min(alc_rescore_batch(ctx, key, DT > DBASE || CPT >= 16 ? TMAX_CAP : 8), TMAX_CAP));
     // the largest batch whose vectors fit in shared memory (the batch size
     // changes no result)
     while (tmax > 1 && b32_smem_bytes(a.nmax, a.p, tmax, NPAD) > ctx->smem_optin) tmax--;
-    auto kern = alc_bulk32_kernel<CPT>;
+    auto kern = alc_bulk32_kernel<CPT, DT>;
     const size_t smem = b32_smem_bytes(a.nmax, a.p, tmax, NPAD);
     if (smem > ctx->smem_optin)
         return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_select: shared memory exceeded (n_max, p too large)");
     LAGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
-    LAGP_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, THREADS, smem));
-    int per_sm = alc_ctas_per_sm(ctx, key, b32_min_blocks<CPT>());
+    LAGP_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, FTHREADS + DT, smem));
+    int per_sm = alc_ctas_per_sm(ctx, key, b32_min_blocks<CPT, DT>());
     if (occ > 0 && per_sm > occ) per_sm = occ;
     int64_t grid = (int64_t)ctx->num_sms * std::max(1, per_sm);
     if (grid > a.M) grid = a.M;
@@ -924,20 +950,25 @@ lagp_status launch_b32(lagp_ctx *ctx, const AlcArgs &a) {
     float2 *Yc = reinterpret_cast<float2 *>(ovi + nO);  // 8-byte aligned: nO is a multiple of 128
     LAGP_CUDA(ctx, cudaMemsetAsync(counter, 0, sizeof(int), st));
     B32Params P{a, counter, work, U, C, Clo, Yc, ovs, ovi, ctx->num_sms, tmax, (float)ctx->tuning.rescore_rel};
-    kern<<<(unsigned)grid, THREADS, smem, st>>>(P);
+    kern<<<(unsigned)grid, FTHREADS + DT, smem, st>>>(P);
     ctx->launches++;
     LAGP_CUDA(ctx, cudaGetLastError());
     return LAGP_OK;
+}
+
+template <int DT>
+lagp_status launch_b32_cpt(lagp_ctx *ctx, const AlcArgs &a) {
+    const int need = (a.Npmax + FTHREADS - 1) / FTHREADS;
+    if (need <= 2) return launch_b32<2, DT>(ctx, a);
+    if (need <= 4) return launch_b32<4, DT>(ctx, a);
+    if (need <= 8) return launch_b32<8, DT>(ctx, a);
+    if (need <= 16) return launch_b32<16, DT>(ctx, a);
+    return launch_b32<32, DT>(ctx, a);
 }
 
 }  // namespace
 
 lagp_status launch_alc_f32(lagp_ctx *ctx, const AlcArgs &a) {
     if (a.nmax > 128) return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_select: n_max above 128 is not supported");
-    const int need = (a.Npmax + FTHREADS - 1) / FTHREADS;
-    if (need <= 2) return launch_b32<2>(ctx, a);
-    if (need <= 4) return launch_b32<4>(ctx, a);
-    if (need <= 8) return launch_b32<8>(ctx, a);
-    if (need <= 16) return launch_b32<16>(ctx, a);
-    return launch_b32<32>(ctx, a);
+    return a.M <= ctx->num_sms ? launch_b32_cpt<DWIDE>(ctx, a) : launch_b32_cpt<DBASE>(ctx, a);
 }

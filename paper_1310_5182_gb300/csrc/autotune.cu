@@ -23,11 +23,11 @@ int alc_ctas_per_sm(lagp_ctx *ctx, const std::string &key, int default_cps) {
     return it != ctx->tuned_ctas.end() ? it->second : default_cps;
 }
 
-int alc_rescore_batch(lagp_ctx *ctx, const std::string &key) {
+int alc_rescore_batch(lagp_ctx *ctx, const std::string &key, int default_batch) {
     if (ctx->tune_tmax_override > 0) return ctx->tune_tmax_override;
     if (ctx->tuning.rescore_max > 0) return ctx->tuning.rescore_max;
     auto it = ctx->tuned_tmax.find(key);
-    return it != ctx->tuned_tmax.end() ? it->second : 8;
+    return it != ctx->tuned_tmax.end() ? it->second : default_batch;
 }
 
 extern "C" lagp_status lagp_autotune(lagp_ctx *ctx, const void *X, int64_t N, int32_t p,

@@ -54,8 +54,8 @@ std::string alc_shape_key(const char *kernel, int cpt, int nmax, int p, bool fus
 // user's tuning, the tuned table, or the kernel's default.
 int alc_ctas_per_sm(lagp_ctx *ctx, const std::string &key, int default_cps);
 // The FP32-bulk re-score batch for a shape: the autotuner's candidate, the
-// user's tuning.rescore_max, the tuned choice, or 8.
-int alc_rescore_batch(lagp_ctx *ctx, const std::string &key);
+// user's tuning.rescore_max, the tuned choice, or the default.
+int alc_rescore_batch(lagp_ctx *ctx, const std::string &key, int default_batch = 8);
 
 // The persistent kernels' work counter (offset 0) and the ALC work counters
 // (4 x uint64 at offset 128; the MLE's 2 x uint64 follow at offset 192) of
