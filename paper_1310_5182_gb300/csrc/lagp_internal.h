@@ -132,7 +132,8 @@ struct AlcArgs {
     // FP32-bulk: counts the locations that end LAGP_ENOTPD (device int)
     int *fail_count = nullptr;
     // FP64 Schur retry of those: when set, only locations whose status is
-    // LAGP_ENOTPD are redone, and nothing at all when *retry_count is 0
+    // LAGP_ENOTPD are redone, and nothing at all when *retry_count is 0 (the
+    // plain FP64 form, after its fixed-point kernel: status FX_REDO)
     const int *retry_count = nullptr;
 };
 

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 import workloads as W
-from test_gpu_parity import L, O, check_pred, dev  # noqa: F401  (fixtures)
+from test_gpu_parity import L, O, check_pred, compare_selection, dev  # noqa: F401  (fixtures)
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +103,33 @@ def test_alc_eval_sizes_and_far_candidates(L, O, n, g, d):
     K = np.exp(-((A[:, None] - A[None]) ** 2).sum(-1) / d) + g * np.eye(n)
     atol = 16 * np.finfo(np.float64).eps / g * max(1.0, np.linalg.cond(K) * g)
     assert np.all(np.abs(delta.cpu().numpy() - ds) <= np.maximum(1e-6 * np.abs(ds), atol))
+
+
+@pytest.mark.parametrize("g,d,n_max", [(1e-2, 2.0, 70), (1e-6, 2.0, 40), (1.0, 2.0, 40), (1e-2, 1e-3, 30),
+                                       (1e-3, 0.05, 40), (1e-2, 2.0, 128)])
+def test_plain_search_in_fixed_point(L, O, g, d, n_max):
+    """The plain FP64 form: uneven n (edges of the blocks of rows) and N', the
+    FP64 kernel's share (g = 1; d = 1e-3: no candidate with K(x_c, x) >= 2^-6;
+    n_max = 128: too large for shared memory); many locations and few (two
+    layouts, the same bits)."""
+    n_arr = np.array([6, 7, 8, 9, 12, 15, 16, 17, 23, 24, 25, 30] + [n_max] * 4, np.int32)
+    Np = np.array([n_max, 130, 200, 131] * 4, np.int32)
+    w = W.borehole(seed=34, N=4_000, M=16, n=n_max, Np=200, g=g)
+    idx = O.knn(w.X, w.Xref, 200)
+    idx = np.where(np.arange(200)[None] < Np[:, None], idx, -1).astype(np.int32)
+    ref = O.alc_select(w.X, w.Xref, idx, 6, n_arr, d, g, topk=4, Np=Np)
+    few = L.lagp_alc_predict(dev(w.X), dev(w.Y), dev(w.Xref), dev(idx), 6, n_arr, d, g, prec="f64", Nprime=Np,
+                             n_max=n_max, want_alc=True)
+    sel = few["sel"].cpu().numpy()
+    diverged = compare_selection(sel, ref, n_arr, 6, g)
+    same = [m for m in range(16) if m not in diverged]
+    p = O.predict(w.X, w.Y, w.Xref, sel, n_arr, d, g)
+    check_pred(few["mean"].cpu().numpy()[same], few["s2"].cpu().numpy()[same], {k: v[same] for k, v in p.items()},
+               w.X, w.Y, w.Xref, sel[same], n_arr[same], d, g)
+    rep = 20  # more locations than SMs
+    tile = lambda a: np.ascontiguousarray(np.tile(a, (rep,) + (1,) * (a.ndim - 1)))
+    many = L.lagp_alc_predict(dev(w.X), dev(w.Y), dev(tile(w.Xref)), dev(tile(idx)), 6, tile(n_arr), d, g, prec="f64",
+                              Nprime=tile(Np), n_max=n_max, want_alc=True)
+    for k in ("sel", "alc", "mean", "s2", "status"):
+        assert torch.equal(torch.nan_to_num(many[k][:16]), torch.nan_to_num(few[k])), k
+        assert torch.equal(torch.nan_to_num(many[k][-16:]), torch.nan_to_num(few[k])), k
