@@ -17,6 +17,10 @@ template <>
 struct Vec2<double> {
     using type = double2;
 };
+template <>
+struct Vec2<long long> {
+    using type = longlong2;
+};
 
 // CPT consecutive values of a candidate-indexed row (vector loads/stores)
 template <int CPT, typename T>

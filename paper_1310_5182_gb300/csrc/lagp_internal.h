@@ -131,10 +131,12 @@ struct AlcArgs {
     double *mean, *s2, *df;
     // FP32-bulk: counts the locations that end LAGP_ENOTPD (device int)
     int *fail_count = nullptr;
-    // FP64 Schur retry of those: when set, only locations whose status is
-    // LAGP_ENOTPD are redone, and nothing at all when *retry_count is 0 (the
-    // plain FP64 form, after its fixed-point kernel: status FX_REDO)
+    // second launches: when set, only locations whose status is retry_status
+    // are done, and nothing at all when *retry_count is 0 (the FP64 Schur retry
+    // of the FP32-bulk forms: LAGP_ENOTPD; the FP64 kernels after their
+    // fixed-point ones: FX_REDO)
     const int *retry_count = nullptr;
+    int retry_status = LAGP_ENOTPD;
 };
 
 lagp_status launch_alc_f64(lagp_ctx *ctx, const AlcArgs &a);

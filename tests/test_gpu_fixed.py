@@ -133,3 +133,23 @@ def test_plain_search_in_fixed_point(L, O, g, d, n_max):
     for k in ("sel", "alc", "mean", "s2", "status"):
         assert torch.equal(torch.nan_to_num(many[k][:16]), torch.nan_to_num(few[k])), k
         assert torch.equal(torch.nan_to_num(many[k][-16:]), torch.nan_to_num(few[k])), k
+
+
+@pytest.mark.parametrize("p,dtype,g,d,Np", [(1, np.float64, 1e-2, 0.3, 60), (2, np.float32, 1e-4, 0.5, 255),
+                                            (3, np.float64, 1e-6, 0.05, 257), (8, np.float32, 1e-3, 2.0, 513),
+                                            (20, np.float64, 1e-2, 5.0, 300), (2, np.float64, 1e-2, 1e-7, 100),
+                                            (2, np.float64, 1.0, 0.5, 100)])
+def test_schur_search_in_fixed_point(L, O, p, dtype, g, d, Np):
+    """The FP64 Schur form with its state in fixed point: dimensions, candidate
+    counts at the edges of the slots a thread, a lengthscale too small for the
+    scaled coordinates (redone in FP64) and g = 1 (FP64); duplicated candidates."""
+    rng = np.random.default_rng(35)
+    X = rng.uniform(size=(3_000, p)).astype(dtype)
+    X[1::10] = X[::10]  # exact duplicates
+    Xref = rng.uniform(size=(20, p)).astype(dtype)
+    n_arr = rng.integers(6, 41, 20).astype(np.int32)
+    idx = O.knn(X, Xref, Np)
+    ref = O.alc_select(X, Xref, idx, 6, n_arr, d, g, topk=4)
+    out = L.lagp_alc_select(dev(X), dev(Xref), dev(idx), 6, n_arr, d, g, prec="f64schur", n_max=40, want_alc=True)
+    assert np.array_equal(out["status"].cpu().numpy(), ref["status"])
+    compare_selection(out["sel"].cpu().numpy(), ref, n_arr, 6, g)
