@@ -74,7 +74,8 @@ __host__ __device__ inline int tc_scale_exp(double B) {
 //     |A| |db| + |b| |dA| + |A_l b_l| <= 2^-21 + 2^-21 + 2^-21 (+ 2^-21 slack)
 //   E_tc = S^2 [ 4p 2^-21                                  (cross terms)
 //              + 2 (gamma_p p + 2^-22 p + 2^-25)           (two norms, splits)
-//              + TC_ACC_ULPS (K/16) 2^-24 4p (1 + 2^-9) ]  (accumulation)
+//              + 4p (2^-22 + 2^-23) + 2^-25                (threshold folded into n_q)
+//              + TC_ACC_ULPS (K/16) 2^-24 8p (1 + 2^-9) ]  (accumulation; |n_q - tau2| <= 4p)
 // A row with s <= tau0 then has exact distance r <= sqrt(tau0 + E_tc) + e2
 // (e2 = 2uB sqrt(p)), and every row of the exact top N' has s <= (r_hi +
 // e2)^2 + E_tc.
@@ -83,7 +84,8 @@ __device__ inline double tc_error_bound(int p, int K, double B) {
     const double S = ldexp(1.0, tc_scale_exp(B));
     const double gp = p * u / (1.0 - p * u);
     return S * S * (4.0 * p * 0x1p-21 + 2.0 * (gp * p + 0x1p-22 * p + 0x1p-25) +
-                    TC_ACC_ULPS * (K / 16) * 0x1p-24 * 4.0 * p * (1.0 + 0x1p-9));
+                    4.0 * p * (0x1p-22 + 0x1p-23) + 0x1p-25 +
+                    TC_ACC_ULPS * (K / 16) * 0x1p-24 * 8.0 * p * (1.0 + 0x1p-9));
 }
 
 __device__ inline double tc_margin(float tau, int p, int K, double B) {

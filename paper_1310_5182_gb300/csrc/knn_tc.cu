@@ -34,17 +34,27 @@
 // queries, 34.6 -> 5.7 ms.  In 8 dimensions few blocks fall away (a ball with
 // 2,000 of 4M uniform rows reaches most of the cube): 40.1 -> 38.1 ms.
 //
-// Kernel layout (one CTA per SM, persistent over blocks of up to 128
-// queries): warp 0 streams the design operand into a ring of shared-memory
-// stages with bulk asynchronous copies, warp 1 owns the tensor memory and
-// issues the MMAs (one thread) into four accumulators of 128 columns, and
-// four groups of four epilogue warps (one per TMEM lane quarter; group g
-// takes the design blocks it = g mod 4, accumulator g) read the distances
-// back.  A lane compares its design row's distances with the queries'
-// thresholds into a bit mask, two columns per FP16 x 2 compare (values
-// rounded down, thresholds up: no hit is lost); only the set bits (about
-// 1.5% of the pairs) are visited to append the row to the query's candidate
-// list.
+// Kernel layout (one CTA per SM, persistent over blocks of up to 64 queries):
+// four groups, each of one warp that copies and multiplies and four epilogue
+// warps (one per TMEM lane quarter), take the listed design blocks in turn.
+// The one thread of a copy and MMA warp streams its design blocks into a ring
+// of shared-memory stages with bulk asynchronous copies and issues their MMAs
+// into the group's two accumulators of 64 columns; the epilogue warps read the
+// distances back.  The thresholds are folded into the queries' norm terms
+// (n_q - tau2), so that a row to collect is a negative accumulator: a lane
+// gathers its design row's sign bits, one funnel shift a column, and visits
+// the set bits (0.1 to 10% of the pairs) to append the row to the queries'
+// candidate lists.
+//
+// What bounds it: the epilogue's instructions (a funnel shift a pair and about
+// 80 more for 64 pairs; 70% of the issue slots) and the design operand's reads
+// from the L2 (5.5 TB/s).  With one thread for all copies, one for all MMAs (and
+// 64-bit divisions in both), every design block waited for them in turn, 490 ns
+// whatever its width; four such threads that also copy for themselves, 25.7 ->
+// 23.8 ms (4M rows, 25,000 queries, p = 8, N' = 2,000); accumulators of 64
+// columns, one TMEM load for all of them, and hits appended by the lane that
+// found them, no queue, 23.8 -> 18.3 ms.  Before all of it 38.1 ms; 500,000 rows
+// in 3 dimensions, 201,600 queries, N' = 1,500: 5.7 -> 3.6 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -59,36 +69,21 @@
 namespace {
 
 constexpr int TC_EPI_GROUPS = 4;  // epilogue groups of four warps (one per TMEM lane quarter)
-constexpr int TC_THREADS = 64 + 128 * TC_EPI_GROUPS;  // warp 0: copies, warp 1: TMEM + MMA, then the epilogue
+constexpr int TC_EPI_WARP = TC_EPI_GROUPS;  // a copy and MMA warp a group, then the epilogue
+constexpr int TC_THREADS = 32 * (TC_EPI_WARP + 4 * TC_EPI_GROUPS);
 constexpr int TC_MROWS = 128;    // design rows per MMA (M)
-constexpr int TC_STAGES_MAX = 8; // design stages in flight (fewer for wide rows)
-constexpr int TC_NACC = 4;       // TMEM accumulators (128 columns each)
-constexpr int TC_ACC_COLS = 128;
+constexpr int TC_STAGES_MAX = 4; // design stages a group (3 for wide rows)
+constexpr int TC_NACC = 2 * TC_EPI_GROUPS;  // TMEM accumulators: two a group
+constexpr int TC_ACC_COLS = 64;
 constexpr int TC_TMEM_COLS = TC_NACC * TC_ACC_COLS;  // 512: the whole tensor memory of the SM
-constexpr int TC_QMAX = 128;     // queries per block (MMA N <= 128)
-constexpr int TC_CHUNK = 16384;  // design blocks whose survivors are listed at a time
-constexpr int TC_QUE = 32 * (TC_QMAX / 16);  // hit-queue entries of an epilogue warp: one a lane and chunk
+constexpr int TC_QMAX = TC_ACC_COLS;  // queries per block (MMA N <= 64)
+constexpr int TC_CHUNK = 8192;  // design blocks whose survivors are listed at a time
 
 // Half offset of element k of operand row r in the no-swizzle K-major
 // layout: 8-row groups of K / 8 core matrices (8 rows x 8 halves, 128 bytes),
 // the core matrices of a group adjacent along K.
 __device__ __forceinline__ int64_t tc_off(int64_t r, int k, int K) {
     return (r >> 3) * (8 * (int64_t)K) + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
-}
-
-// Two FP32 values as FP16 x 2, rounded toward zero with negatives clamped to
-// zero (never above the value they stand for, for a value >= 0; NaN stays
-// NaN): x in the low half, y in the high half.
-__device__ __forceinline__ uint32_t f16x2_rz_relu(float x, float y) {
-    uint32_t r;
-    asm("cvt.rz.relu.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
-    return r;
-}
-// per half: 0xFFFF when a <= b, else 0 (NaN: 0)
-__device__ __forceinline__ uint32_t le_mask_h2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("set.le.u32.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
 }
 
 // v = h + l with h, l FP16 (round to nearest): |v - h - l| <= max(2^-22 |v|, 2^-25)
@@ -148,6 +143,10 @@ __global__ void knn_tc_prep(const void *__restrict__ X, int64_t N, int64_t Npad,
                 row[p + i] = des ? vh : vl;
                 row[2 * p + i] = des ? vl : vh;
             }
+            if (!(n2 < CUDART_INF_F)) {  // a NaN or infinite coordinate: an infinite distance, not a NaN of some sign
+                for (int i = 0; i < 3 * p; i++) row[i] = zero;
+                nh = __ushort_as_half(0x7c00), nl = zero;
+            }
             row[3 * p] = des ? one : nh;
             row[3 * p + 1] = des ? one : nl;
             row[3 * p + 2] = des ? nh : one;
@@ -180,7 +179,7 @@ struct TcArgs {
     int32_t *cand, Cmax;
     int32_t *cand_count, *status, *retry;
     int nq, nblocks;  // queries per block, blocks
-    int stages;       // shared-memory stages of the design ring
+    int stages;       // shared-memory stages of a group's design ring
     float *dump;      // diagnostic: every value s (M x N) instead of the collection
     int stall;        // test hook: the producer stops after the first design block
     int *err;         // raised when a bounded wait gave up (the block's queries go to the retry)
@@ -190,30 +189,26 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int K = a.K, S = a.stages;
     const int stage_halves = TC_MROWS * K;
-    __half *sA = reinterpret_cast<__half *>(smem_raw);         // S stages x 128 rows
-    __half *sQ = sA + (size_t)S * stage_halves;                // TC_QMAX rows
+    __half *sA = reinterpret_cast<__half *>(smem_raw);         // S stages a group x 128 rows
+    __half *sQ = sA + (size_t)TC_EPI_GROUPS * S * stage_halves;                // TC_QMAX rows
     float *s_tau2 = reinterpret_cast<float *>(sQ + (size_t)TC_QMAX * K);  // TC_QMAX
-    uint32_t *s_t2h = reinterpret_cast<uint32_t *>(s_tau2 + TC_QMAX);  // TC_QMAX/2: FP16 x 2, rounded up
-    int *s_cnt = reinterpret_cast<int *>(s_t2h + TC_QMAX / 2);       // TC_QMAX
-    uint2 *s_que = reinterpret_cast<uint2 *>(s_cnt + TC_QMAX);  // per epilogue warp: TC_QUE entries
-    uint16_t *s_list = reinterpret_cast<uint16_t *>(s_que + TC_QUE * 4 * TC_EPI_GROUPS);  // TC_CHUNK design blocks
+    int *s_cnt = reinterpret_cast<int *>(s_tau2 + TC_QMAX);    // TC_QMAX
+    uint16_t *s_list = reinterpret_cast<uint16_t *>(s_cnt + TC_QMAX);  // TC_CHUNK design blocks
     uint64_t *bar = reinterpret_cast<uint64_t *>(s_list + TC_CHUNK);
-    uint64_t *full = bar, *empty = bar + S, *tfull = bar + 2 * S, *tempty = bar + 2 * S + TC_NACC;
+    uint64_t *full = bar, *tfull = bar + TC_EPI_GROUPS * S, *tempty = tfull + TC_NACC;
     __shared__ uint32_t s_tmem;
     __shared__ int s_err, s_blk, s_nlist;
     __shared__ int32_t s_q[TC_QMAX];  // the block's locations
+    __shared__ int32_t *s_cand[TC_QMAX];  // and their candidate lists
     __shared__ double s_c[64], s_B;
     __shared__ uint32_t s_qlo[20], s_qhi[20], s_tmax;  // order-preserving keys of floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
-        for (int s = 0; s < S; s++) {
-            mbar_init(full + s, 1);
-            mbar_init(empty + s, 1);
-        }
+        for (int s = 0; s < TC_EPI_GROUPS * S; s++) mbar_init(full + s, 1);
         for (int c = 0; c < TC_NACC; c++) {
             mbar_init(tfull + c, 1);
-            mbar_init(tempty + c, 4);  // the four warps of the group that reads it (group c)
+            mbar_init(tempty + c, 4);  // the four warps of the group that reads it (group c / 2)
         }
         mbar_init_fence();
         s_err = 0;
@@ -234,7 +229,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
     // the operands carry 2^-e, the accumulators 2^-2e
     const float s2 = ldexpf(1.f, -2 * tc_scale_exp(s_B));
 
-    long long it0 = 0;  // design blocks processed by this CTA so far (ring positions)
+    // the warp's group (copies and MMAs: warp g; epilogue: four warps), and the
+    // design blocks that it has seen, modulo 2^32 (its position in its ring)
+    const int g = warp < TC_EPI_WARP ? warp : (warp - TC_EPI_WARP) >> 2;
+    uint32_t round0 = 0;
+    int ld_slot = 0, mma_slot = 0;  // the copying thread's: ring positions, and the phase of the copies awaited
+    uint32_t mma_phase = 0;
     for (;;) {
         if (tid == 0) s_blk = atomicAdd(a.counter, 1);
         if (tid < 20) s_qlo[tid] = 0xFFFFFFFFu, s_qhi[tid] = 0u;
@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
             s_tau2[c] = t2 * s2;  // an exact scaling
             s_cnt[c] = 0;
             s_q[c] = c < nqb ? (int32_t)(a.order.query ? a.order.query[q0 + c] : q0 + c) : 0;
+            s_cand[c] = a.cand + s_q[c] * (int64_t)a.Cmax;
             if (a.order.box && t2 == t2) atomicMax(&s_tmax, fkey(t2));
         }
         // the bounding box of the block's queries
@@ -280,13 +281,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
                 }
             }
         __syncthreads();
-        // the thresholds in FP16, rounded up (so that a value below a threshold
-        // stays below it after both roundings), two a word
-        for (int c2 = tid; c2 < TC_QMAX / 2; c2 += TC_THREADS) {
-            const float ta = s_tau2[2 * c2], tb = s_tau2[2 * c2 + 1];
-            const __half ha = __float2half_ru(ta), hb = __float2half_ru(tb);
-            s_t2h[c2] = (uint32_t)__half_as_ushort(ha) | ((uint32_t)__half_as_ushort(hb) << 16);
-        }
+        // the thresholds folded into the queries' norms, n_q - tau2, so that an
+        // accumulator is negative exactly for a row to collect (a query that
+        // is not screened: infinite, never negative)
+        if (!a.dump)
+            for (int c = tid; c < nqb; c += TC_THREADS) {
+                __half *nh = sQ + tc_off(c, 3 * a.p, K), *nl = sQ + tc_off(c, 3 * a.p + 1, K);
+                const float t2 = s_tau2[c];
+                __half h = __ushort_as_half(0x7c00), l = __float2half_rn(0.f);
+                if (t2 == t2) f16_split((__half2float(*nh) + __half2float(*nl)) - t2 * (1.f + 0x1p-20f), h, l);
+                *nh = h;
+                *nl = l;
+            }
         fence_proxy_async_smem();
         // Design blocks that may hold a row to collect, a chunk at a time: with
         // boxes, those whose box lies within the largest threshold of the
@@ -318,142 +324,106 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
         }
         __syncthreads();
         const int nlist = s_nlist;
+        const int cnt = (nlist - g + TC_EPI_GROUPS - 1) / TC_EPI_GROUPS;  // the group's: g, g + 4, ...
 
-        if (warp == 0) {
-            if (lane == 0) {  // producer: design blocks into the stage ring
-                int issued = 0;
-                for (int li = 0; li < nlist && !*err; li++) {
-                    if (a.stall && li == 1) break;  // the MMA's wait on this block then runs out
-                    const long long it = it0 + li;
-                    const int mb = chunk + s_list[li];
-                    const int s = (int)(it % S);
-                    const uint32_t round = (uint32_t)(it / S);
-                    if (!mbar_wait(empty + s, (round & 1u) ^ 1u, err, 128)) break;
-                    mbar_arrive_expect_tx(full + s, stage_bytes);
-                    bulk_g2s(sA + (size_t)s * stage_halves, a.A + (size_t)mb * stage_halves, stage_bytes, full + s);
-                    issued = li + 1;
-                }
-                if (*err && issued > 0) {  // let the copies in flight land before the CTA moves on
-                    for (int li = max(0, issued - S); li < issued; li++) {
-                        const long long it = it0 + li;
-                        int quiet = 0;
-                        mbar_wait(full + (int)(it % S), (uint32_t)(it / S) & 1u, &quiet);
-                    }
-                }
-            }
-        } else if (warp == 1) {
-            if (lane == 0) {  // MMA issuer
+        if (warp < TC_EPI_WARP) {
+            if (lane == 0) {  // one thread: the group's copies and MMAs
                 const uint32_t idesc = idesc_f16_f32(TC_MROWS, nmma);
-                const uint32_t qaddr = smem_u32(sQ);
-                long long last = -1;
-                for (int li = 0; li < nlist && !*err; li++) {
-                    const long long it = it0 + li;
-                    const int s = (int)(it % S);
-                    const int ac = (int)(it % TC_NACC);
-                    if (!mbar_wait(full + s, (uint32_t)(it / S) & 1u, err, 32)) break;
-                    if (!mbar_wait(tempty + ac, ((uint32_t)(it / TC_NACC) & 1u) ^ 1u, err, 32)) break;
+                const uint64_t qdesc = smem_desc_kmajor(smem_u32(sQ), 128u, sbo);
+                __half *ring = sA + (size_t)g * S * stage_halves;
+                const uint64_t adesc = smem_desc_kmajor(smem_u32(ring), 128u, sbo);
+                uint64_t *const gfull = full + g * S;
+                int loaded = 0, landed = 0, issued = 0;
+                auto load = [&]() {  // the next design block into the ring
+                    const int li = g + loaded * TC_EPI_GROUPS;
+                    if (loaded >= cnt || (a.stall && li >= 1)) return;  // (stall: the wait on it then runs out)
+                    mbar_arrive_expect_tx(gfull + ld_slot, stage_bytes);
+                    bulk_g2s(ring + (size_t)ld_slot * stage_halves, a.A + (size_t)(chunk + s_list[li]) * stage_halves,
+                             stage_bytes, gfull + ld_slot);
+                    loaded++;
+                    if (++ld_slot == S) ld_slot = 0;
+                };
+                auto land = [&](volatile int *e) {  // waits for the next copy
+                    if (!mbar_wait(gfull + mma_slot, mma_phase, e, 32)) return false;
+                    landed++;
+                    return true;
+                };
+                auto next = [&]() {
+                    if (++mma_slot == S) mma_slot = 0, mma_phase ^= 1u;
+                };
+                for (int k = 0; k < S; k++) load();
+                for (int k = 0; k < cnt; k++) {
+                    const uint32_t round = round0 + (uint32_t)k, ac = (uint32_t)g * 2u + (round & 1u);
+                    if (!mbar_wait(tempty + ac, ((round >> 1) & 1u) ^ 1u, err, 32)) break;
+                    // the accumulator was read, so the block two before this one
+                    // is through its MMAs: its stage takes the next copy
+                    if (k > 1) load();
+                    if (!land(err)) break;
                     tc_fence_after_sync();
-                    const uint32_t aaddr = smem_u32(sA + (size_t)s * stage_halves);
+                    // (descriptors address shared memory in 16-byte units)
+                    const uint64_t ad = adesc + ((uint32_t)mma_slot * stage_bytes >> 4);
                     for (int ks = 0; ks < K / 16; ks++)  // 16 halves (two core matrices) per MMA
-                        mma_f16(tmem + (uint32_t)(ac * TC_ACC_COLS), smem_desc_kmajor(aaddr + ks * 256u, 128u, sbo),
-                                smem_desc_kmajor(qaddr + ks * 256u, 128u, sbo), idesc, ks > 0 ? 1u : 0u);
-                    mma_commit(empty + s);    // the stage may be overwritten once these MMAs are done
-                    mma_commit(tfull + ac);   // the accumulator is ready
-                    last = it;
+                        mma_f16(tmem + ac * TC_ACC_COLS, ad + 16u * ks, qdesc + 16u * ks, idesc, ks > 0 ? 1u : 0u);
+                    mma_commit(tfull + ac);  // the accumulator is ready
+                    issued = k + 1;
+                    next();
                 }
-                if (*err && last >= 0) {  // the MMAs issued finish before the TMEM is released
+                if (*err) {  // the copies in flight land and the MMAs issued finish before the CTA moves on
                     int quiet = 0;
-                    mbar_wait(tfull + (int)(last % TC_NACC), (uint32_t)(last / TC_NACC) & 1u, &quiet);
+                    if (landed > issued) next();
+                    for (; landed < loaded; next())
+                        if (!land(&quiet)) break;
+                    if (issued) {
+                        const uint32_t round = round0 + (uint32_t)issued - 1u;
+                        mbar_wait(tfull + g * 2 + (round & 1u), (round >> 1) & 1u, &quiet);
+                    }
                 }
             }
         } else {
-            // epilogue: group g reads accumulator g, of the design blocks with
-            // it = g (mod 4); each warp its TMEM lane quarter (32 design rows)
-            const int g = (warp - 2) >> 2, quarter = warp & 3;
-            uint2 *que = s_que + (size_t)(warp - 2) * TC_QUE;
-            const uint32_t lt_mask = (1u << lane) - 1u;
-            for (int li = 0; li < nlist; li++) {
-                const long long it = it0 + li;
-                if ((int)(it % TC_NACC) != g) continue;
+            // epilogue: group g reads accumulators 2g and 2g + 1 in turn, of the listed
+            // design blocks g, g + 4, ...; each warp its TMEM lane quarter (32 design rows)
+            const int quarter = warp & 3;
+            // the columns that are queries, the first one's bit on top
+            const unsigned long long cols = nqb < 64 ? ~(~0ull >> nqb) : ~0ull;
+            for (int k = 0; k < cnt; k++) {
+                const uint32_t round = round0 + (uint32_t)k, ac = (uint32_t)g * 2u + (round & 1u);
+                const int li = g + k * TC_EPI_GROUPS;
                 const int mb = chunk + s_list[li];
                 // every lane waits; the warp goes on only together (the TMEM
                 // loads are warp-collective)
-                const bool ready = mbar_wait(tfull + g, (uint32_t)(it / TC_NACC) & 1u, err, 64);
+                const bool ready = mbar_wait(tfull + ac, (round >> 1) & 1u, err, 64);
                 if (!__all_sync(LAGP_FULL_MASK, ready)) break;
                 tc_fence_after_sync();
                 const int64_t row = (int64_t)mb * TC_MROWS + quarter * 32 + lane;
-                const bool live = row < a.N;
-                int qn = 0;  // hit-queue entries of this design block
-                const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * TC_ACC_COLS);
-                for (int cb = 0; cb < nmma; cb += 64) {
-                    // up to four chunks of 16 columns in flight, one wait
-                    uint32_t v[4][16];
-#pragma unroll
-                    for (int h = 0; h < 4; h++)
-                        if (cb + 16 * h < nmma) tmem_ld16(taddr + (uint32_t)(cb + 16 * h), v[h]);
-#pragma unroll
-                    for (int h = 0; h < 4; h++)
-                        if (cb + 16 * h < nmma) tmem_wait_ld16(v[h]);
-                    if (cb + 64 >= nmma) {  // every column read: release the accumulator
-                        tc_fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(tempty + g);
-                    }
-#pragma unroll
-                    for (int h = 0; h < 4; h++) {
-                        const int c0 = cb + 16 * h;
-                        if (c0 >= nmma) break;
-                        if (a.dump) {
-                            if (live)
-#pragma unroll
-                                for (int i = 0; i < 16; i++)
-                                    if (c0 + i < nqb)
-                                        a.dump[(q0 + c0 + i) * a.N + row] = __uint_as_float(v[h][i]) / s2;
-                            continue;
-                        }
-                        // hit mask, compared two columns a time in FP16 (values
-                        // rounded down, thresholds up: no hit is lost; the
-                        // rounding admits at most a few extra rows): column
-                        // c0 + 2i sets bit i, column c0 + 2i + 1 bit 16 + i
-                        const uint4 *t4 = reinterpret_cast<const uint4 *>(s_t2h + c0 / 2);
-                        uint32_t m2 = 0;
-#pragma unroll
-                        for (int i4 = 0; i4 < 2; i4++) {
-                            const uint4 t = t4[i4];
-                            const uint32_t tt[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-                            for (int q2 = 0; q2 < 4; q2++) {
-                                const int i = 4 * i4 + q2;  // the pair of columns c0 + 2i, c0 + 2i + 1
-                                const uint32_t hv = f16x2_rz_relu(__uint_as_float(v[h][2 * i]), __uint_as_float(v[h][2 * i + 1]));
-                                m2 |= le_mask_h2(hv, tt[q2]) & (0x00010001u << i);
-                            }
-                        }
-                        if (!live) m2 = 0u;
-                        // a lane with hits queues (chunk and lane, mask); the
-                        // queue is drained lane-parallel after the block
-                        const uint32_t b = __ballot_sync(LAGP_FULL_MASK, m2 != 0u);
-                        if (m2) que[qn + __popc(b & lt_mask)] = make_uint2(((uint32_t)(c0 >> 4) << 5) | (uint32_t)lane, m2);
-                        qn += __popc(b);
-                    }
-                }
+                uint32_t v[64];
+                tmem_ld64(tmem + ((uint32_t)(quarter * 32) << 16) + ac * TC_ACC_COLS, v);
+                tmem_wait_ld64(v);
+                tc_fence_before_sync();
                 __syncwarp();
-                for (int e = lane; e < qn; e += 32) {
-                    const uint2 w = que[e];
-                    const int cb0 = (int)(w.x >> 5) * 16;
-                    const int32_t hrow = (int32_t)(mb * TC_MROWS + quarter * 32 + (w.x & 31u));
-                    uint32_t mm = w.y;  // bit i: column cb0 + 2i; bit 16 + i: column cb0 + 2i + 1
-                    while (mm) {
-                        const int bit = __ffs(mm) - 1;
-                        const int c = cb0 + (bit < 16 ? 2 * bit : 2 * (bit - 16) + 1);
-                        mm &= mm - 1u;
-                        const int pos = atomicAdd(&s_cnt[c], 1);
-                        if (pos < a.Cmax) a.cand[s_q[c] * (int64_t)a.Cmax + pos] = hrow;
-                    }
+                if (lane == 0) mbar_arrive(tempty + ac);  // every column read: release the accumulator
+                if (a.dump) {
+#pragma unroll
+                    for (int c = 0; c < 64; c++)
+                        if (c < nqb && row < a.N) a.dump[(q0 + c) * a.N + row] = __uint_as_float(v[c]) / s2;
+                    __syncwarp();
+                    continue;
+                }
+                uint32_t m0 = 0, m1 = 0;  // the sign bits, the first column's on top
+#pragma unroll
+                for (int i = 0; i < 32; i++) {
+                    m0 = __funnelshift_l(v[i], m0, 1);
+                    m1 = __funnelshift_l(v[32 + i], m1, 1);
+                }
+                for (unsigned long long m = row < a.N ? ((unsigned long long)m0 << 32 | m1) & cols : 0ull; m;) {
+                    const int c = __clzll((long long)m);
+                    m &= ~(0x8000000000000000ull >> c);
+                    const int pos = atomicAdd(&s_cnt[c], 1);
+                    if (pos < a.Cmax) s_cand[c][pos] = (int32_t)row;
                 }
                 __syncwarp();
             }
         }
-        it0 += nlist;
+        round0 += (uint32_t)cnt;
         }
         __syncthreads();
         // per-query results: the collected rows and the threshold they were
@@ -575,16 +545,17 @@ lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, con
     const int64_t nb = std::min<int64_t>(M, round_up(nb_min, sms));
     a.nq = (int)((M + nb - 1) / nb);
     a.nblocks = (int)((M + a.nq - 1) / a.nq);
-    // as many stages as fit (at most TC_STAGES_MAX): the CTA then has the SM
-    // (and its tensor memory) to itself
-    const size_t fixed = (size_t)TC_QMAX * K * 2 + (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS + TC_CHUNK / 2) * 4 +
-                         (2 * TC_STAGES_MAX + 2 * TC_NACC) * 8 + 1024;
+    // as many stages as fit: the CTA then has the SM (and its tensor memory)
+    // to itself
+    const size_t fixed = (size_t)TC_QMAX * K * 2 + (2 * TC_QMAX + TC_CHUNK / 2) * 4;
     const size_t stage_bytes = (size_t)TC_MROWS * K * 2;
-    a.stages = (int)std::min<size_t>(TC_STAGES_MAX, (ctx->smem_optin - fixed) / stage_bytes);
-    if (a.stages < 2) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: tensor-core screen exceeds shared memory");
-    size_t smem = (size_t)a.stages * stage_bytes + (size_t)TC_QMAX * K * 2 +
-                  (2 * TC_QMAX + TC_QMAX / 2 + 2 * TC_QUE * 4 * TC_EPI_GROUPS + TC_CHUNK / 2) * 4 +
-                  (2 * (size_t)a.stages + 2 * TC_NACC) * 8;
+    auto smem_of = [&](int stages) {
+        return fixed + TC_EPI_GROUPS * stages * stage_bytes + (TC_EPI_GROUPS * (size_t)stages + 2 * TC_NACC) * 8;
+    };
+    a.stages = TC_STAGES_MAX;
+    while (a.stages > 2 && smem_of(a.stages) + 4096 > ctx->smem_optin) a.stages--;
+    size_t smem = smem_of(a.stages);
+    if (smem + 4096 > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: tensor-core screen exceeds shared memory");
     // more than half of the SM's shared memory: one CTA per SM, which then
     // holds the whole tensor memory
     smem = std::max(smem, ctx->smem_optin / 2 + 4096);
