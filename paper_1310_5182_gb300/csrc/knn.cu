@@ -7,6 +7,8 @@
 //               reference locations (the centre c and half-width B).
 //   knn_prep    centred FP32 copy of the design, y = fl32(x - c), with the
 //               FP32 squared norm |y|^2 as an extra column.
+//   knn_sample  with the tensor-core collection: the sampled thresholds alone
+//               (its passes A and B by a bound from part of the sample).
 //   knn_screen  persistent; 16 queries per CTA, two per warp, sharing every
 //               design tile in shared memory.  The main launch evaluates
 //               |y_x|^2 + |y_q|^2 - 2 y_x . y_q (one add and p FMAs a pair);
@@ -40,6 +42,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <numeric>
 #include <vector>
 
 #include "device_util.cuh"
@@ -55,6 +58,8 @@ constexpr int HB = 1024;              // histogram bins per level (10 bits)
 constexpr int L1_SHIFT = 21;          // level 1: FP32 distance bits [30:21]
 constexpr int L2_SHIFT = 11;          // level 2: bits [20:11] inside the boundary bin
 constexpr uint32_t L2_LOW = (1u << L2_SHIFT) - 1;
+constexpr int SAMPLE_DEPTH = 16;       // sampled distances that a thread lists below the first sweep's bound
+constexpr int SAMPLE_TILE_FLOATS = 5120;
 constexpr int TILE_FLOATS = 4096;     // floats of one design tile (tile length x row stride)
 
 // Floats per centred row: p coordinates and the squared norm, padded to an
@@ -69,6 +74,12 @@ __host__ __device__ inline int tile_len(int ps) {
     return t > 512 ? 512 : (t < 32 ? 32 : t);
 }
 
+
+// Rows of a tile of the sampling sweep: a multiple of 64, at most 1,024.
+__host__ __device__ inline int sample_tile(int ps) {
+    int t = (SAMPLE_TILE_FLOATS / ps) & ~63;
+    return t > 1024 ? 1024 : (t < 64 ? 64 : t);
+}
 
 // 16-byte asynchronous global-to-shared copy (bypassing L1), and its fences
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -167,14 +178,18 @@ __device__ __forceinline__ void centred_row(const void *X, int64_t N, int64_t r,
 // serialise the threads that wait for the margin).
 __device__ __forceinline__ double pow_bound(double u, double n) { return 1.0 / (1.0 - ceil(n) * u); }
 
-// In the order of perm (null: as given).  Y: all rows (Npad of them), Ys: positions 0, s, 2s, ... (nsamp_pad of them;
-// null when s = 1, where the sample is the whole design), Yv: the
+// In the order of perm (null: as given).  Y: all rows (Npad of them), Ys: the
+// nsamp positions 0, s, 2s, ... (null when s = 1, where the sample is the whole
+// design; padded with zero rows to nsamp_pad), stepping through them by `spread`
+// positions (prime to nsamp, near the golden section), so that its first rows
+// are themselves an even sample, Yv: the
 // coordinates of Y with a row stride of p rounded up to 4; kc: the launch's
 // constants (block 0).
 __global__ void knn_prep(const void *__restrict__ X, int64_t N, int p, lagp_dtype dt,
                          const unsigned long long *kmax, const unsigned long long *kmin,
                          const int32_t *__restrict__ perm, float *__restrict__ Y, int64_t Npad,
-                         float *__restrict__ Ys, int64_t nsamp_pad, int64_t sstride, KnnConst *kc,
+                         float *__restrict__ Ys, int64_t nsamp, int64_t nsamp_pad, int64_t sstride, int64_t spread,
+                         KnnConst *kc,
                          float *__restrict__ Yv) {
     __shared__ double c[64];
     __shared__ double sB;
@@ -200,7 +215,7 @@ __global__ void knn_prep(const void *__restrict__ X, int64_t N, int p, lagp_dtyp
     }
     if (Ys)
         for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nsamp_pad; r += stride)
-            centred_row(X, N, r * sstride, perm, p, ps, dt, c, Ys + r * ps);
+            centred_row(X, N, r < nsamp ? r * spread % nsamp * sstride : N, perm, p, ps, dt, c, Ys + r * ps);
 }
 
 // ------------------------------------------------------------ spatial order
@@ -393,6 +408,14 @@ __device__ void find_bin(const uint32_t *h, uint32_t target, int lane, uint32_t 
     }
 }
 
+// Rank, in a sample of every stride-th row (nsamp of them), of the threshold
+// for k rows: 1.3 k / stride + 16, exactly k when the sample is the design.
+__host__ __device__ inline int sample_rank(int k, int64_t stride, int64_t nsamp) {
+    if (stride == 1) return k;
+    const int64_t rt = (13 * (int64_t)k + 10 * stride - 1) / (10 * stride) + 16;
+    return (int)(rt < nsamp ? rt : nsamp);
+}
+
 // One design tile against a warp's QPW queries, rows r0, r0 + rstep, ... of
 // the tile.  PASS 0: level-1 histogram; PASS 1: level-2 histogram inside the
 // boundary bin; PASS 2: collection.
@@ -489,7 +512,7 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
            const unsigned long long *__restrict__ kmax, const unsigned long long *__restrict__ kmin,
            int32_t *__restrict__ cand, int32_t Cmax, int32_t *__restrict__ cand_count,
            int32_t *__restrict__ status, int64_t stride, int32_t *__restrict__ retry, int retry_pass,
-           int *__restrict__ counter, float *__restrict__ tau_out) {
+           int *__restrict__ counter) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int pp = row_stride(p);              // floats per centred row (coordinates, norm, pad)
     const int TT = tile_len(pp);               // rows per tile
@@ -530,7 +553,7 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
             if (retry_pass) ok[h] = ok[h] && retry[q[h]] != 0;  // exact retry: flagged queries only
             mine_any |= ok[h];
             rtarget[h] = stride == 1 ? k[h]
-                                     : (int)min((int64_t)((13 * (int64_t)k[h] + 10 * stride - 1) / (10 * stride)) + 16, nsamp);
+                                     : sample_rank(k[h], stride, nsamp);
             if (lane == 0) {
                 float n2 = 0.f;
                 for (int i = 0; i < p; i++) {
@@ -614,10 +637,7 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
         // exactly when s <= t rounded down to a float, so the hot loop compares
         // in FP32 (an FP64 compare per point would occupy the slow FP64 unit)
         float tau0[QPW] = {}, tau2f[QPW] = {};
-        // with tau_out, passes A and B only: the sampled threshold tau0 of
-        // every query (NaN for one that is not screened) for the collection
-        // pass on the tensor cores
-        const int npass = !any_ok ? 0 : (tau_out ? 2 : 3);
+        const int npass = any_ok ? 3 : 0;
         for (int pass = 0; pass < npass; pass++) {
             // passes A, B: the sampled rows (contiguous in Ys); C: all rows
             const float *src = pass < 2 ? Ys : Y32;
@@ -684,12 +704,6 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
             }
             __syncthreads();
         }
-        if (tau_out) {
-#pragma unroll
-            for (int h = 0; h < QPW; h++)
-                if (active[h] && lane == 0) tau_out[q[h]] = ok[h] ? tau0[h] : CUDART_NAN_F;
-            continue;
-        }
 #pragma unroll
         for (int h = 0; h < QPW; h++) {
             if (!active[h] || lane != 0) continue;
@@ -708,6 +722,263 @@ knn_screen(const float *__restrict__ Y32, const float *__restrict__ Ys, int64_t 
                 if (status) status[q[h]] = c0 < k[h] ? LAGP_EINVAL : (c > Cmax ? LAGP_ENOMEM : LAGP_OK);
             }
         }
+        __syncthreads();
+    }
+}
+
+// Sampled thresholds of the tensor-core collection: per query the rank-th
+// smallest distance (norm expansion) to the sampled rows, rounded up to the
+// end of its 2^-12-wide bin (bits [30:11]); NaN for a query that is not
+// screened.  Eight warps share nq = 8 QW / W queries: groups of W warps, QW
+// queries a warp, the group's warps splitting every tile's rows.
+//   First sweep (nsub > 0): the first nsub rows of Ys (an even subset: the
+//   order spreads them), histogram of bits [30:19].  The bin's end U at the
+//   wanted rank bounds the threshold of all rows from above, whatever the
+//   subset.
+//   Second sweep: all rows; the values up to U (a few hundred) are listed, and the wanted rank selected from the list.
+//   Without a first sweep (a rank too large for the list: small designs), or
+//   when a list overflows, two histogram sweeps over all rows instead, bits
+//   [30:21], then [20:11] inside the boundary bin.
+// What bounds it: the second sweep's instructions, about half of the issue
+// slots, the rest latency and the barrier a tile (four smaller tiles in flight:
+// 15% slower; lists shared through an atomic or a ballot: 10 to 50% slower).
+// Two histogram sweeps with two queries a warp (an atomic a pair, most of a
+// warp's lanes in the same few bins) took 4.1 -> 2.2 ms (62,500 sampled rows,
+// p = 8, 25,000 queries), 4.9 -> 3.1 ms (12,196 rows, p = 3, 201,600 queries) and
+// 93 -> 25 us (10,000 rows, p = 2, 100 queries: sixteen a CTA met 7 SMs).
+template <int P, int QW, int W>
+__global__ void __launch_bounds__(SCREEN_THREADS, 2)
+knn_sample(const float *__restrict__ Ys, int64_t nsamp, int64_t nsub, int p, const void *__restrict__ Xref,
+           lagp_dtype dt, int64_t M, const int32_t *__restrict__ Np, int32_t Npmax, int64_t stride,
+           const unsigned long long *__restrict__ kmax, const unsigned long long *__restrict__ kmin,
+           int *__restrict__ counter, float *__restrict__ tau_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int pp = row_stride(p), TT = sample_tile(pp), np = P > 0 ? P : p, PS = P > 0 ? ((P + 1) | 1) : pp;
+    constexpr int nq = 8 * QW / W;
+    constexpr int COLS = 32 * W, SLOT = SAMPLE_DEPTH * COLS;  // a query's list: SAMPLE_DEPTH values a thread of its group
+    static_assert(SLOT >= HB, "a query's histogram fits its list's place");
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw);   // nq x SLOT: histograms (HB words), or lists
+    float *tiles = reinterpret_cast<float *>(hist + nq * SLOT);  // 2 x TT x pp, 16-byte aligned
+    float *qs = tiles + 2 * (size_t)TT * pp;                   // nq x pp: centred queries
+    __shared__ int32_t s_rt[nq];
+    __shared__ float s_U[nq], s_tau[nq];
+    __shared__ uint8_t s_n[nq * COLS];  // list lengths
+    __shared__ int64_t s_blk;
+    __shared__ double s_c[64], s_B;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q0 = w / W * QW, sub = w % W;  // the warp's first query slot, its share of the rows
+    if (threadIdx.x == 0) centre_and_bound(kmax, kmin, p, s_c, s_B);
+    __syncthreads();
+    // first sweep's bins: 16 an octave, 64 octaves down from above the largest distance
+    const int cbase = (int)(__float_as_uint((float)(4.0 * p * s_B * s_B * 1.01)) >> 19) - (HB - 1);
+
+    for (;;) {
+        if (threadIdx.x == 0) s_blk = atomicAdd(counter, 1);
+        __syncthreads();
+        const int64_t blk = s_blk;
+        if (blk * nq >= M) break;
+        for (int ql = threadIdx.x; ql < nq; ql += SCREEN_THREADS) {
+            const int64_t q = blk * nq + ql;
+            const int k = q < M ? (Np ? Np[q] : Npmax) : 0;
+            s_rt[ql] = k >= 1 && k <= Npmax ? sample_rank(k, stride, nsamp) : 0;  // 0: not screened
+            s_tau[ql] = CUDART_NAN_F;
+            float n2 = 0.f;
+            for (int i = 0; i < p; i++) {
+                const float y = q < M ? (float)(load_coord64(Xref, q, p, i, dt) - s_c[i]) : 0.f;
+                qs[ql * pp + i] = y;
+                n2 = fmaf(y, y, n2);
+            }
+            qs[ql * pp + p] = n2;
+        }
+        auto clear = [&]() {
+            for (int b = threadIdx.x; b < nq * HB; b += SCREEN_THREADS) hist[b / HB * SLOT + b % HB] = 0;
+            __syncthreads();
+        };
+        clear();
+        int rt[QW];
+        float qr[QW][P > 0 ? P : 1] = {}, qn[QW];
+        bool any = false;
+#pragma unroll
+        for (int h = 0; h < QW; h++) {
+            rt[h] = s_rt[q0 + h];
+            any |= rt[h] > 0;
+            qn[h] = qs[(q0 + h) * pp + p];
+            if constexpr (P > 0) {
+#pragma unroll
+                for (int i = 0; i < P; i++) qr[h][i] = -2.f * qs[(q0 + h) * pp + i];
+            }
+        }
+        // body(h, value, whether the lane holds a row) for the first nrows rows
+        auto clamp = [](float v) { return v < 0.f ? 0.f : v; };  // keeps NaN
+        auto sweep = [&](int64_t nrows, auto body) {
+            const int64_t ntiles = (nrows + TT - 1) / TT;
+            // a tile's rows, rounded up to a multiple of 4 (within the padded copy), 16 bytes a copy
+            auto issue = [&](int64_t tile) {
+                const int64_t base = tile * TT;
+                const int nchunk = (int)round_up(min((int64_t)TT, nrows - base), 4) * pp / 4;
+                const float *g = Ys + base * pp;
+                float *t = tiles + (size_t)(tile & 1) * TT * pp;
+                for (int e = threadIdx.x; e < nchunk; e += SCREEN_THREADS) cp_async16(t + 4 * e, g + 4 * e);
+                cp_async_commit();
+            };
+            issue(0);
+            cp_async_wait_all();
+            __syncthreads();
+            for (int64_t tile = 0; tile < ntiles; tile++) {
+                if (tile + 1 < ntiles) issue(tile + 1);  // in flight during the sweep
+                const int cnt = (int)min((int64_t)TT, nrows - tile * TT);
+                const float *t = tiles + (size_t)(tile & 1) * TT * pp;
+                for (int pt = 32 * sub; pt < cnt; pt += 32 * W) {
+                    // (lanes past the last row read the buffer, and are masked)
+                    const bool live = pt + lane < cnt;
+                    const float *row = t + (pt + lane) * PS;
+                    float sd[QW];
+                    const float xn = row[np];
+#pragma unroll
+                    for (int h = 0; h < QW; h++) sd[h] = xn + qn[h];
+                    if constexpr (P > 0) {
+#pragma unroll
+                        for (int i = 0; i < P; i++) {
+                            const float x = row[i];
+#pragma unroll
+                            for (int h = 0; h < QW; h++) sd[h] = fmaf(x, qr[h][i], sd[h]);
+                        }
+                    } else {
+                        for (int i = 0; i < p; i++) {
+                            const float x = row[i];
+#pragma unroll
+                            for (int h = 0; h < QW; h++) sd[h] = fmaf(x, -2.f * qs[(q0 + h) * pp + i], sd[h]);
+                        }
+                    }
+#pragma unroll
+                    for (int h = 0; h < QW; h++) body(h, sd[h], live);
+                }
+                // the next tile has landed and every warp is done with this one
+                cp_async_wait_all();
+                __syncthreads();
+            }
+        };
+        bool two = true;  // two histogram sweeps over all rows
+        if (!__syncthreads_or(any)) {
+            two = false;
+        } else if (nsub > 0) {
+            sweep(nsub, [&](int h, float v, bool live) {
+                const int b = min(max((int)(__float_as_uint(clamp(v)) >> 19) - cbase, 0), HB - 1);
+                if (rt[h] > 0 && live) atomicAdd(&hist[(q0 + h) * SLOT + b], 1u);
+            });
+            float U[QW];
+#pragma unroll
+            for (int h = 0; h < QW; h++) {
+                U[h] = -1.f;
+                if (rt[h] == 0) continue;
+                uint32_t b, before;
+                find_bin(hist + (q0 + h) * SLOT, (uint32_t)rt[h], lane, b, before);
+                U[h] = b == HB - 1 ? CUDART_INF_F : __uint_as_float((uint32_t)((int)b + cbase) << 19 | 0x7FFFFu);
+                if (lane == 0) s_U[q0 + h] = U[h];  // (the warps of a group write the same value)
+            }
+            __syncthreads();
+            // each thread a column of its own in the lists: no atomic, no branch
+            int n[QW] = {};
+            uint32_t *col = hist + q0 * SLOT + sub * 32 + lane;
+            sweep(nsamp, [&](int h, float v, bool live) {
+                const bool hit = live && v <= U[h];
+                if (hit && n[h] < SAMPLE_DEPTH) col[h * SLOT + n[h] * COLS] = __float_as_uint(v);
+                n[h] += hit;
+            });
+#pragma unroll
+            for (int h = 0; h < QW; h++) s_n[(q0 + h) * COLS + sub * 32 + lane] = (uint8_t)min(n[h], 255);
+            __syncthreads();
+            // A list holds the wanted rank unless a column overflowed, or the
+            // subset's bound is no number.  Selection by a warp a query: histogram of the
+            // distance below U in units of 2^17 (64ths of an octave), then of 2^11.
+            bool bad = false;
+            uint32_t *h2 = reinterpret_cast<uint32_t *>(tiles) + w * 256;
+            for (int ql = w; ql < nq; ql += 8) {
+                const int target = s_rt[ql];
+                if (target == 0) continue;
+                int len[W], n = 0, longest = 0;  // of the lane's columns
+#pragma unroll
+                for (int v = 0; v < W; v++) {
+                    len[v] = s_n[ql * COLS + v * 32 + lane];
+                    n += len[v];
+                    longest = max(longest, len[v]);
+                }
+                n = (int)__reduce_add_sync(LAGP_FULL_MASK, (unsigned)n);
+                if (__any_sync(LAGP_FULL_MASK, longest > SAMPLE_DEPTH) || n < target || !(s_U[ql] < CUDART_INF_F)) {
+                    bad = true;
+                    continue;
+                }
+                const uint32_t Ub = __float_as_uint(s_U[ql]), *list = hist + ql * SLOT + lane;
+                // (descending distance below U: the smallest values lie in the last bins)
+                uint32_t d17 = 0;
+                int rank = n - target + 1;  // of the wanted value by distance below U, the smallest first
+                for (int level = 0; level < 2; level++) {
+                    const int nb = level == 0 ? 256 : 64;
+                    for (int b = lane; b < nb; b += 32) h2[b] = 0;
+                    __syncwarp();
+#pragma unroll
+                    for (int v = 0; v < W; v++)
+                        for (int e = 0; e < len[v]; e++) {
+                            const float f = __uint_as_float(list[e * COLS + v * 32]);
+                            const uint32_t d = Ub - __float_as_uint(clamp(f));
+                            if (level == 0) atomicAdd(&h2[min(d >> 17, 255u)], 1u);
+                            else if (min(d >> 17, 255u) == d17) atomicAdd(&h2[d >> 11 & 63u], 1u);
+                        }
+                    __syncwarp();
+                    // the bin that holds the rank, 8 (2) bins a lane
+                    const int per = nb / 32;
+                    int sum = 0;
+                    for (int b = 0; b < per; b++) sum += (int)h2[lane * per + b];
+                    int incl = sum;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int t = __shfl_up_sync(LAGP_FULL_MASK, incl, o);
+                        if (lane >= o) incl += t;
+                    }
+                    const int L = __ffs(__ballot_sync(LAGP_FULL_MASK, incl >= rank)) - 1;
+                    int c = __shfl_sync(LAGP_FULL_MASK, incl - sum, L);
+                    int b = L * per;
+                    for (; b < L * per + per - 1 && c + (int)h2[b] < rank; b++) c += (int)h2[b];
+                    rank -= c;
+                    __syncwarp();
+                    if (level == 0) {
+                        d17 = (uint32_t)b;
+                        if (d17 == 255u) {  // four octaves below the bound or more
+                            bad = true;
+                            break;
+                        }
+                    } else if (lane == 0) {
+                        s_tau[ql] = __uint_as_float(((Ub >> L2_SHIFT) - (d17 << 6 | (uint32_t)b)) << L2_SHIFT | L2_LOW);
+                    }
+                }
+            }
+            two = __syncthreads_or(bad);
+            if (two) clear();
+        }
+        if (two) {
+            uint32_t b1[QW] = {}, before[QW] = {};
+            for (int pass = 0; pass < 2; pass++) {
+                sweep(nsamp, [&](int h, float v, bool live) {
+                    const uint32_t bits = __float_as_uint(clamp(v));
+                    uint32_t *hh = hist + (q0 + h) * SLOT;
+                    if (rt[h] == 0 || !live) return;
+                    if (pass == 0) atomicAdd(&hh[bits >> L1_SHIFT & (HB - 1)], 1u);
+                    else if ((bits >> L1_SHIFT & (HB - 1)) == b1[h]) atomicAdd(&hh[bits >> L2_SHIFT & (HB - 1)], 1u);
+                });
+#pragma unroll
+                for (int h = 0; h < QW; h++) {
+                    if (rt[h] == 0) continue;
+                    uint32_t b, bf;
+                    find_bin(hist + (q0 + h) * SLOT, (uint32_t)rt[h] - before[h], lane, b, bf);
+                    if (pass == 0) b1[h] = b, before[h] = bf;
+                    else if (lane == 0) s_tau[q0 + h] = __uint_as_float(b1[h] << L1_SHIFT | b << L2_SHIFT | L2_LOW);
+                }
+                __syncthreads();
+                if (pass == 0) clear();
+            }
+        }
+        __syncthreads();
+        for (int ql = threadIdx.x; ql < nq && blk * nq + ql < M; ql += SCREEN_THREADS) tau_out[blk * nq + ql] = s_tau[ql];
         __syncthreads();
     }
 }
@@ -1311,27 +1582,54 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     for (int t = tid; t < Npmax; t += NT) out[t] = t < k ? (int32_t)(uint32_t)sk[t] : -1;
 }
 
-// The screen's first launch: the sampled threshold and the collection on the
-// norm expansion (CUDA cores), or with tau0 the sampled threshold only (the
-// collection then runs on the tensor cores); and the exact retry of the
-// flagged queries on the direct form.
+// The screen on CUDA cores (norm expansion), and the exact retry of the
+// flagged queries (direct form).
 template <int P>
 void launch_screen(lagp_ctx *ctx, bool retry_pass, dim3 grid, size_t smem, const float *Y32, const float *Ys,
                    int64_t N, int p, const void *Xref, lagp_dtype dt, int64_t M, const int32_t *Np, int32_t Npmax,
                    const unsigned long long *kmax, const unsigned long long *kmin, int32_t *cand, int32_t Cmax,
-                   int32_t *cc, int32_t *status, int64_t stride, int32_t *retry, int *counters, float *tau0) {
+                   int32_t *cc, int32_t *status, int64_t stride, int32_t *retry, int *counters) {
     cudaStream_t st = ctx->stream;
     if (!retry_pass) {
         cudaFuncSetAttribute(knn_screen<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         knn_screen<P, true><<<grid, SCREEN_THREADS, smem, st>>>(Y32, Ys, N, p, Xref, dt, M, Np, Npmax, kmax, kmin,
-                                                                cand, Cmax, cc, status, stride, retry, 0,
-                                                                counters, tau0);
+                                                                cand, Cmax, cc, status, stride, retry, 0, counters);
     } else {
         cudaFuncSetAttribute(knn_screen<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         knn_screen<P, false><<<grid, SCREEN_THREADS, smem, st>>>(Y32, Y32, N, p, Xref, dt, M, Np, Npmax, kmax,
                                                                  kmin, cand, Cmax, cc, status, 1, retry, 1,
-                                                                 counters + 1, nullptr);
+                                                                 counters + 1);
     }
+    ctx->launches++;
+}
+
+// The sampled thresholds.  Queries a warp, warps a query group and rows of the
+// first sweep follow the problem: four queries a warp keep the sweep off the
+// shared-memory loads (9 loads for 36 multiply-adds at p = 8); with few
+// queries all eight warps share a group, and then one query, so that M = 100
+// still meets 100 SMs.
+template <int P>
+void launch_sample(lagp_ctx *ctx, const float *Ys, int64_t nsamp, int p, const void *Xref, lagp_dtype dt, int64_t M,
+                   const int32_t *Np, int32_t Npmax, int64_t stride, const unsigned long long *kmax,
+                   const unsigned long long *kmin, int *counter, float *tau0) {
+    const int64_t rt = sample_rank(Npmax, stride, nsamp);
+    const int pp = row_stride(p);
+    auto go = [&](auto kern, int qw, int W) {
+        // first sweep: one row in `first`, so that a thread lists about a
+        // quarter of its column's depth (a few in 10^4 columns overflow)
+        const int64_t first = std::min<int64_t>(8, SAMPLE_DEPTH / 5 * 32 * W / rt);
+        int64_t nsub = first >= 2 ? (nsamp + first - 1) / first : 0;
+        if (nsub < rt) nsub = 0;
+        const int nq = 8 * qw / W;
+        const size_t smem = (size_t)nq * SAMPLE_DEPTH * 32 * W * 4 + 2 * (size_t)sample_tile(pp) * pp * 4 + (size_t)nq * pp * 4;
+        const int64_t nblk = (M + nq - 1) / nq;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kern<<<(unsigned)std::min<int64_t>(nblk, (int64_t)ctx->num_sms * 2), SCREEN_THREADS, smem, ctx->stream>>>(
+            Ys, nsamp, nsub, p, Xref, dt, M, Np, Npmax, stride, kmax, kmin, counter, tau0);
+    };
+    if (M >= 32 * (int64_t)ctx->num_sms) go(knn_sample<P, 4, 2>, 4, 2);
+    else if (M >= 4 * (int64_t)ctx->num_sms) go(knn_sample<P, 4, 8>, 4, 8);
+    else go(knn_sample<P, 1, 8>, 1, 8);
     ctx->launches++;
 }
 
@@ -1358,7 +1656,7 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     if (stride > 1) {
         int32_t pow2 = 1;
         while (pow2 < Cmax) pow2 <<= 1;
-        const int64_t rt = std::min<int64_t>((13 * (int64_t)Npmax + 10 * stride - 1) / (10 * stride) + 16, nsamp);
+        const int64_t rt = sample_rank(Npmax, stride, nsamp);
         const double want = (double)rt * stride + 6.0 * std::sqrt((double)rt) * stride + 512.0;
         Cmax = (int32_t)std::min<double>(std::max<double>(Cmax, std::ceil(want)), std::min(pow2, CAND_CAP));
     }
@@ -1404,8 +1702,10 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
         order.query = query;
         order.box = reinterpret_cast<float *>(w + oBox);
     }
+    int64_t spread = std::max<int64_t>(1, (int64_t)(0.6180339887 * (double)nsamp));
+    while (std::gcd(spread, nsamp) != 1) spread++;
     knn_prep<<<blocks, 256, 0, st>>>(X, N, p, dtype, kmax, kmin, order.row, Y32, Npad, stride > 1 ? Ys : nullptr,
-                                     nsamp_pad, stride, kc, Yv);
+                                     nsamp, nsamp_pad, stride, spread, kc, Yv);
     ctx->launches += 2;
     if (order.box) {
         knn_boxes<<<blocks, 256, 0, st>>>(Y32, N, p, (int)((N + 127) / 128), order.box);
@@ -1437,10 +1737,10 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     cudaFuncSetAttribute(knn_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_big);
     auto screen = [&](bool retry_pass) {
         switch (p) {
-            case 2: launch_screen<2>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters, tau0); break;
-            case 3: launch_screen<3>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters, tau0); break;
-            case 8: launch_screen<8>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters, tau0); break;
-            default: launch_screen<0>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters, tau0); break;
+            case 2: launch_screen<2>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters); break;
+            case 3: launch_screen<3>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters); break;
+            case 8: launch_screen<8>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters); break;
+            default: launch_screen<0>(ctx, retry_pass, grid, smem, Y32, Ys, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, cand, Cmax, cc, status, stride, retry, counters); break;
         }
     };
     auto rank = [&]() {
@@ -1460,7 +1760,16 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
                                                     idx, kc, rflags, bigf);
         ctx->launches++;
     };
-    screen(false);
+    if (tc_ws) {
+        switch (p) {
+            case 2: launch_sample<2>(ctx, Ys, nsamp, p, Xref, dtype, M, Np, Npmax, stride, kmax, kmin, counters, tau0); break;
+            case 3: launch_sample<3>(ctx, Ys, nsamp, p, Xref, dtype, M, Np, Npmax, stride, kmax, kmin, counters, tau0); break;
+            case 8: launch_sample<8>(ctx, Ys, nsamp, p, Xref, dtype, M, Np, Npmax, stride, kmax, kmin, counters, tau0); break;
+            default: launch_sample<0>(ctx, Ys, nsamp, p, Xref, dtype, M, Np, Npmax, stride, kmax, kmin, counters, tau0); break;
+        }
+    } else {
+        screen(false);
+    }
     LAGP_CUDA(ctx, cudaGetLastError());
     if (tc_ws) {
         // collection on the tensor cores, the sort (which checks each query's
