@@ -1354,8 +1354,10 @@ knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
 // above (3, 5, 6).  Linear in the number of rows, eight barriers, against the
 // bitonic sort's (log^2) with a radix selection before it: N' = 1500 of 2,600
 // rows, 201,600 queries, 32.8 -> 8.7 ms; N' = 2000 of 3,600, 25,000 queries,
-// 14.7 -> 3.9 ms.  Bound: instruction issue and the
-// latency of the gathers.  Left to knn_sort (bigf): distances that are not
+// 14.7 -> 3.9 ms.  With the FP64 distances of all tied rows computed side by side
+// (a run a thread kept the FP64 unit busy for 41% of the time): 7.3 and 2.4 ms.
+// Bound: instruction issue and the latency of the gathers between barriers
+// (128 or 512 threads a query in place of 256: 30% slower).  Left to knn_sort (bigf): distances that are not
 // finite, a bucket of more than RANK_BUCKET rows, runs longer than 32 (many
 // equal distances), survivors past the placed buckets.
 constexpr int RANK_BUCKET = 24;
@@ -1384,17 +1386,18 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     double *dk = reinterpret_cast<double *>(smem_raw);                                  // cap, after the buckets
     unsigned long long *sk = reinterpret_cast<unsigned long long *>(smem_raw + (size_t)nb * 4);  // cap (s, row) keys
     uint32_t *tied = reinterpret_cast<uint32_t *>(sk + cap);                            // cap / 32 + 1
+    uint16_t *list = reinterpret_cast<uint16_t *>(tied + cap / 32 + 1);                 // cap: rows in runs of ties
     __shared__ double xq[64];
     __shared__ float yq[64];
     __shared__ int wsum[NT / 32];
     __shared__ uint32_t s_lo, s_hi;
-    __shared__ int s_kb, s_left, s_fail, s_S;
+    __shared__ int s_kb, s_left, s_fail, s_S, s_ties;
     __shared__ float s_tauf, s_d2f;
     if (tid < p) {
         xq[tid] = load_coord64(Xref, q, p, tid, dt);
         yq[tid] = (float)(xq[tid] - kc->c[tid]);
     }
-    if (tid == 0) s_lo = 0xFFFFFFFFu, s_hi = 0u, s_left = 0;
+    if (tid == 0) s_lo = 0xFFFFFFFFu, s_hi = 0u, s_left = s_ties = 0;
     for (int b = tid; b < nb; b += NT) start[b] = 0u;
     __syncthreads();
     // direct-form FP32 values (non-negative floats order like their bits)
@@ -1544,6 +1547,22 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     }
     __syncthreads();
     auto is_tied = [&](int i) { return (tied[i >> 5] >> (i & 31)) & 1u; };
+    // FP64 distances of the rows in runs, gathered so that they share the FP64
+    // unit's instructions (it takes as long for one lane as for 32)
+    for (int i = tid; i < S; i += NT)
+        if (is_tied(i) || (i > 0 && is_tied(i - 1))) list[atomicAdd(&s_ties, 1)] = (uint16_t)i;
+    __syncthreads();
+    for (int e = tid; e < s_ties; e += NT) {
+        const int t = list[e];
+        const int32_t r = (int32_t)(uint32_t)sk[t];
+        double sd = 0.0;
+        for (int c = 0; c < p; c++) {
+            const double diff = __dsub_rn(xq[c], load_coord64(X, r, p, c, dt));
+            sd = __dadd_rn(sd, __dmul_rn(diff, diff));
+        }
+        dk[t] = sd;
+    }
+    __syncthreads();
     for (int i = tid; i < S; i += NT) {
         if (!is_tied(i) || (i > 0 && is_tied(i - 1))) continue;  // not the start of a run
         int end = i + 1;  // the run is [i, end]
@@ -1551,15 +1570,6 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
         if (end - i >= 32) {
             s_left = 1;
             continue;
-        }
-        for (int t = i; t <= end; t++) {
-            const int32_t r = (int32_t)(uint32_t)sk[t];
-            double sd = 0.0;
-            for (int c = 0; c < p; c++) {
-                const double diff = __dsub_rn(xq[c], load_coord64(X, r, p, c, dt));
-                sd = __dadd_rn(sd, __dmul_rn(diff, diff));
-            }
-            dk[t] = sd;
         }
         for (int t = i + 1; t <= end; t++) {  // insertion sort on (d2, row)
             const double dv = dk[t];
@@ -1731,7 +1741,7 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     // shared memory of the rank (rows placed: N' and what shares the last
     // buckets) and of the general sort
     const int cap = std::min<int>((Npmax + Npmax / 8 + 128 + 31) & ~31, (Cmax + 31) & ~31);
-    const size_t smem_rank = (size_t)rank_buckets(cap) * 4 + (size_t)cap * 8 + (size_t)(cap / 32 + 1) * 4;
+    const size_t smem_rank = (size_t)rank_buckets(cap) * 4 + (size_t)cap * 10 + (size_t)(cap / 32 + 1) * 4;
     const size_t smem_big = (size_t)Cp * 16;
     if (std::max(smem_big, smem_rank) > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "lagp_knn: N' too large for the sort");
     cudaFuncSetAttribute(knn_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_big);
