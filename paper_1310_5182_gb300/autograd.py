@@ -29,7 +29,7 @@ class LocalGP(torch.autograd.Function):
     def backward(ctx, gmean, gs2):
         (d,) = ctx.saved_tensors
         X, Y, Xref, sel, n, gval, g_is_tensor = ctx.args
-        r = _L.lagp_predict_grad(X, Y, Xref, sel, n, d, gval)
+        r = _L._predict_grad(X, Y, Xref, sel, n, d, gval, _L._GRADS[:4])
         gmean = torch.zeros_like(d) if gmean is None else gmean
         gs2 = torch.zeros_like(d) if gs2 is None else gs2
         grad_d = gmean * r["dmean_dd"] + gs2 * r["ds2_dd"]
@@ -41,8 +41,8 @@ class LocalLogLik(torch.autograd.Function):
     @staticmethod
     def forward(ctx, d, g, X, Y, Xref, sel, n):
         gval = float(g.detach().item()) if isinstance(g, torch.Tensor) else float(g)
-        r = _L.lagp_predict_grad(X, Y, Xref, sel, n, d.detach(), gval)
-        ll = _L.lagp_mle_step(X, Y, sel, n, d.detach(), gval, 1e-300, 1e300, 0)["llik"]
+        r = _L._predict_grad(X, Y, Xref, sel, n, d.detach(), gval, _L._GRADS[4:])
+        ll = _L._mle_step(X, Y, sel, n, d.detach(), gval, 1e-300, 1e300, 0, ("llik",))["llik"]
         ctx.save_for_backward(r["dllik_dd"], r["dllik_dg"])
         ctx.g_is_tensor = isinstance(g, torch.Tensor)
         return ll

@@ -543,7 +543,9 @@ struct GradOut {
 // Bound: the FP64 unit and the barriers of the column-by-column factor.  l'
 // and dl/dg need tr(K^{-1} K') and tr(K^{-1}) only: no product K^{-1} K' (n^3,
 // the larger half of the work before); w comes with the factorisation, b from
-// one column-by-column solve.  5,000 locations, n = 50: 3.85 -> 2.2 ms.
+// one column-by-column solve.  The prediction's derivatives alone need no
+// inverse either: two solves, a warp each.  5,000 locations, n = 50: all six
+// 3.85 -> 2.2 ms, the prediction's four 1.4 ms.
 __global__ void __launch_bounds__(GP_THREADS)
 grad_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, GradOut o) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -553,6 +555,8 @@ grad_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, G
     GpWork W = work_for_block(ws, nmax, ld);
     __shared__ int s_loc, s_flag, s_chol;
     Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
+    // (what is not wanted stays as shared memory holds it, and reaches no output)
+    const bool want_p = o.dmean_dd || o.dmean_dg || o.ds2_dd || o.ds2_dg, want_l = o.dllik_dd || o.dllik_dg;
     for (;;) {
         if (b.tid == 0) s_loc = atomicAdd(counter, 1);
         __syncthreads();
@@ -587,10 +591,14 @@ grad_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, G
                 }
                 block_sums<2>(q, b);
                 const double psi = q[0], ww = q[1];
-                inverse_from_L(W, nm, ld, S.rd, S.t3, S.a, b);  // K^{-1}, a = K^{-1} y
+                if (want_l) {
+                    inverse_from_L(W, nm, ld, S.rd, S.t3, S.a, b);  // K^{-1}, a = K^{-1} y
+                } else if (b.warp == 1) {  // side by side with b
+                    warp_backward(W.L, ld, S.rd, S.t3, S.a, nm, b.lane);
+                }
                 // b = K^{-1} kx (t1) by the second triangular solve (v = 1 + g -
                 // w^T w: no explicit inverse, no cancellation against k^T b)
-                if (b.warp == 0) warp_backward(W.L, ld, S.rd, S.t2, S.t1, nm, b.lane);
+                if (want_p && b.warp == 0) warp_backward(W.L, ld, S.rd, S.t2, S.t1, nm, b.lane);
                 __syncthreads();
                 // K'a and K'b (K' symmetric: read by columns, the lanes of a
                 // warp side by side)
@@ -607,7 +615,7 @@ grad_kernel(GpArgs a, const double *__restrict__ dv, int *counter, double *ws, G
                 }
                 // tr(K^{-1} K') over the lower triangle (K' has a zero diagonal), tr(K^{-1})
                 double trKiK1 = 0.0, trKi = 0.0;
-                for (int e = b.tid; e < nm * (nm + 1) / 2; e += GP_THREADS) {
+                for (int e = b.tid; want_l && e < nm * (nm + 1) / 2; e += GP_THREADS) {
                     int i, k;
                     tri_index(e, i, k);
                     const double q = W.Ki[(size_t)i * ld + k];

@@ -454,43 +454,54 @@ def lagp_predict_noalloc(X, Y, Xref, sel, n, d, g, out=None):
 def lagp_mle_step(X, Y, sel, n, d0, g, dmin, dmax, max_iter):
     """a8: per-location Newton MLE of d.  Returns dict(d, llik, dllik,
     d2llik, iters, status)."""
+    return _mle_step(X, Y, sel, n, d0, g, dmin, dmax, max_iter, ("llik", "dllik", "d2llik"))
+
+
+def _mle_step(X, Y, sel, n, d0, g, dmin, dmax, max_iter, keys):
     ctx = context(X.device)
     N, p = X.shape
     M, n_max = sel.shape
     nt, npp = _opt_i32(n, M, X.device, "n", uniform=n_max)
     d = _per_loc_f64(d0, M, X.device)
-    out = {k: torch.empty(M, dtype=torch.float64, device=X.device) for k in ("llik", "dllik", "d2llik")}
+    out = {k: torch.empty(M, dtype=torch.float64, device=X.device) for k in keys}
     iters = torch.empty(M, dtype=torch.int32, device=X.device)
     status = torch.empty(M, dtype=torch.int32, device=X.device)
     if M:
         _check(_lib.lagp_mle_step(ctx, _dev(X, "X"), _dev(Y, "Y", X.dtype), N, p, _dtype_code(X), M,
                                   _dev(sel, "sel", torch.int32), npp, n_max, _dev(d, "d"), float(g),
-                                  float(dmin), float(dmax), int(max_iter), _dev(out["llik"], "llik"),
-                                  _dev(out["dllik"], "dllik"), _dev(out["d2llik"], "d2llik"),
+                                  float(dmin), float(dmax), int(max_iter),
+                                  *[_dev(out[k], k) if k in keys else None for k in ("llik", "dllik", "d2llik")],
                                   _dev(iters, "iters"), _dev(status, "status")),
                ctx, "lagp_mle_step")
     out.update(d=d, iters=iters, status=status)
     return out
 
 
-def lagp_predict_grad(X, Y, Xref, sel, n, d, g):
-    """Adjoint: d/dd, d/dg of mean, s2 and the log-likelihood, per location."""
+_GRADS = ("dmean_dd", "dmean_dg", "ds2_dd", "ds2_dg", "dllik_dd", "dllik_dg")
+
+
+def _predict_grad(X, Y, Xref, sel, n, d, g, keys):
     ctx = context(X.device)
     N, p = X.shape
     M, n_max = sel.shape
     nt, npp = _opt_i32(n, M, X.device, "n", uniform=n_max)
     dt = _per_loc_f64(d, M, X.device)
-    keys = ("dmean_dd", "dmean_dg", "ds2_dd", "ds2_dg", "dllik_dd", "dllik_dg")
     out = {k: torch.empty(M, dtype=torch.float64, device=X.device) for k in keys}
     status = torch.empty(M, dtype=torch.int32, device=X.device)
     if M:
         _check(_lib.lagp_predict_grad(ctx, _dev(X, "X"), _dev(Y, "Y", X.dtype), N, p, _dtype_code(X),
                                       _dev(Xref, "Xref", X.dtype), M, _dev(sel, "sel", torch.int32),
                                       npp, n_max, _dev(dt, "d"), float(g),
-                                      *[_dev(out[k], k) for k in keys], _dev(status, "status")),
+                                      *[_dev(out[k], k) if k in keys else None for k in _GRADS],
+                                      _dev(status, "status")),
                ctx, "lagp_predict_grad")
     out["status"] = status
     return out
+
+
+def lagp_predict_grad(X, Y, Xref, sel, n, d, g):
+    """Adjoint: d/dd, d/dg of mean, s2 and the log-likelihood, per location."""
+    return _predict_grad(X, Y, Xref, sel, n, d, g, _GRADS)
 
 
 def lagp_agp(X, Y, Xref, n0, n, Nprime, d0, g, prec="f32bulk", mle=None, rounds=1, device=0):
