@@ -1,6 +1,6 @@
 // Cholesky factorisation of a local correlation matrix in 59-bit fixed point
 // (fx59.cuh), with further rows and, optionally, its first and second
-// derivatives in forward mode; one CTA of FXT threads, all in shared memory.
+// derivatives in forward mode; one CTA of T threads (FXT unless stated), all in shared memory.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -121,12 +121,12 @@ __device__ __forceinline__ void fx_acc(long long &hi, long long &mid, int xh, in
 
 // The sums of columns c, c + 1 over k < c, subtracted from the rows below the
 // diagonal block, by the warps 1 and up.  2^KL lanes share a row's sum.
-template <int NM, int KL>
+template <int NM, int KL, int T>
 __device__ __forceinline__ void fx_sums(const FxFactor &F, int c, int lane, int warp) {
     constexpr int RP = 32 >> KL, KS = 1 << KL;  // row pairs and shares of a warp
     const int m = F.m, n = F.n;
     const int rp = lane & (RP - 1), ks = lane / RP;
-    for (int base = min(c + 2, n) + (warp - 1) * 2 * RP; base < m; base += (FXW - 1) * 2 * RP) {
+    for (int base = min(c + 2, n) + (warp - 1) * 2 * RP; base < m; base += (T / 32 - 1) * 2 * RP) {
         const int iA = base + rp, iB = iA + RP;
         const int ia = min(iA, m - 1), ib = min(iB, m - 1), j1 = min(c + 1, m - 1);
         long long hi[NM][2][2], mid[NM][2][2];
@@ -306,7 +306,7 @@ __device__ __forceinline__ void fx_diagonal(const FxFactor &F, FxDiag *diag, int
 // makes the next diagonal block (a serial chain of some 1,500 cycles) while
 // the others form the sums of the next two columns.  Returns the flag
 // (block-uniform).
-template <int NM>
+template <int NM, int T = FXT>
 __device__ int fx_factorise(const FxFactor &F, const Blk &b) {
     const int n = F.n, m = F.m;
     __shared__ FxDiag s_diag;
@@ -319,21 +319,21 @@ __device__ int fx_factorise(const FxFactor &F, const Blk &b) {
         const bool two = c + 1 < n;
         const FxDiag D = s_diag;
         // (rows from warp 1 on: warp 0 has the serial chains)
-        for (int i = c + (two ? 2 : 1) + (b.warp + FXW - 1) % FXW * 32 + b.lane; i < m; i += FXT) {
+        for (int i = c + (two ? 2 : 1) + (b.warp + T / 32 - 1) % (T / 32) * 32 + b.lane; i < m; i += T) {
             unsigned bad = 0;
             const int at = fx_slot(i, c, m);  // columns c, c + 1 of a row are adjacent
-            long long S[NM], T[NM];
+            long long S[NM], S2[NM];
 #pragma unroll
             for (int g = 0; g < NM; g++) {
                 const longlong2 v = *reinterpret_cast<const longlong2 *>(fx_raw(F, g, at));
                 S[g] = v.x;
-                T[g] = v.y;
+                S2[g] = v.y;
             }
             FxRow<NM> r, q;
             fx_column<NM>(S, D.y[0], D.t[0], D.nl1[0], D.nl2[0], r, bad);
             if (two) {
-                fx_update<NM>(T, r, D.na, D.nb, D.ne);
-                fx_column<NM>(T, D.y[1], D.t[1], D.nl1[1], D.nl2[1], q, bad);
+                fx_update<NM>(S2, r, D.na, D.nb, D.ne);
+                fx_column<NM>(S2, D.y[1], D.t[1], D.nl1[1], D.nl2[1], q, bad);
             }
             // |x| < 1 in the further rows, whose norm nothing bounds
             if (i >= n)
@@ -355,9 +355,9 @@ __device__ int fx_factorise(const FxFactor &F, const Blk &b) {
         if (c + 2 < n) {
             const int R = m - (c + 4);
             if (b.warp == 0) fx_diagonal<NM>(F, &s_diag, &s_out, c + 2, b.lane);
-            else if (R > 24) fx_sums<NM, 2>(F, c + 2, b.lane, b.warp);
-            else if (R > 12) fx_sums<NM, 3>(F, c + 2, b.lane, b.warp);
-            else fx_sums<NM, 4>(F, c + 2, b.lane, b.warp);
+            else if (R > 24) fx_sums<NM, 2, T>(F, c + 2, b.lane, b.warp);
+            else if (R > 12) fx_sums<NM, 3, T>(F, c + 2, b.lane, b.warp);
+            else fx_sums<NM, 4, T>(F, c + 2, b.lane, b.warp);
             __syncthreads();
         }
     }
@@ -365,15 +365,16 @@ __device__ int fx_factorise(const FxFactor &F, const Blk &b) {
 }
 
 // Exponent e with max_i |v_i| < 2^e over the block's n values (INT_MAX when
-// one is not finite or all are zero); red: FXW ints.
+// one is not finite or all are zero); red: T / 32 ints.
+template <int T = FXT>
 __device__ int fx_exponent(const double *v, int n, int *red, const Blk &b) {
     int top = 0;
     __syncthreads();
-    for (int i = b.tid; i < n; i += FXT) top = max(top, (__double2hiint(v[i]) >> 20) & 0x7ff);
+    for (int i = b.tid; i < n; i += T) top = max(top, (__double2hiint(v[i]) >> 20) & 0x7ff);
     top = __reduce_max_sync(LAGP_FULL_MASK, top);
     if (b.lane == 0) red[b.warp] = top;
     __syncthreads();
-    top = max(max(red[0], red[1]), max(red[2], red[3]));
+    for (int w = 0; w < T / 32; w++) top = max(top, red[w]);
     __syncthreads();
     // (subnormal responses and those near the largest double: FP64 kernels)
     return top < 64 || top > 1983 ? INT32_MAX : top - 1022;

@@ -35,9 +35,9 @@ struct Blk {
 
 // Block sums of NV values at once: warp sums, then one warp adds the warps'
 // partials (not every thread); three barriers for all NV.
-template <int NV>
+template <int NV, int T = GP_THREADS>
 __device__ void block_sums(double (&v)[NV], const Blk &b) {
-    __shared__ double part[GP_WARPS * NV], tot[NV];
+    __shared__ double part[T / 32 * NV], tot[NV];
 #pragma unroll
     for (int i = 0; i < NV; i++) v[i] = warp_sum(v[i]);
     __syncthreads();  // earlier readers of part / tot are done
@@ -47,7 +47,7 @@ __device__ void block_sums(double (&v)[NV], const Blk &b) {
     __syncthreads();
     if (b.warp == 0 && b.lane < NV) {
         double t = 0.0;
-        for (int w = 0; w < GP_WARPS; w++) t += part[w * NV + b.lane];
+        for (int w = 0; w < T / 32; w++) t += part[w * NV + b.lane];
         tot[b.lane] = t;
     }
     __syncthreads();
@@ -56,6 +56,7 @@ __device__ void block_sums(double (&v)[NV], const Blk &b) {
 }
 
 // Validate a location and load its design; returns the per-location status.
+template <int T = GP_THREADS>
 __device__ int load_design(const GpArgs &a, int64_t loc, int nm, const double *dptr, double *xd,
                            double *y, int *flag, const Blk &b) {
     if (b.tid == 0) *flag = LAGP_OK;
@@ -65,17 +66,17 @@ __device__ int load_design(const GpArgs &a, int64_t loc, int nm, const double *d
     __syncthreads();
     if (*flag != LAGP_OK) return *flag;
     const int32_t *s = a.sel + loc * a.nmax;
-    for (int t = b.tid; t < nm; t += GP_THREADS) {
+    for (int t = b.tid; t < nm; t += T) {
         int32_t r = s[t];
         if (r < 0 || r >= a.N) *flag = LAGP_EINVAL;
     }
     __syncthreads();
     if (*flag != LAGP_OK) return *flag;
-    for (int e = b.tid; e < nm * a.p; e += GP_THREADS) {
+    for (int e = b.tid; e < nm * a.p; e += T) {
         int t = e / a.p, i = e - t * a.p;
         xd[e] = load_coord64(a.X, s[t], a.p, i, a.dtype);
     }
-    for (int t = b.tid; t < nm; t += GP_THREADS)
+    for (int t = b.tid; t < nm; t += T)
         y[t] = a.dtype == LAGP_F64 ? static_cast<const double *>(a.Y)[s[t]]
                                    : (double)static_cast<const float *>(a.Y)[s[t]];
     __syncthreads();

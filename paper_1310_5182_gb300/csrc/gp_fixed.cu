@@ -155,12 +155,12 @@ struct FxEval {
 
 // l, and with NM = 3 l' and l'', of Eq. (gpk) at d from the packed squared distances; zs: the
 // power of two that z is scaled by; lgam: log Gamma(n/2) - (n/2) log 2 pi.
-template <int NM>
+template <int NM, int T>
 __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, double d, double g, int zs,
                           double lgam, const Blk &b) {
     const int n = F.n, m = F.m;
     const double ninv_d = -1.0 / d;
-    for (int e = b.tid; e < n * (n + 1) / 2; e += FXT) {
+    for (int e = b.tid; e < n * (n + 1) / 2; e += T) {
         int i, k;
         fx_tri(e, i, k);
         const double t = -(dist[e] * ninv_d);
@@ -173,20 +173,20 @@ __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, dou
             *fx_raw(F, 2, s) = fx_from(K2);
         }
     }
-    for (int k = b.tid; k < n; k += FXT) {
+    for (int k = b.tid; k < n; k += T) {
         const int s = fx_slot(n, k, m);
         *fx_raw(F, 0, s) = fx_from(fx_shift(fx_y(F)[k], -zs));
         if constexpr (NM == 3) *fx_raw(F, 1, s) = *fx_raw(F, 2, s) = 0;
     }
     FxEval r;
-    r.flag = fx_factorise<NM>(F, b);
+    r.flag = fx_factorise<NM, T>(F, b);
     r.l = r.dl = r.d2l = CUDART_NAN;
     if (r.flag) return r;
     // log|K| = -2 log prod r, r = 1 / l = y 2^t with y in (0.7, 1.42]: the
     // product of a warp's y stays in range, one logarithm for all
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     double prod = 1.0;
-    for (int i = b.tid; i < n; i += FXT) {
+    for (int i = b.tid; i < n; i += T) {
         const double yr = fx_double(fx_ry(F)[i]), ri = fx_shift(yr, fx_rt(F)[i]);
         prod *= yr;
         v[0] += fx_rt(F)[i];
@@ -204,13 +204,15 @@ __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, dou
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) prod *= __shfl_xor_sync(LAGP_FULL_MASK, prod, o);
-    __shared__ double s_prod[FXW];
+    __shared__ double s_prod[T / 32];
     if (b.lane == 0) s_prod[b.warp] = prod;
-    block_sums<6>(v, b);  // (its barriers order s_prod)
+    block_sums<6, T>(v, b);  // (its barriers order s_prod)
     __shared__ FxEval s_r;
     if (b.warp == 0) {
         // the two logarithms side by side, the other scalars on every lane
-        const double arg = b.lane ? scalbn(v[3], 2 * zs) / 2.0 : (s_prod[0] * s_prod[1]) * (s_prod[2] * s_prod[3]);
+        double all = 1.0;
+        for (int w = 0; w < T / 32; w += 2) all *= s_prod[w] * s_prod[w + 1];
+        const double arg = b.lane ? scalbn(v[3], 2 * zs) / 2.0 : all;
         const double lg = log(arg);
         const double half_logdet = -(__shfl_sync(LAGP_FULL_MASK, lg, 0) + v[0] * CUDART_LN2);
         const double logpsi = __shfl_sync(LAGP_FULL_MASK, lg, 1);
@@ -230,8 +232,8 @@ __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, dou
 // NM = 1: the likelihood at d alone (max_iter = 0, no derivative wanted), a
 // sixth of the arithmetic, a third of the shared memory: 5,000 locations, n =
 // 50, 1.3 -> 0.55 ms.
-template <int NM>
-__global__ void __launch_bounds__(FXT, NM == 3 ? 4 : 8)
+template <int NM, int T>
+__global__ void __launch_bounds__(T, (NM == 3 ? 512 : 1024) / T)
 mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int max_iter, MleOut o,
               unsigned long long *work) {
     const int nmax = f.cls_hi, p = a.p;
@@ -239,7 +241,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
     const int y_at = (int)max(NM * f.words * 16, (nmax * p * 8 + 15) & ~15);
     double *y = reinterpret_cast<double *>(fx_smem + y_at);
     double *dist = f.dist + (size_t)blockIdx.x * (nmax * (nmax + 1) / 2);
-    __shared__ int s_loc, s_flag, red[FXW];
+    __shared__ int s_loc, s_flag, red[T / 32];
     __shared__ double s_lgam;
     const Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
     unsigned long long n_llik = 0, n_derivs = 0;  // evaluations x n^3 (thread 0's count)
@@ -251,7 +253,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
         if (loc >= a.M) break;
         const int nm = a.n ? a.n[loc] : a.nmax;
         if (!fx_mine(f, nm, a.nmax)) continue;
-        int st = load_design(a, loc, nm, dv, xd, y, &s_flag, b);
+        int st = load_design<T>(a, loc, nm, dv, xd, y, &s_flag, b);
         const unsigned long long n3 = (unsigned long long)nm * nm * nm;
         FxEval r{CUDART_NAN, CUDART_NAN, CUDART_NAN, 0};
         int it = 0;
@@ -260,7 +262,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
             const double g = a.g;
             d = fmin(fmax(d, dmin), dmax);
             bool odd = false;
-            for (int e = b.tid; e < nm * (nm + 1) / 2; e += FXT) {
+            for (int e = b.tid; e < nm * (nm + 1) / 2; e += T) {
                 int i, k;
                 fx_tri(e, i, k);
                 const double D = sqd(xd + (size_t)i * p, xd + (size_t)k * p, p);
@@ -271,17 +273,17 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
                 const double hn = 0.5 * nm;
                 s_lgam = lgamma(hn) - hn * log(2.0 * CUDART_PI);
             }
-            const int ey = fx_exponent(y, nm, red, b);
+            const int ey = fx_exponent<T>(y, nm, red, b);
             odd = __syncthreads_or(odd) || ey == INT32_MAX;
             const double lgam = s_lgam;
             const FxFactor F{f.words, nm, nm + 1, y_at, nmax};
             int zs = ey + FX_Z0;
             // one evaluation; out of range: once more with a wider z
             auto eval = [&](double at) {
-                FxEval q = fx_llik<NM>(F, dist, at, g, zs, lgam, b);
+                FxEval q = fx_llik<NM, T>(F, dist, at, g, zs, lgam, b);
                 if (q.flag && zs < ey + FX_Z1) {
                     zs = ey + FX_Z1;
-                    q = fx_llik<NM>(F, dist, at, g, zs, lgam, b);
+                    q = fx_llik<NM, T>(F, dist, at, g, zs, lgam, b);
                 }
                 return q;
             };
@@ -363,8 +365,10 @@ size_t fx_mle_smem(int n, int p, int nm) {
 
 // Upper ends of the size classes: one launch a class, so that a location's
 // shared memory (n^2, 48 KB at n = 60 for the MLE) follows its own design size
-// and not the largest one's.
-constexpr int FX_CLASSES[] = {40, 64, 80, 104, 128};
+// and not the largest one's.  They lie where one CTA less fits an SM for the
+// MLE: four up to 64 rows, three to 76, two to 94 (against 40, 64, 80, 104, 128:
+// 20,000 locations of 30 to 100 rows, whole method, 307 -> 285 ms).
+constexpr int FX_CLASSES[] = {40, 64, 76, 94, 128};
 
 // Calls fn(lo, hi, first) for every class of sizes up to nmax, the largest
 // first (one class when all locations have the same size).
@@ -384,10 +388,10 @@ lagp_status fx_each_class(const GpArgs &a, Fn fn) {
 }
 
 template <typename Kern>
-int fx_grid(lagp_ctx *ctx, Kern kern, size_t smem, int64_t M) {
+int fx_grid(lagp_ctx *ctx, Kern kern, int threads, size_t smem, int64_t M) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, FXT, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * std::max(occ, 1), M));
 }
 
@@ -406,7 +410,7 @@ lagp_status launch_predict_fixed(lagp_ctx *ctx, const GpArgs &a, const double *d
                                  double *df, int32_t *status, int *counters, int *redo) {
     return fx_each_class(a, [&](int lo, int hi, bool first) -> lagp_status {
         const size_t smem = fx_predict_smem(hi, a.p);
-        const int grid = fx_grid(ctx, predict_fx_kernel, smem, a.M);
+        const int grid = fx_grid(ctx, predict_fx_kernel, FXT, smem, a.M);
         const FxLaunch f{lo, hi, first, fx_words(hi, hi + 2), counters++, redo, nullptr};
         predict_fx_kernel<<<grid, FXT, smem, ctx->stream>>>(a, f, d, mean, s2, df, status);
         ctx->launches++;
@@ -417,14 +421,21 @@ lagp_status launch_predict_fixed(lagp_ctx *ctx, const GpArgs &a, const double *d
 lagp_status launch_mle_fixed(lagp_ctx *ctx, const GpArgs &a, double *d, double dmin, double dmax, int32_t max_iter,
                              const MleOut &o, unsigned long long *work, double *ws, int *counters, int *redo) {
     return fx_each_class(a, [&](int lo, int hi, bool first) -> lagp_status {
-        auto go = [&](auto kern, int nm) {
-            const size_t smem = fx_mle_smem(hi, a.p, nm);
-            const int grid = std::min(fx_grid(ctx, kern, smem, a.M), ctx->num_sms * 16);
+        const int nm = max_iter == 0 && !o.dllik && !o.d2llik ? 1 : 3;
+        const size_t smem = fx_mle_smem(hi, a.p, nm);
+        auto go = [&](auto kern, int threads) {
+            const int grid = std::min(fx_grid(ctx, kern, threads, smem, a.M), ctx->num_sms * 16);
             const FxLaunch f{lo, hi, first, fx_words(hi, hi + 1), counters++, redo, ws};
-            kern<<<grid, FXT, smem, ctx->stream>>>(a, f, d, dmin, dmax, max_iter, o, work);
+            kern<<<grid, threads, smem, ctx->stream>>>(a, f, d, dmin, dmax, max_iter, o, work);
         };
-        if (max_iter == 0 && !o.dllik && !o.d2llik) go(mle_fx_kernel<1>, 1);
-        else go(mle_fx_kernel<3>, 3);
+        // where shared memory leaves room for two CTAs an SM, or one, a CTA has
+        // twice or three times the warps: 2,000 locations, n = 100, 13.7 -> 11.1 ms
+        // (256 threads 11.4, 512 11.6; 256 threads where three CTAs fit: no gain)
+        const int fit = (int)(ctx->smem_optin / (smem + 2048));
+        if (nm == 1) go(mle_fx_kernel<1, FXT>, FXT);
+        else if (fit < 2) go(mle_fx_kernel<3, 3 * FXT>, 3 * FXT);
+        else if (fit < 3) go(mle_fx_kernel<3, 2 * FXT>, 2 * FXT);
+        else go(mle_fx_kernel<3, FXT>, FXT);
         ctx->launches++;
         return lagp_cuda_check(ctx, cudaGetLastError(), "mle_fx_kernel");
     });
