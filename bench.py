@@ -112,12 +112,17 @@ def fp32_flops_per_location(n, Np, p):
 EXP_FLOPS = 16
 
 
-def fp64_schur_pass_flops_per_location(n, Np, p):
-    """FP64 flops of the FP64 Schur form's bulk pass: after step j every
-    unchosen candidate takes the dot product with the pivot column (2j), its
-    squared distance to the new point (3p), the scale by -1/d and the
-    EXP_FLOPS of the table-driven exp, and the updates of u, v and r (6)."""
-    return sum((Np - j - 1) * (2 * j + 3 * p + 7 + EXP_FLOPS) for j in range(0, n - 1))
+# 32 x 32 + 64-bit integer multiply-adds of a 59-bit fixed-point product, and
+# their rate: four cycles a warp instruction and sub-partition
+FX_MADS, FX_MADS_PER_CYCLE_SM = 3, 32
+
+
+def fx_schur_pass_mads_per_location(n, Np, p):
+    """Integer multiply-adds of the FP64 Schur form's bulk pass (its state is
+    59-bit fixed point): after step j every unchosen candidate takes the dot
+    product with the pivot column (j products), its squared distance to the
+    new point (p) and the updates of u, v and r (3)."""
+    return FX_MADS * sum((Np - j - 1) * (j + p + 3) for j in range(0, n - 1))
 
 
 def fp64_flops(work, M, n, p, fused):
@@ -427,16 +432,17 @@ def config_leg(L, dev, w, prec, steps, warmup, flush=None, oracle_S=0):
     else:
         res["stage_ms"] = {"knn": round(st_ms[0], 3), "search": round(st_ms[1], 3), "mle": round(st_ms[2], 3),
                            "predict": round(st_ms[3], 3)}
-        # the Newton MLE's FP64 work, counted by the kernel (n^3/3 flops a
-        # factorisation, 2 n^3 a derivative evaluation), against the FP64 peak
-        # from the unit counts (2 FMA lanes a cycle an SM) at the maximum clock
-        fl = (mw["llik_n3"] / 3 + 2 * mw["derivs_n3"]) / steps
+        # the Newton MLE's work, counted by the kernel (n^3 fixed-point products
+        # an evaluation: the factorisation, n^3/6, and its two derivatives),
+        # against the integer pipe's multiply-adds at the maximum clock
+        mads = FX_MADS * mw["llik_n3"] / steps
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        peak = sms * 4 * 2070e6 / 1e12
-        ach = fl / (st_ms[2] / 1e3) / 1e12
-        res["mle_roofline"] = {"bound": "alu", "kernel": "mle_kernel", "unit": "TFLOP/s", "achieved": ach,
-                               "peak": peak, "frac": ach / peak, "fp64_flops_per_launch": fl,
-                               "peak_source": f"derived: FP64 FMA, {sms} SMs x 4 flop/cycle x 2070 MHz"}
+        peak = sms * FX_MADS_PER_CYCLE_SM * 2070e6 / 1e12
+        ach = mads / (st_ms[2] / 1e3) / 1e12
+        res["mle_roofline"] = {"bound": "alu", "kernel": "mle_fx_kernel", "unit": "T integer multiply-adds/s",
+                               "achieved": ach, "peak": peak, "frac": ach / peak, "mads_per_launch": mads,
+                               "peak_source": f"derived: 32 x 32 + 64-bit integer multiply-add, {sms} SMs x "
+                                              f"{FX_MADS_PER_CYCLE_SM} a cycle x 2070 MHz"}
     if graph is not None:
         res["cuda_graph"] = graph
     if oracle_S:
@@ -453,7 +459,8 @@ def alc_eval_sweep(L, dev, flush, ns=range(16, 513, 4), Nc=60_000, oracle_ns=(16
     first 512 (inputs ordered by a numpy argsort of the squared distances).
     The factorisation of K_n (one CTA) is timed apart from the
     candidates' evaluation, as the paper times the ALC computation with the
-    matrices given.  FP64 flops per candidate: n^2 (the triangular solve) +
+    matrices given.  FP64 flops per candidate (of the criterion; the substitution
+    runs in fixed point, and the rate may pass the FP64 peak): n^2 (the triangular solve) +
     n (3p + 1 + EXP_FLOPS) (kernel values) + 4n (s, q) + 10."""
     import torch
     w = W.toy2d(seed=0, N=100_000, M=1)
@@ -715,8 +722,8 @@ def run_ours(args, rank, world, local_rank):
         work_s = {k: v / 3 for k, v in L.alc_work(dev).items()}
         f64s = {"value": M / (ms_s / 1e3), "unit": "predictions/s", "ms_per_step": ms_s,
                 "alc_kernel_ms": statistics.mean(s_alc),
-                "fp64_flops_per_launch": fp64_flops(work_s, M, n, w.p, True) +
-                M * fp64_schur_pass_flops_per_location(n, Np, w.p),
+                "fp64_flops_per_launch": fp64_flops(work_s, M, n, w.p, True),
+                "mads_per_launch": M * fx_schur_pass_mads_per_location(n, Np, w.p),
                 "rmse": float(np.sqrt(np.mean((ps["mean"].cpu().numpy() - w.truth) ** 2))),
                 "identical_designs_frac_vs_f32bulk":
                     float((ss["sel"] == s["sel"]).all(dim=1).float().mean().item())}
@@ -777,12 +784,11 @@ def run_ours(args, rank, world, local_rank):
     E = work_per_location(n0, n, Np)
     alc_avg = statistics.mean(alc_ms) / 1e3
     # peaks from the unit counts and the SM clock sampled during the timed
-    # region: FP32 (the FP32-bulk kernel issues no FP64 instruction) and FP64
-    # (the FP64 forms)
+    # region: FP32 (the FP32-bulk kernel issues no FP64 instruction) and integer
+    # multiply-adds (the fixed-point state of the FP64 Schur form)
     props = torch.cuda.get_device_properties(dev)
     sms = props.multi_processor_count
     mhz = (clocks or {}).get("sm_mhz") or 2070.0
-    fp64_peak = sms * 4 * mhz * 1e6 / 1e12      # 2 FP64 FMA lanes / cycle / SM
     fp32_peak = sms * 128 * 2 * mhz * 1e6 / 1e12  # 128 FP32 FMA lanes / cycle / SM
     fl32 = M * fp32_flops_per_location(n, Np, w.p)
     traffic = None
@@ -798,9 +804,11 @@ def run_ours(args, rank, world, local_rank):
                 "peak_source": f"derived: FP32 FMA, {sms} SMs x 256 flop/cycle x {mhz:.0f} MHz (sampled)",
                 "rescored_per_step": work["rescored"] / max(1, work["locations"]) / n}
     if f64s is not None:
-        a64 = f64s["fp64_flops_per_launch"] / (f64s["alc_kernel_ms"] / 1e3) / 1e12
-        f64s["roofline"] = {"bound": "alu", "kernel": "alc_bulk_kernel (FP64 state)", "unit": "TFLOP/s",
-                            "achieved": a64, "peak": fp64_peak, "frac": a64 / fp64_peak}
+        afx = f64s["mads_per_launch"] / (f64s["alc_kernel_ms"] / 1e3) / 1e12
+        fx_peak = sms * FX_MADS_PER_CYCLE_SM * mhz * 1e6 / 1e12
+        f64s["roofline"] = {"bound": "alu", "kernel": "alc_bulk_kernel (fixed-point state)",
+                            "unit": "T integer multiply-adds/s", "achieved": afx, "peak": fx_peak,
+                            "frac": afx / fx_peak}
     cpu, vs_oracle = None, None
     if not args.no_cpu and world == 1:
         S = 1024

@@ -58,7 +58,9 @@ typedef enum { LAGP_F64 = 0, LAGP_F32 = 1 } lagp_dtype;
 
 /* arithmetic of the ALC search (lagp_alc_select)
  *  LAGP_PREC_F64     the plain form: every candidate's criterion evaluated
- *                    with Eq. (dxy) in FP64, O(j^2) per candidate per step.
+ *                    with Eq. (dxy), O(j^2) per candidate per step: the
+ *                    quadratic form in 59-bit fixed point, in FP64 what leaves
+ *                    its range.
  *  LAGP_PREC_F32BULK candidates screened in FP32 through the Schur-complement
  *                    form of the same criterion (O(j) per candidate per
  *                    step); every contender (FP32 score within the
@@ -77,8 +79,9 @@ typedef enum { LAGP_F64 = 0, LAGP_F32 = 1 } lagp_dtype;
  *                    LAGP_PREC_F64SCHUR form; status LAGP_ENOTPD only if
  *                    that fails too.
  *  LAGP_PREC_F64SCHUR the same Schur-complement form with the candidate
- *                    state in FP64 (the incremental O(j) form of the
- *                    criterion, exact to FP64 rounding); the contenders
+ *                    state in 59-bit fixed point, or FP64 where that does not
+ *                    hold (the incremental O(j) form of the criterion, exact to
+ *                    FP64 rounding); the contenders
  *                    within a margin of 1e-5 of the best score are
  *                    re-scored with Eq. (dxy) as above.
  *  LAGP_PREC_F32BULK_F64 the FP32 screen of LAGP_PREC_F32BULK with its
@@ -105,7 +108,8 @@ typedef struct {
     int32_t block_threads;  /* threads per CTA of the ALC kernels */
     int32_t rescore_max;    /* F32BULK: contenders re-scored together in one
                                batch, 1..32, used up to 16; 0 = automatic (the
-                               autotuner's choice for the shape, else 8).
+                               autotuner's choice for the shape, else 8, or 16
+                               with few locations or N' > 1024).
                                More contenders take further batches, none is
                                dropped.  (F64SCHUR and F32BULK_F64: the
                                contenders re-scored, 0 = 8; beyond it those
@@ -164,11 +168,13 @@ int64_t lagp_launch_count(const lagp_ctx *ctx);
 lagp_status lagp_alc_work(lagp_ctx *ctx, uint64_t out[4]);
 
 /* Work counters of the Newton MLE of d (lagp_mle_step; not part of the
- * paper's method, they give its FP64 operation count, Eq. gpk):
- *   out[0]  sum over likelihood evaluations of n^3 (each factorises K_n:
- *           ~n^3/3 flops)
- *   out[1]  sum over derivative evaluations of n^3 (L^{-1}, K^{-1} and
- *           L^{-1} K' L^{-T}: ~2 n^3 flops)
+ * paper's method, they give its operation count, Eq. gpk):
+ *   out[0]  sum over likelihood evaluations of n^3 (in FP64 each factorises
+ *           K_n, ~n^3/3 flops; in fixed point each takes the factor and its
+ *           two derivatives, ~n^3 products)
+ *   out[1]  sum over derivatives used of n^3 (in FP64 L^{-1}, K^{-1} and
+ *           L^{-1} K' L^{-T}, ~2 n^3 flops; in fixed point they come with the
+ *           evaluation)
  * summed over every lagp_mle_step launched on this context since it was
  * created or last read.  Reading synchronises the context's stream and
  * resets the counters to zero. */
@@ -305,8 +311,9 @@ lagp_status lagp_alc_predict(lagp_ctx *ctx, const void *X, const void *Y, int64_
  * Predictive equations (Eqs. predgp, preds2) on each location's local design:
  *   mean = k^T K^{-1} Y_n,   psi = Y_n^T K^{-1} Y_n,
  *   s2   = psi (1 + g - k^T K^{-1} k) / n,   df = n,
- * with K_n factorised by FP64 Cholesky.  The predictive variance is
- * s2 * df / (df - 2).
+ * with the Cholesky factor of K_n: in 59-bit fixed point for designs of up to
+ * 128 rows and g < 1, in FP64 for the rest and for the locations whose values
+ * leave the fixed-point range.  The predictive variance is s2 * df / (df - 2).
  *   Y      N responses (dtype);  sel  M x n_max design rows (from
  *          lagp_alc_select);  n  M sizes or NULL (= n_max);  d  M lengthscales
  *          (a location whose sel row holds a row outside [0, N), n[m] outside
@@ -321,10 +328,12 @@ lagp_status lagp_predict(lagp_ctx *ctx, const void *X, const void *Y, int64_t N,
  * The ALC criterion of Eq. (dxy) for Nc candidates at one reference location
  * x and a given design of n rows — the computation Sec. 4.1 times (one x,
  * N' = 60,000 candidates, n = 16..512).  Per candidate, with K_n = L L^T
- * (FP64 Cholesky of the design's covariance, nugget g on the diagonal):
+ * (the Cholesky factor of the design's covariance, nugget g on the diagonal):
  *   u_c = L^{-1} k_n(x_c),  s_c = |u_c|^2,  q_c = (L^{-1} k_n(x))^T u_c,
  *   delta[c] = (K(x_c, x) - q_c)^2 / (1 + g - s_c)
- * (Eq. (dxy) with Eq. (piedef), simplified), FP64 throughout.
+ * (Eq. (dxy) with Eq. (piedef), simplified); for g < 1 the
+ * substitutions (and for n <= 128 the factor) in 59-bit fixed point, in FP64 what
+ * leaves its range.
  *   X        N x p design (dtype), device
  *   x        p FP64 coordinates of the location, device
  *   design   n design rows (int32, device), 1 <= n <= 1024
@@ -359,7 +368,9 @@ lagp_status lagp_scale_inputs(lagp_ctx *ctx, const void *X, int64_t N, int32_t p
  * Per-location Newton maximisation in d of the concentrated log-likelihood
  * of Eq. (gpk), log p(Y_n | d) = log Gamma(n/2) - (n/2) log(2 pi)
  *   - (1/2) log|K_n| - (n/2) log(psi/2), on the local design (Fig. 1 step 3),
- * with analytic first and second derivatives in d, all in FP64.  Step rule:
+ * with analytic first and second derivatives in d; the factor of K_n and its
+ * derivatives in 59-bit fixed point for designs of up to 128 rows and g < 1, in
+ * FP64 for the rest and for what leaves the fixed-point range.  Step rule:
  * Newton step -l'/l'' when l'' < 0, else doubling/halving in the gradient's
  * direction; proposals are clipped to [dmin, dmax]; a Newton step no longer
  * than 1e-3 d is taken as it is (near the maximiser the rise in l it brings
@@ -369,7 +380,8 @@ lagp_status lagp_scale_inputs(lagp_ctx *ctx, const void *X, int64_t N, int32_t p
  *   d       M lengthscales, in: starting values, out: estimates
  *   llik, dllik, d2llik   M FP64 outputs at the final d (any may be NULL)
  *   iters   M int32 iterations taken (may be NULL);  status  M int32
- * max_iter = 0 evaluates the likelihood and its derivatives at d only. */
+ * max_iter = 0 evaluates the likelihood and its derivatives at d only (without
+ * dllik and d2llik: the likelihood alone). */
 lagp_status lagp_mle_step(lagp_ctx *ctx, const void *X, const void *Y, int64_t N, int32_t p,
                           lagp_dtype dtype, int64_t M, const int32_t *sel, const int32_t *n,
                           int32_t n_max, double *d, double g, double dmin, double dmax,
@@ -390,8 +402,8 @@ lagp_status lagp_predict_grad(lagp_ctx *ctx, const void *X, const void *Y, int64
                               double *dllik_dg, int32_t *status);
 
 /* ----------------------------------------- a7 without device allocation
- * The paper has no counterpart to this entry point.  It computes exactly what
- * lagp_predict computes, for callers that cannot allocate device memory:
+ * The paper has no counterpart to this entry point.  It computes what
+ * lagp_predict computes (in FP64), for callers that cannot allocate device memory:
  * applications whose own allocator owns all device memory after start-up,
  * services under a device-memory budget fixed when they start, and
  * latency-critical paths that cannot afford cudaMalloc's implicit device

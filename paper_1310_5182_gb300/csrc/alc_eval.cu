@@ -444,7 +444,7 @@ eval_cands_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const
         const double minv = (1.0 + g) - s;  // m^{-1}(x_c), Eq. (piedef)
         const double r = kap - q;
         delta[c] = minv > 0.0 ? r * r / minv : CUDART_NAN;
-        bad |= !(minv > 0.0);  // (for FP64 to judge)
+        bad |= !(minv > 0.0);  // (for FP64 to decide)
         left[c] = bad ? 1 : 0;
         if (bad) atomicExch(redo, 1);
     }

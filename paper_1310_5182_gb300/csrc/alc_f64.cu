@@ -585,7 +585,7 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
                     const double kxg = -m * kxb;           // k_j(x)^T g_j(x_c)
                     const double kap = kappa[c];
                     const double dl = kxg * kxg * minv + 2.0 * kxg * kap + kap * kap * m;
-                    bad |= !(minv > 0.0);  // for FP64 to judge
+                    bad |= !(minv > 0.0);  // for FP64 to decide
                     if (better(dl, cands[c], best.v, best.row)) best = ArgBest{dl, cands[c], c};
                 }
                 best = warp_argmax(best);

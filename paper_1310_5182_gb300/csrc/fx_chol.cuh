@@ -254,7 +254,7 @@ __device__ __forceinline__ void fx_diagonal(const FxFactor &F, FxDiag *diag, int
     FxDiag D;
     auto pivot = [&](int j, const long long (&s)[NM]) {
         long long s0 = s[0], l;
-        // (a pivot below 2^-47, or not positive, is for FP64 to judge)
+        // (a pivot below 2^-47, or not positive, is for FP64 to decide)
         const bool odd = s0 < (1ll << 12) || s0 >= (1ll << 60);
         bad |= odd;
         if (odd) s0 = FX_ONE;

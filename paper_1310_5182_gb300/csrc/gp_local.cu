@@ -1,5 +1,7 @@
 // a7 (local prediction), a8 (local Newton MLE of d) and the analytic adjoint
-// of both in (d, g), on each location's selected design, all in FP64.
+// of both in (d, g), on each location's selected design, in FP64.  Prediction
+// and MLE run here for what gp_fixed.cu leaves: designs of more than 128 rows,
+// g >= 1, and locations whose values leave its range.
 //
 //   predict   Eqs. (predgp), (preds2): K_n = L L^T (Cholesky), z = L^{-1} Y_n,
 //             w = L^{-1} k_n(x);  mean = w^T z,  psi = z^T z,
