@@ -46,9 +46,9 @@
 // the set bits (0.1 to 10% of the pairs) to append the row to the queries'
 // candidate lists.
 //
-// What bounds it: the epilogue's instructions (a funnel shift a pair and about
-// 80 more for 64 pairs; 70% of the issue slots) and the design operand's reads
-// from the L2 (5.5 TB/s).  With one thread for all copies, one for all MMAs (and
+// What bounds it: the epilogue's funnel shifts, one a pair (the ALU pipe 62%
+// busy, 55% of the issue slots taken; the tensor pipe 15%), and the design
+// operand's reads from the L2 (5.5 TB/s).  With one thread for all copies, one for all MMAs (and
 // 64-bit divisions in both), every design block waited for them in turn, 490 ns
 // whatever its width; four such threads that also copy for themselves, 25.7 ->
 // 23.8 ms (4M rows, 25,000 queries, p = 8, N' = 2,000); accumulators of 64
