@@ -150,7 +150,7 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
 
 struct FxEval {
     double l, dl, d2l;
-    int flag;  // fx_factorise's
+    int flag;  // fx_factorise's; 2: derivatives too small for a fixed point
 };
 
 // l, and with NM = 3 l' and l'', of Eq. (gpk) at d from the packed squared distances; zs: the
@@ -221,12 +221,13 @@ __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, dou
             s_r.l = lgam - half_logdet - hn * logpsi;
             s_r.dl = (-v[1] - hn * q1) * id;
             s_r.d2l = (-v[2] - hn * fma(-q1, q1, v[5] * ipsi)) * id * id;
+            // K next to diagonal: l' as small as its terms, whose errors are
+            // absolute (2^-59 an operation), and the sign decides the step
+            s_r.flag = NM == 3 && n > 1 && !(fabs(v[1]) + hn * fabs(q1) >= 0x1p-16) ? 2 : 0;
         }
     }
     __syncthreads();
-    FxEval o = s_r;
-    o.flag = 0;
-    return o;
+    return s_r;
 }
 
 // NM = 1: the likelihood at d alone (max_iter = 0, no derivative wanted), a
@@ -281,7 +282,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
             // one evaluation; out of range: once more with a wider z
             auto eval = [&](double at) {
                 FxEval q = fx_llik<NM, T>(F, dist, at, g, zs, lgam, b);
-                if (q.flag && zs < ey + FX_Z1) {
+                if (q.flag == 1 && zs < ey + FX_Z1) {
                     zs = ey + FX_Z1;
                     q = fx_llik<NM, T>(F, dist, at, g, zs, lgam, b);
                 }
