@@ -313,14 +313,15 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
                             dn = fmin(fmax(d + delta, dmin), dmax);
                             t = eval(dn);
                             ll += n3;
-                            if (t.flag) break;
+                            if (t.flag == 1) break;
                             if (short_newton || t.l >= r.l) {
                                 accepted = true;
                                 break;
                             }
                             delta *= 0.5;
                         }
-                        if (t.flag) {
+                        // (flag 2: only a point that is taken needs its derivatives)
+                        if (t.flag == 1 || (accepted && t.flag)) {
                             st = FX_REDO;
                             break;
                         }
