@@ -198,8 +198,9 @@ __device__ __forceinline__ void fx_sums(const FxFactor &F, int c, int lane, int 
 
 // The diagonal block of columns c, c + 1, one warp: the sums of its three
 // entries (eight lanes an entry), then the block's factor, every lane the same.
+// Returns nonzero when a value left the range.
 template <int NM>
-__device__ __forceinline__ void fx_diagonal(const FxFactor &F, FxDiag *diag, int *flag, int c, int lane) {
+__device__ __forceinline__ unsigned fx_diagonal(const FxFactor &F, FxDiag *diag, int c, int lane) {
     const int n = F.n, m = F.m;
     const bool two = c + 1 < n;
     const int slot[3] = {fx_slot(c, c, m), fx_slot(c + 1, c, m), fx_slot(c + 1, c + 1, m)};
@@ -294,33 +295,31 @@ __device__ __forceinline__ void fx_diagonal(const FxFactor &F, FxDiag *diag, int
             if (lane == 0) fx_store(F, g, slot[1], r.v[g]);
         pivot(1, S[2]);
     }
-    if (lane == 0) {
-        *diag = D;
-        if (bad) atomicOr(flag, 1);
-    }
+    if (lane == 0) *diag = D;
+    return bad;
 }
 
 // The factorisation (and its derivatives for NM = 3), in place; shared memory holds
 // the raw values on entry and the limbs of L (L1, L2) after.  Two phases a
 // pair of columns: one thread a row finishes the two columns, then one warp
 // makes the next diagonal block (a serial chain of some 1,500 cycles) while
-// the others form the sums of the next two columns.  Returns the flag
-// (block-uniform).
+// the others form the sums of the next two columns.  Returns true when a value
+// left the range, as soon as the pair of columns is done.  The verdict travels
+// with the barriers and not through a word of shared memory, so that every
+// thread has the same one and a caller may factorise again at once.
 template <int NM, int T = FXT>
-__device__ int fx_factorise(const FxFactor &F, const Blk &b) {
+__device__ bool fx_factorise(const FxFactor &F, const Blk &b) {
     const int n = F.n, m = F.m;
     __shared__ FxDiag s_diag;
-    __shared__ int s_out;
-    if (b.tid == 0) s_out = 0;
+    unsigned bad = 0;  // this thread's share of the verdict
     __syncthreads();
-    if (b.warp == 0) fx_diagonal<NM>(F, &s_diag, &s_out, 0, b.lane);
+    if (b.warp == 0) bad = fx_diagonal<NM>(F, &s_diag, 0, b.lane);
     __syncthreads();
     for (int c = 0; c < n; c += 2) {
         const bool two = c + 1 < n;
         const FxDiag D = s_diag;
         // (rows from warp 1 on: warp 0 has the serial chains)
         for (int i = c + (two ? 2 : 1) + (b.warp + T / 32 - 1) % (T / 32) * 32 + b.lane; i < m; i += T) {
-            unsigned bad = 0;
             const int at = fx_slot(i, c, m);  // columns c, c + 1 of a row are adjacent
             long long S[NM], S2[NM];
 #pragma unroll
@@ -349,19 +348,18 @@ __device__ int fx_factorise(const FxFactor &F, const Blk &b) {
                 else
                     fx_store(F, g, at, r.v[g]);
             }
-            if (bad) atomicOr(&s_out, 1);
         }
-        __syncthreads();
+        if (__syncthreads_or(bad)) return true;
         if (c + 2 < n) {
             const int R = m - (c + 4);
-            if (b.warp == 0) fx_diagonal<NM>(F, &s_diag, &s_out, c + 2, b.lane);
+            if (b.warp == 0) bad |= fx_diagonal<NM>(F, &s_diag, c + 2, b.lane);
             else if (R > 24) fx_sums<NM, 2, T>(F, c + 2, b.lane, b.warp);
             else if (R > 12) fx_sums<NM, 3, T>(F, c + 2, b.lane, b.warp);
             else fx_sums<NM, 4, T>(F, c + 2, b.lane, b.warp);
             __syncthreads();
         }
     }
-    return s_out;
+    return false;
 }
 
 // Exponent e with max_i |v_i| < 2^e over the block's n values (INT_MAX when
