@@ -284,12 +284,24 @@ eval_prep_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const 
     }
 }
 
-// The same from the FP64 factor (n > 128): the limbs of its entries.
+// The same from the FP64 factor (n > 128): the limbs of its entries.  z is
+// scaled by the power of two that brings its largest entry below 1/4 (every
+// block finds it; |z^T u| then stays below 16): a location far from the design
+// has a z as small as its covariances, and the same relative precision.
 __global__ void eval_limbs_kernel(const double *L64, const double *rd, const double *z64, int np64, int n, int np,
                                   int2 *L, long long *ry, int *rt, int2 *z, int *ws, const int32_t *status,
                                   int *redo) {
     if (*status != LAGP_OK) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ int s_top;
+    if (threadIdx.x == 0) s_top = 0;
+    __syncthreads();
+    int top = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) top = max(top, (__double2hiint(z64[i]) >> 20) & 0x7ff);
+    atomicMax(&s_top, top);
+    __syncthreads();
+    top = s_top;
+    const int zs = top == 0 ? 0 : top - 1022 + 2;
     for (int e = tid; e < np * np; e += gridDim.x * blockDim.x) {
         const int i = e / np, k = e - i * np;
         const double v = i < n && k <= i ? L64[(size_t)i * np64 + k] : (i == k ? 1.0 : 0.0);
@@ -303,10 +315,13 @@ __global__ void eval_limbs_kernel(const double *L64, const double *rd, const dou
         if (ex < 0 || ex > 24) redo[0] = redo[1] = 1;  // (as fx_rsqrt's range)
         rt[i] = ex;
         ry[i] = fx_from(fx_shift(r, -ex));
-        const Fx f = fx_split(fx_from(i < n ? z64[i] : 0.0));
+        const Fx f = fx_split(fx_from(i < n && top < 0x7ff ? fx_shift(z64[i], -zs) : 0.0));
         z[i] = make_int2(f.h, f.l);
     }
-    if (tid == 0) *ws = 0;
+    if (tid == 0) {
+        *ws = zs;
+        if (top == 0x7ff) redo[0] = redo[1] = 1;  // not finite
+    }
 }
 
 __global__ void __launch_bounds__(EF_THREADS, 8)

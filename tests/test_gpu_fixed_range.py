@@ -35,3 +35,40 @@ def test_responses_out_of_range_in_an_uneven_batch(L, O):
     out = L.lagp_predict(dev(w.X), dev(Y), dev(w.Xref), dev(sel), n_arr, d, g)
     assert (out["status"].cpu().numpy() == 0).all()
     check_pred(out["mean"].cpu().numpy(), out["s2"].cpu().numpy(), ref, w.X, Y, w.Xref, sel, n_arr, d, g)
+
+
+def exact_eval(X, x, design, cands, d, g):
+    """Eq. (dxy), simplified, in extended precision."""
+    LD = np.longdouble
+    A, C, q = X[design].astype(LD), X[cands].astype(LD), np.asarray(x).astype(LD)
+    n = len(design)
+    k = lambda U, V: np.exp(-((U[:, None] - V[None]) ** 2).sum(-1) / LD(d))
+    L = k(A, A) + LD(g) * np.eye(n)
+    B = np.concatenate([k(A, q[None]), k(A, C)], axis=1)
+    for c in range(n):  # L L^T in place, and L^{-1} B beside it
+        L[c:, c] -= L[c:, :c] @ L[c, :c]
+        L[c, c] = np.sqrt(L[c, c])
+        L[c + 1:, c] /= L[c, c]
+        B[c] = (B[c] - L[c, :c] @ B[:c]) / L[c, c]
+    u, z = B[:, 1:], B[:, 0]
+    r = k(C, q[None])[:, 0] - z @ u
+    return r * r / (1 + LD(g) - (u * u).sum(0))
+
+
+@pytest.mark.parametrize("n", [60, 128, 129, 200])
+@pytest.mark.parametrize("shift", [0.0, 2.0, 3.5, 6.0])
+def test_alc_eval_with_the_location_away_from_the_design(L, O, n, shift):
+    """The location moved off the design and its candidates (largest covariance
+    with the design down to 1e-30).  Bar: cond(K) 2^-53 is 2e-11 here, the root
+    of a criterion value of 1e-6 of the best is 1e-3 of the best's, and ten
+    times the quotient of the two is 2e-7: a relative 1e-6."""
+    g, d = 1e-3, 0.5
+    w = W.toy2d(seed=52, N=6_000, M=1)
+    idx = O.knn(w.X, w.Xref, n + 800)[0]
+    design, cands = idx[:n], idx[n:][::4]
+    x = w.Xref[0] + np.array([shift, 0.0])
+    delta, st = L.lagp_alc_eval(dev(w.X), x, dev(design), dev(cands), d, g)
+    assert int(st.cpu()[0]) == 0
+    ref = exact_eval(w.X, x, design, cands, d, g).astype(np.float64)
+    top = ref >= 1e-6 * ref.max()
+    np.testing.assert_allclose(delta.cpu().numpy()[top], ref[top], rtol=1e-6)
