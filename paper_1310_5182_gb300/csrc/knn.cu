@@ -1359,7 +1359,10 @@ knn_sort(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
 // Bound: instruction issue and the latency of the gathers between barriers
 // (128 or 512 threads a query in place of 256: 30% slower).  Left to knn_sort (bigf): distances that are not
 // finite, a bucket of more than RANK_BUCKET rows, runs longer than 32 (many
-// equal distances), survivors past the placed buckets.
+// equal distances), survivors past the placed buckets.  knn_sort does not
+// check the collection: a query is left to it only when the N'-th value, or the
+// largest of its bucket, lies within the radius collected in full; otherwise,
+// and with distances that are not finite, it goes to the exact retry.
 constexpr int RANK_BUCKET = 24;
 
 // Buckets for up to `cap` placed rows (cap FP64 keys reuse their space).
@@ -1390,14 +1393,14 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     __shared__ double xq[64];
     __shared__ float yq[64];
     __shared__ int wsum[NT / 32];
-    __shared__ uint32_t s_lo, s_hi;
+    __shared__ uint32_t s_lo, s_hi, s_vk;
     __shared__ int s_kb, s_left, s_fail, s_S, s_ties;
     __shared__ float s_tauf, s_d2f;
     if (tid < p) {
         xq[tid] = load_coord64(Xref, q, p, tid, dt);
         yq[tid] = (float)(xq[tid] - kc->c[tid]);
     }
-    if (tid == 0) s_lo = 0xFFFFFFFFu, s_hi = 0u, s_left = s_ties = 0;
+    if (tid == 0) s_lo = 0xFFFFFFFFu, s_hi = s_vk = 0u, s_left = s_ties = 0;
     for (int b = tid; b < nb; b += NT) start[b] = 0u;
     __syncthreads();
     // direct-form FP32 values (non-negative floats order like their bits)
@@ -1437,8 +1440,12 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     }
     __syncthreads();
     const float base = __uint_as_float(s_lo), scale = (float)nb / (__uint_as_float(s_hi) - base);
+    // at least the exact distance of a row whose direct-form value is v
+    auto reach = [&](uint32_t v) { return sqrt((double)__uint_as_float(v)) * kc->g_half * (1.0 + 1e-13) + kc->e2; };
     if (s_hi >= 0x7f800000u) {  // infinite or NaN
-        if (tid == 0) bigf[q] = 1;
+        if (tid == 0) (rcol ? retry : bigf)[q] = 1;
+        if (rcol)
+            for (int t = tid; t < Npmax; t += NT) out[t] = -1;
         return;
     }
     // (equal values: 0 * infinity, bucket 0)
@@ -1481,7 +1488,18 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     const int last = min(s_kb + 1, nb - 1);  // the buckets placed: 0 .. last
     const int cut = last + 1 < nb ? (int)start[last + 1] : C;
     if (s_left || cut > cap) {
-        if (tid == 0) bigf[q] = 1;
+        // the N'-th value is at most the largest of its bucket
+        uint32_t top = 0u;
+#pragma unroll
+        for (int i = 0; i < IT; i++)
+            if (pos[i] >= 0 && bucket(key[i]) == s_kb) top = max(top, key[i]);
+        top = __reduce_max_sync(LAGP_FULL_MASK, top);
+        if (lane == 0) atomicMax(&s_vk, top);
+        __syncthreads();
+        const bool fail = rcol && !(reach(s_vk) <= (double)rcol[q]);
+        if (tid == 0) (fail ? retry : bigf)[q] = 1;
+        if (fail)
+            for (int t = tid; t < Npmax; t += NT) out[t] = -1;
         return;
     }
 #pragma unroll
@@ -1508,15 +1526,15 @@ knn_rank(const void *__restrict__ X, const float *__restrict__ Yv, const int32_t
     if (tid == 0) {
         // the margins with the launch's constants
         const double g = kc->g_half, e2 = kc->e2;
-        const float vk = __uint_as_float((uint32_t)(sk[k - 1] >> 32));
-        const double rk = sqrt((double)vk) * g * (1.0 + 1e-13) + e2;  // >= exact N'-th distance
+        const uint32_t vkb = (uint32_t)(sk[k - 1] >> 32);
+        const float vk = __uint_as_float(vkb);
         const float tauf = __double2float_rd(screen_margin_c(vk, g, e2));
         s_tauf = tauf;
         s_d2f = __double2float_ru(2.0 * tie_bound(tauf, g, kc->g_full, e2));
         // rows collected on the tensor cores: the N'-th of them must lie
         // within the radius collected in full, else the query goes to the
         // exact retry
-        s_fail = rcol ? !(rk <= (double)rcol[q]) : 0;
+        s_fail = rcol ? !(reach(vkb) <= (double)rcol[q]) : 0;
         // the survivors (s <= tauf) must all be placed
         if (cut < C && bucket(__float_as_uint(tauf)) > last) s_left = 1;
         s_S = k;
