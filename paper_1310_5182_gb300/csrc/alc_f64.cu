@@ -421,9 +421,16 @@ alc_f64_kernel(AlcArgs a, int *__restrict__ counter, double *__restrict__ panel_
 // K^{-1}'s largest diagonal entry (no entry is larger; the partial sums c_t
 // then stay in range), so that the quadratic form carries an error of about
 // 2^(es - 59) sqrt(j), below the 2^-53 |k|^T |K^{-1}| |k| of an FP64 evaluation.
-// The covariances are absolute (2^-59): a location whose nearest candidate has
-// K(x_c, x) < 2^-6 is left to the FP64 kernel, and so is one whose values leave
-// the range.
+// The covariances are absolute (2^-59), so that this holds where the winner's
+// are not small.  R = K(x*, x) - k_j(x)^T K^{-1} k* carries up to 2^(es - 58) (1 +
+// |k*|_1) here, and 2^(es - 57) |k_j(x)|_1 |k*|_1 in FP64 (the K^{-1} basis): a step
+// is trusted when the second is at least a quarter of the first, or |R| is 2^30
+// times the first.  The winner's criterion is evaluated again in FP64, from the
+// products that the update of K^{-1} needs.  A location with a step that is not
+// trusted is left to the FP64 kernel, and so is one whose nearest candidate
+// has K(x_c, x) < 2^-6 or whose values leave the range.  (Candidates many
+// lengthscales apart: the first of them are taken as before, and the others'
+// criterion was noise.)
 //
 // Bound: the integer multiply pipe; a product costs three multiply-adds, 12
 // cycles a warp against 64 on the FP64 unit, and half as many are made; the
@@ -533,7 +540,6 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
         if (tid == 0) s_top = 0;  // from here: exponent field of the largest diagonal entry
         for (int j = 0; j < nm && status == LAGP_OK; j++) {
             int cstar;
-            double delta = CUDART_NAN;
             if (j < a.n0) {
                 cstar = j;  // Fig. 1 step 2(a): the nearest neighbours, in order
             } else {
@@ -601,14 +607,10 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
                 if (warp == 0) {
                     ArgBest b0{lane < W ? w_v[lane] : 0.0, lane < W ? w_row[lane] : -1, lane < W ? w_slot[lane] : -1};
                     b0 = warp_argmax(b0);
-                    if (lane == 0) {
-                        s_cstar = b0.slot;
-                        s_delta = b0.v;
-                    }
+                    if (lane == 0) s_cstar = b0.slot;
                 }
                 __syncthreads();
                 cstar = s_cstar;
-                delta = s_delta;
                 if (cstar < 0) {  // (no candidate compares: left to FP64 as well)
                     status = FX_REDO;
                     break;
@@ -636,19 +638,33 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
             __syncthreads();
             if (warp == 0) {
                 double q = 0.0, xb = 0.0, yb = 0.0;
+                float ks = 0.f, xs = 0.f;
                 for (int t = lane; t < j; t += 32) {
                     q = fma(kst[t], bstar[t], q);
                     xb = fma(kx[t], bstar[t], xb);
+                    ks += (float)kst[t];
+                    xs += (float)kx[t];
                     if (fused) yb = fma(yd[t], bstar[t], yb);
                 }
                 q = warp_sum(q);
                 xb = warp_sum(xb);
                 if (fused) yb = warp_sum(yb);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    ks += __shfl_xor_sync(LAGP_FULL_MASK, ks, o);
+                    xs += __shfl_xor_sync(LAGP_FULL_MASK, xs, o);
+                }
                 if (lane == 0) {
-                    const double minv = (1.0 + g) - q;
-                    s_mu = 1.0 / minv;
+                    const double minv = (1.0 + g) - q, kap = kappa[cstar], m = 1.0 / minv;
+                    s_mu = m;
                     if (!(minv > 0.0)) s_bad = FX_REDO;
-                    s_cx = kappa[cstar] - xb;  // K(x*,x) - k_j(x)^T K^{-1} k*
+                    s_cx = kap - xb;  // K(x*,x) - k_j(x)^T K^{-1} k*
+                    if (j >= a.n0) {
+                        const double kxg = -m * xb;
+                        s_delta = kxg * kxg * minv + 2.0 * kxg * kap + kap * kap * m;
+                        const float err = ldexpf(1.f + ks, s_top - 1022 + PF_HEAD - 58);
+                        if (!(8.f * xs * ks >= 1.f + ks) && !(fabs(s_cx) >= 0x1p30 * err)) s_bad = FX_REDO;
+                    }
                     if (fused) {
                         s_ystar = a.dtype == LAGP_F64 ? static_cast<const double *>(a.Y)[rstar]
                                                       : (double)static_cast<const float *>(a.Y)[rstar];
@@ -694,7 +710,7 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
                 kx[j] = kappa[cstar];
                 chosen[cstar] = 1;
                 sel[j] = rstar;
-                if (alc) alc[j] = delta;
+                if (alc && j >= a.n0) alc[j] = s_delta;
             }
             __syncthreads();
             if (j + 1 < nm) {

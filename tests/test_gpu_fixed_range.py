@@ -8,7 +8,7 @@ import torch
 
 import workloads as W
 from test_gpu_fixed import check_mle
-from test_gpu_parity import L, O, check_pred, dev  # noqa: F401  (fixtures)
+from test_gpu_parity import L, O, check_pred, compare_selection, dev  # noqa: F401  (fixtures)
 
 pytestmark = pytest.mark.gpu
 
@@ -72,3 +72,33 @@ def test_alc_eval_with_the_location_away_from_the_design(L, O, n, shift):
     ref = exact_eval(w.X, x, design, cands, d, g).astype(np.float64)
     top = ref >= 1e-6 * ref.max()
     np.testing.assert_allclose(delta.cpu().numpy()[top], ref[top], rtol=1e-6)
+
+
+def wide_candidates(p, seed):
+    """Candidate sets that reach many lengthscales from the location: the 300
+    nearest rows, with d such that all but a few have tiny covariances."""
+    w = W.toy2d(seed=seed, N=20_000, M=60) if p == 2 else W.borehole(seed=seed, N=4_000, M=60, n=40, Np=300, g=1e-2)
+    idx = np.argsort(((w.X[None] - w.Xref[:, None]) ** 2).sum(-1), axis=1, kind="stable")[:, :300].astype(np.int32)
+    return w, idx
+
+
+def check_search(out, O, w, idx, n, d, g):
+    ref = O.alc_select(w.X, w.Xref, idx, 6, n, d, g, topk=4)
+    assert np.array_equal(out["status"].cpu().numpy(), ref["status"])
+    sel, alc = out["sel"].cpu().numpy(), out["alc"].cpu().numpy()
+    diverged = compare_selection(sel, ref, np.full(w.M, n, np.int32), 6, g)
+    assert len(diverged) <= 2  # (near ties are rare)
+    same = [m for m in range(w.M) if m not in diverged]
+    # the criterion of the rows taken, where it is a normal number (and the
+    # square of one): cond(K) is below 1e3 in these cases, ten times cond 2^-53 is 1e-12
+    a, r = alc[same, 6:], ref["alc"][same, 6:]
+    ok = r > 1e-280
+    np.testing.assert_allclose(a[ok], r[ok], rtol=1e-9)
+
+
+@pytest.mark.parametrize("p,d", [(2, 1e-5), (2, 1e-4), (2, 3e-4), (8, 0.003), (8, 0.01), (8, 0.03)])
+def test_plain_search_many_lengthscales_away(L, O, p, d):
+    w, idx = wide_candidates(p, 3)
+    g, n = 1e-2, 40
+    out = L.lagp_alc_select(dev(w.X), dev(w.Xref), dev(idx), 6, n, d, g, prec="f64", want_alc=True)
+    check_search(out, O, w, idx, n, d, g)
