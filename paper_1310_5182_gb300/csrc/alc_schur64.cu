@@ -34,14 +34,17 @@
 // FP64 form keeps u_c (as limbs), v_c, r_c and the candidates' coordinates
 // (relative to x, scaled by a power of two so that squared distances stay below
 // 1) in 59-bit fixed point.  All of them are bounded by 2, so that the state's
-// rounding, 2^-59, is below FP64's 2^-53 of the partial sums, and a product
-// costs three integer multiply-adds (12 cycles a warp) instead of the FP64
+// rounding, 2^-59, is below FP64's 2^-53 of the partial sums (a covariance
+// carries that of its squared distance, up to 2^-59 4^sc / d, in the exponent),
+// and a product costs three integer multiply-adds (12 cycles a warp) instead of the FP64
 // unit's 64; the exponential stays in FP64 (11 operations a candidate and
 // step, 57 before at p = 8, j = 25) and runs beside them.  The state selects
 // the contenders only; the re-score, every decision and every output are the
 // FP64 code's, and the same bit for bit when the same contenders come up.  A
 // location whose coordinates spread too far for the lengthscale (4^sc / d >=
-// 2^16), or whose pivot leaves the range, is redone with the FP64 state.
+// 2^16), or whose pivot leaves the range, is redone with the FP64 state, and so
+// is one whose best score is below FX_SCORE_MIN: the rounding is absolute, and
+// the scores of candidates many lengthscales from x would be noise.
 // 1,000 borehole locations: 6.5 -> 3.8 ms, designs and values bit-identical.
 //
 // Layout: one persistent CTA per location at a time (atomic work counter),
@@ -116,6 +119,10 @@ struct F32Params {
     int etab_smem;    // 1: the exp table copied to shared memory; 0: read through L1 (when
                       // the copy would cost the SM a resident CTA)
 };
+
+// Smallest best score that the fixed-point state decides, r_c^2 / v_c, so that
+// |r_c| is at least 2^-25 sqrt(v_c) and its absolute rounding below the margins.
+constexpr float FX_SCORE_MIN = 0x1p-50f;
 
 // Limbs kept in a 64-bit word of the panel.
 __device__ __forceinline__ Fx fx_limbs(long long w) { return Fx{(int)(w >> 32), (int)w}; }
@@ -427,6 +434,10 @@ alc_bulk_kernel(F32Params P) {
                 float gmax = w_max[0];
 #pragma unroll
                 for (int w = 1; w < F32_WARPS; w++) gmax = fmaxf(gmax, w_max[w]);
+                if (FXS && gmax < FX_SCORE_MIN) {  // (block-uniform)
+                    status = FX_REDO;
+                    break;
+                }
                 const float thr = gmax - margin * fabsf(gmax);
                 unsigned flags = 0;
 #pragma unroll

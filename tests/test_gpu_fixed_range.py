@@ -102,3 +102,13 @@ def test_plain_search_many_lengthscales_away(L, O, p, d):
     g, n = 1e-2, 40
     out = L.lagp_alc_select(dev(w.X), dev(w.Xref), dev(idx), 6, n, d, g, prec="f64", want_alc=True)
     check_search(out, O, w, idx, n, d, g)
+
+
+@pytest.mark.parametrize("p,d", [(2, 1e-4), (2, 3e-4), (8, 0.01), (8, 0.03)])
+def test_schur_search_many_lengthscales_away(L, O, p, d):
+    """(Scores are r^2 / v in FP32: with still smaller d they underflow to zero,
+    in the FP64 state as well, and the lowest rows are taken.)"""
+    w, idx = wide_candidates(p, 3)
+    g, n = 1e-2, 40
+    out = L.lagp_alc_select(dev(w.X), dev(w.Xref), dev(idx), 6, n, d, g, prec="f64schur", want_alc=True)
+    check_search(out, O, w, idx, n, d, g)
