@@ -209,21 +209,27 @@ __device__ __noinline__ FxEval fx_llik(const FxFactor F, const double *dist, dou
     block_sums<6, T>(v, b);  // (its barriers order s_prod)
     __shared__ FxEval s_r;
     if (b.warp == 0) {
-        // the two logarithms side by side, the other scalars on every lane
+        // the logarithms side by side, the other scalars on every lane
         double all = 1.0;
         for (int w = 0; w < T / 32; w += 2) all *= s_prod[w] * s_prod[w + 1];
-        const double arg = b.lane ? scalbn(v[3], 2 * zs) / 2.0 : all;
+        const double arg = b.lane == 0 ? all : (b.lane == 1 ? scalbn(v[3], 2 * zs) / 2.0 : 1.0 + g);
         const double lg = log(arg);
         const double half_logdet = -(__shfl_sync(LAGP_FULL_MASK, lg, 0) + v[0] * CUDART_LN2);
         const double logpsi = __shfl_sync(LAGP_FULL_MASK, lg, 1);
+        const double logdiag = __shfl_sync(LAGP_FULL_MASK, lg, 2);
         const double hn = 0.5 * n, ipsi = 1.0 / v[3], id = -ninv_d, q1 = v[4] * ipsi;
         if (b.lane == 0) {
             s_r.l = lgam - half_logdet - hn * logpsi;
             s_r.dl = (-v[1] - hn * q1) * id;
             s_r.d2l = (-v[2] - hn * fma(-q1, q1, v[5] * ipsi)) * id * id;
-            // K next to diagonal: l' as small as its terms, whose errors are
-            // absolute (2^-59 an operation), and the sign decides the step
-            s_r.flag = NM == 3 && n > 1 && !(fabs(v[1]) + hn * fabs(q1) >= 0x1p-16) ? 2 : 0;
+            // K next to diagonal (|K| within e^{-n/8} of the diagonal's product):
+            // the terms of d l' are small, and their errors absolute, about 2^-52
+            // n: below n / 16 they would exceed FP64's.  (8-d, n = 60, d = 0.004:
+            // l' off by a relative 1e-9.)  With terms below 2^-16 rounding would
+            // decide the sign, and so the step, whatever K is.
+            const double terms = fabs(v[1]) + hn * fabs(q1);
+            const bool diagonal = half_logdet > hn * (logdiag - 0.125);
+            s_r.flag = NM == 3 && n > 1 && !(terms >= 0x1p-16 && (!diagonal || terms >= 0.125 * hn)) ? 2 : 0;
         }
     }
     __syncthreads();

@@ -112,3 +112,42 @@ def test_schur_search_many_lengthscales_away(L, O, p, d):
     g, n = 1e-2, 40
     out = L.lagp_alc_select(dev(w.X), dev(w.Xref), dev(idx), 6, n, d, g, prec="f64schur", want_alc=True)
     check_search(out, O, w, idx, n, d, g)
+
+
+@pytest.mark.parametrize("n", [2, 8, 60])
+@pytest.mark.parametrize("responses", ["smooth", "noise"])
+def test_likelihood_derivatives_at_nearly_diagonal_k(L, n, responses):
+    """l' and l'' where the correlations of the design are small (lengthscales
+    from 0.002 of the box on), against extended precision.  Bar: (n^2 + t) 2^-50 of
+    the sum of the terms' magnitudes: sums of n^2 products, eight roundings each,
+    and exp(-t) of the nearest pair, t = D / d rounded."""
+    LD = np.longdouble
+    w = W.borehole(seed=31, N=4_000, M=40, n=60, Np=200, g=1e-3)
+    sel = np.argsort(((w.X[None] - w.Xref[:, None]) ** 2).sum(-1), axis=1, kind="stable")[:, :n].astype(np.int32)
+    Y = w.Y if responses == "smooth" else np.random.default_rng(7).normal(size=w.N)
+    g = 1e-3
+    for d in (0.002, 0.004, 0.01, 0.03, 0.1, 0.3):
+        out = L.lagp_mle_step(dev(w.X), dev(Y), dev(sel), n, d, g, 1e-300, 1e300, 0)
+        assert (out["status"].cpu().numpy() == 0).all()
+        for m in range(w.M):
+            A, y = w.X[sel[m]].astype(LD), Y[sel[m]].astype(LD)
+            D = ((A[:, None] - A[None]) ** 2).sum(-1)
+            E = np.exp(-D / LD(d))
+            t0 = float(D[np.triu_indices(n, 1)].min() / d)
+            K1, K2 = D / LD(d) ** 2 * E, (D * D / LD(d) ** 4 - 2 * D / LD(d) ** 3) * E
+            Ki = np.eye(n, dtype=LD)  # by Gauss-Jordan (K is nearly diagonal)
+            K = E + LD(g) * np.eye(n)
+            for c in range(n):
+                Ki[c], K[c] = Ki[c] / K[c, c], K[c] / K[c, c]
+                f = K[:, c].copy()
+                f[c] = 0
+                Ki, K = Ki - f[:, None] * Ki[c], K - f[:, None] * K[c]
+            a = Ki @ y
+            psi, t, B = y @ a, K1 @ a, Ki @ K1
+            phi = a @ t
+            one = [-np.trace(B) / 2, LD(n) / 2 * phi / psi]
+            two = [(B * B.T).sum() / 2, -(Ki * K2).sum() / 2,
+                   LD(n) / 2 * (a @ K2 @ a) / psi, -LD(n) * (t @ Ki @ t) / psi, LD(n) / 2 * (phi / psi) ** 2]
+            for k, terms in (("dllik", one), ("d2llik", two)):
+                err = abs(LD(out[k][m].item()) - sum(terms))
+                assert err <= (n * n + t0) * 2.0 ** -50 * sum(abs(v) for v in terms), (k, d, m, float(err))
