@@ -78,6 +78,7 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
     double *y = reinterpret_cast<double *>(fx_smem + f.words * 16);
     double *xd = y + 3 * nmax, *xq = xd + nmax * p, *kx = xq + p;  // (after y: the pivots)
     __shared__ int s_loc, s_flag, red[FXW];
+    __shared__ float s_part[FXW];
     const Blk b{(int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5};
     for (;;) {
         if (b.tid == 0) s_loc = atomicAdd(f.counter, 1);
@@ -121,18 +122,35 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
             }
             if (st == LAGP_OK) {
                 double v[3] = {0.0, 0.0, 0.0};
+                float part = 0.f;  // |w|_1 + |z|_1 - 2^11 |w|^T |z| (from the high limbs)
                 for (int i = b.tid; i < nm; i += FXT) {
-                    const double z = fx_double(fx_load(F, 0, fx_slot(nm, i, m)));
-                    const double w = fx_double(fx_load(F, 0, fx_slot(nm + 1, i, m)));
+                    const long long zf = fx_load(F, 0, fx_slot(nm, i, m)), wf = fx_load(F, 0, fx_slot(nm + 1, i, m));
+                    const double z = fx_double(zf), w = fx_double(wf);
                     v[0] = fma(w, z, v[0]);
                     v[1] = fma(z, z, v[1]);
                     v[2] = fma(w, w, v[2]);
+                    const float zh = fabsf((float)(int)(zf >> 30)) * 0x1p-29f, wh = fabsf((float)(int)(wf >> 30)) * 0x1p-29f;
+                    part += zh + wh - 0x1p11f * (zh * wh);
                 }
-                block_sums<3>(v, b);
-                mu = scalbn(v[0], zs + ws);
-                const double psi = scalbn(v[1], 2 * zs), kk = scalbn(v[2], 2 * ws);
-                sv = psi * ((1.0 + g) - kk) / nm;
-                dfv = nm;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(LAGP_FULL_MASK, part, o);
+                if (b.lane == 0) s_part[b.warp] = part;
+                block_sums<3>(v, b);  // (its barriers order s_part)
+                part = 0.f;
+                for (int q = 0; q < FXW; q++) part += s_part[q];
+                // w and z are absolute (2^-59): a mean made of a few small responses
+                // beside far larger ones has fewer bits than in FP64 (responses
+                // over twelve decades, K nearly diagonal: relative 3e-9 against
+                // 1e-14).  It goes there when 2^-58 (|w|_1 + |z|_1) exceeds both
+                // 2^-47 of its terms' magnitudes and 2^-44 of itself.
+                if (0x1p-14 * part > fabs(v[0])) {
+                    st = FX_REDO;
+                } else {
+                    mu = scalbn(v[0], zs + ws);
+                    const double psi = scalbn(v[1], 2 * zs), kk = scalbn(v[2], 2 * ws);
+                    sv = psi * ((1.0 + g) - kk) / nm;
+                    dfv = nm;
+                }
             }
         }
         if (b.tid == 0) {

@@ -151,3 +151,32 @@ def test_likelihood_derivatives_at_nearly_diagonal_k(L, n, responses):
             for k, terms in (("dllik", one), ("d2llik", two)):
                 err = abs(LD(out[k][m].item()) - sum(terms))
                 assert err <= (n * n + t0) * 2.0 ** -50 * sum(abs(v) for v in terms), (k, d, m, float(err))
+
+
+@pytest.mark.parametrize("d", [0.01, 0.1, 0.5])
+def test_mean_of_small_responses_beside_large_ones(L, d):
+    """Responses over twelve decades and a nearly diagonal K: the mean is a small
+    response times its covariance, far below the largest response.  Bar: 2^-40
+    relative (the covariances' exponents are rounded at t 2^-53, t up to 100), or
+    64 times FP64's rounding of the terms, cond(K) n 2^-53 |w| |z|."""
+    LD = np.longdouble
+    g, n = 1e-3, 40
+    w = W.borehole(seed=31, N=4_000, M=60, n=n, Np=200, g=g)
+    sel = np.argsort(((w.X[None] - w.Xref[:, None]) ** 2).sum(-1), axis=1, kind="stable")[:, :n].astype(np.int32)
+    rng = np.random.default_rng(7)
+    Y = rng.normal(size=w.N) * 10.0 ** rng.uniform(-6, 6, size=w.N)
+    out = L.lagp_predict(dev(w.X), dev(Y), dev(w.Xref), dev(sel), n, d, g)
+    assert (out["status"].cpu().numpy() == 0).all()
+    for m in range(w.M):
+        A, q = w.X[sel[m]].astype(LD), w.Xref[m].astype(LD)
+        K = np.exp(-((A[:, None] - A[None]) ** 2).sum(-1) / LD(d)) + LD(g) * np.eye(n)
+        cond = np.linalg.cond(K.astype(np.float64))
+        v = np.stack([np.exp(-((A - q) ** 2).sum(-1) / LD(d)), Y[sel[m]].astype(LD)], 1)
+        for c in range(n):  # K = L L^T in place, L^{-1} v beside it
+            K[c:, c] -= K[c:, :c] @ K[c, :c]
+            K[c, c] = np.sqrt(K[c, c])
+            K[c + 1:, c] /= K[c, c]
+            v[c] = (v[c] - K[c, :c] @ v[:c]) / K[c, c]
+        mean, mag = v[:, 0] @ v[:, 1], abs(v[:, 0]) @ abs(v[:, 1])
+        err = abs(LD(out["mean"][m].item()) - mean)
+        assert err <= max(2.0 ** -40 * abs(mean), 64 * cond * n * 2.0 ** -53 * mag), (m, float(err / abs(mean)))
