@@ -139,19 +139,20 @@ eval_cands_kernel(const void *X, int p, lagp_dtype dt, const double *x, const in
     const int64_t c = (int64_t)blockIdx.x * EV_THREADS + tid;
     if (redo && *redo == 0) return;
     // after the fixed-point kernels: the candidates they left (all when the
-    // factorisation itself left the range)
-    const bool write = c < Nc && (!left || left[c] != 0);
+    // factorisation itself left the range, and when it fails in FP64)
+    const bool failed = *status != LAGP_OK;
+    const bool write = c < Nc && (!left || left[c] != 0 || failed);
     if (left && !__syncthreads_or(write)) return;
     const bool live = c < Nc;
+    if (failed) {  // the design's K_n was not positive definite
+        if (write) delta[c] = CUDART_NAN;
+        return;
+    }
     for (int i = tid; i < EXP64_TABLE_SIZE; i += EV_THREADS) etab[i] = exp64_table_g[i];
     for (int e = tid; e < n * p; e += EV_THREADS) xd[e] = load_coord64(X, design[e / p], p, e % p, dt);
     const int32_t crow = live ? cands[c] : 0;
     for (int i = 0; i < p; i++) xc[(size_t)tid * p + i] = load_coord64(X, crow, p, i, dt);
     __syncthreads();
-    if (*status != LAGP_OK) {  // the design's K_n was not positive definite
-        if (write) delta[c] = CUDART_NAN;
-        return;
-    }
     const double ninv_d = -1.0 / d;
     const double *mx = xc + (size_t)tid * p;
     double s = 0.0, q = 0.0;

@@ -180,3 +180,24 @@ def test_mean_of_small_responses_beside_large_ones(L, d):
         mean, mag = v[:, 0] @ v[:, 1], abs(v[:, 0]) @ abs(v[:, 1])
         err = abs(LD(out["mean"][m].item()) - mean)
         assert err <= max(2.0 ** -40 * abs(mean), 64 * cond * n * 2.0 ** -53 * mag), (m, float(err / abs(mean)))
+
+
+def test_alc_eval_status_and_values_agree(L):
+    """Singular to rounding (no nugget, smooth kernel): the fixed-point factor
+    may succeed where the FP64 one fails.  A candidate that is a design row leaves
+    the range (1 - s = 0), and then FP64 decides for the call: ENOTPD and NaN
+    for every candidate, or OK and the others' values."""
+    rng = np.random.default_rng(5)
+    both = 0
+    for trial in range(1500):
+        n = int(rng.integers(8, 26))
+        X = rng.uniform(-2, 2, size=(200, 1 + trial % 2))
+        d = 10.0 ** rng.uniform(-0.5, 2.0)
+        cands = np.concatenate([np.arange(n, 200), [3]]).astype(np.int32)
+        delta, st = L.lagp_alc_eval(dev(X), X[n], dev(np.arange(n, dtype=np.int32)), dev(cands), d, 0.0)
+        delta, st = delta.cpu().numpy(), int(st.cpu()[0])
+        assert st in (0, 2)
+        if st == 2:
+            assert np.isnan(delta).all(), (trial, n, d)
+        both |= 1 << st
+    assert both == 5
