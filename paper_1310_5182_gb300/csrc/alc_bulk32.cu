@@ -972,10 +972,11 @@ lagp_status launch_b32(lagp_ctx *ctx, const AlcArgs &a) {
     int tmax = std::max(1, std::min(alc_rescore_batch(ctx, key, DT > DBASE || CPT >= 16 ? TMAX_CAP : 8), TMAX_CAP));
     // the largest batch whose vectors fit in shared memory (the batch size
     // changes no result)
-    while (tmax > 1 && b32_smem_bytes(a.nmax, a.p, tmax, NPAD) > ctx->smem_optin) tmax--;
     auto kern = alc_bulk32_kernel<CPT, DT>;
+    const size_t room = lagp_smem_room(ctx, kern);
+    while (tmax > 1 && b32_smem_bytes(a.nmax, a.p, tmax, NPAD) > room) tmax--;
     const size_t smem = b32_smem_bytes(a.nmax, a.p, tmax, NPAD);
-    if (smem > ctx->smem_optin)
+    if (smem > room)
         return lagp_fail(ctx, LAGP_EINVAL, "lagp_alc_select: shared memory exceeded (n_max, p too large)");
     LAGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;

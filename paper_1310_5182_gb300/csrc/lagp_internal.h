@@ -65,6 +65,14 @@ lagp_status alc_counters(lagp_ctx *ctx, int **counter, unsigned long long **work
 // status helpers (lagp_api.cu)
 lagp_status lagp_fail(lagp_ctx *ctx, lagp_status s, const std::string &msg);
 lagp_status lagp_cuda_check(lagp_ctx *ctx, cudaError_t e, const char *what);
+// Dynamic shared memory that a kernel can be launched with: the device's limit
+// for a block less the kernel's own static arrays.
+template <typename Kern>
+size_t lagp_smem_room(const lagp_ctx *ctx, Kern kern) {
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, kern) != cudaSuccess) return 0;
+    return ctx->smem_optin - at.sharedSizeBytes;
+}
 // returns nullptr and sets the error on failure
 void *lagp_ws(lagp_ctx *ctx, WsSlot slot, size_t bytes);
 
