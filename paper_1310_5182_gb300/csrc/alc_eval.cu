@@ -506,8 +506,8 @@ extern "C" lagp_status lagp_alc_eval(lagp_ctx *ctx, const void *X, int64_t N, in
     const int nf = (n + EF_B - 1) / EF_B * EF_B;
     const size_t smem_fx = (size_t)EF_K * EF_B * 8 + ((size_t)n * p + (size_t)EF_THREADS * p) * 8 +
                            ((size_t)n + EF_THREADS) * p * 4;
-    const bool fx = fixed && smem_fx <= ctx->smem_optin;
-    const bool fx_prep = fx && n <= FX_NMAX && ef_prep_smem(n, p) <= ctx->smem_optin;
+    const bool fx = fixed && smem_fx <= lagp_smem_room(ctx, eval_cands_fx_kernel);
+    const bool fx_prep = fx && n <= FX_NMAX && ef_prep_smem(n, p) <= lagp_smem_room(ctx, eval_prep_fx_kernel);
     auto prep64 = [&](const int *redo) {
         cudaFuncSetAttribute(eval_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_prep);
         eval_prep_kernel<<<1, PREP_THREADS, smem_prep, st>>>(X, p, dtype, x, design, n, np, d, g, Lm, rd, z, status,

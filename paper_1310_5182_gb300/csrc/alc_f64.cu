@@ -810,10 +810,10 @@ lagp_status launch_alc_f64(lagp_ctx *ctx, const AlcArgs &args) {
     // in fixed point where that holds (nugget below 1, K^{-1} twice in shared
     // memory: n_max up to about 115), then in FP64 what it leaves
     const size_t smem_fx = pf_smem(a.nmax, a.p);
-    const bool fixed = a.g < 1.0 && smem_fx <= ctx->smem_optin;
     int64_t grid_fx = 0;
     // one CTA an SM with all its registers for up to a location an SM, else two
     const auto kern_fx = a.M <= ctx->num_sms ? alc_f64fx_kernel<PF_BMAX> : alc_f64fx_kernel<4>;
+    const bool fixed = a.g < 1.0 && smem_fx <= lagp_smem_room(ctx, kern_fx);
     if (fixed) {
         cudaFuncSetAttribute(kern_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fx);
         int occ = 0;
