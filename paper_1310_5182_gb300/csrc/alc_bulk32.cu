@@ -237,7 +237,7 @@ __device__ __noinline__ void df_tri_upper(const float2 *us, const float2 *LT, in
 // next phase, off this chain)
 __device__ __noinline__ void winner_scalars(dfl vs, dfl rs, dfl rys, int j, bool fused, int32_t *sel, int row,
                                             int lane, float2 *wv, float2 *zv, float2 *LT, int ldl, float2 &s_il,
-                                            float2 &s_qx, float2 &s_psi, float2 &s_mean, int &s_total) {
+                                            float2 &s_qx, float2 &s_psi, float2 &s_mean) {
     const dfl il = df_rsqrt(vs);  // 1 / lambda
     const dfl wn = df_mul(rs, il);
     const dfl zn = fused ? df_mul(rys, il) : df_zero();
@@ -254,7 +254,6 @@ __device__ __noinline__ void winner_scalars(dfl vs, dfl rs, dfl rys, int j, bool
         st2(&s_psi, psi);
         st2(&s_mean, mean);
         sel[j] = row;
-        s_total = 0;
     }
 }
 
@@ -516,7 +515,7 @@ alc_bulk32_kernel(B32Params P) {
                 best_dl = make_float2(-FLT_MAX, 0.f);
             }
             __syncthreads();
-            const int total = s_total;
+            const int total = s_total;  // (written again only behind the next step's first barrier)
             if (total < 1) {
                 status = LAGP_ENOTPD;
                 break;
@@ -690,7 +689,7 @@ alc_bulk32_kernel(B32Params P) {
                                     s_work[3] += (unsigned long long)j * j;
                                 }
                                 winner_scalars(vc, rc, ryc, j, fused, sel, bat_row[0], lane, wv, zv, LT, ldl, s_il, s_qx,
-                                               s_psi, s_mean, s_total);
+                                               s_psi, s_mean);
                             }
                         }
                     }
@@ -895,7 +894,7 @@ alc_bulk32_kernel(B32Params P) {
             if (!lone && dw == 0)
                 winner_scalars(ld2(saved ? win_s : con_v + wl), ld2(saved ? win_s + 1 : con_r + wl),
                                ld2(saved ? win_s + 2 : con_ry + wl), j, fused, sel, best_row, lane, wv, zv, LT, ldl,
-                               s_il, s_qx, s_psi, s_mean, s_total);
+                               s_il, s_qx, s_psi, s_mean);
             if (dt == 32) {
                 // the ALC value (a lone contender's Delta is computed here) and
                 // the contender margin's error estimate
