@@ -200,9 +200,12 @@ lagp_status lagp_df_check(lagp_ctx *ctx, const double *a, int64_t n, float *spli
  * every admissible number of resident CTAs per SM of the persistent kernel
  * and, for F32BULK with tuning.rescore_max == 0, for double-float re-score
  * batches of 16, 8 and 4 contenders, and records the fastest for problems of
- * this shape (precision, N' capacity, n_max, p, with or without prediction)
- * on this context; later calls with tuning.ctas_per_sm == 0 (and
- * rescore_max == 0) use it.  Results do not depend on either choice.
+ * this shape (precision, N' capacity, n_max, p, with or without prediction,
+ * up to or above a location an SM where the kernels differ) on this context;
+ * later calls with tuning.ctas_per_sm == 0 (and rescore_max == 0) use it.
+ * A sample too small to fill every grid tried tells nothing about the CTAs per
+ * SM of a larger batch: only grids that differ are timed, and the number is
+ * returned but not recorded.  Results do not depend on either choice.
  * Synchronises the stream.  Arguments as lagp_alc_predict;
  * *best_ctas_per_sm and *best_rescore_max (either may be NULL) receive the
  * choices. */

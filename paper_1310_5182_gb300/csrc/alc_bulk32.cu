@@ -963,7 +963,7 @@ template <int CPT, int DT>
 lagp_status launch_b32(lagp_ctx *ctx, const AlcArgs &a) {
     constexpr int NPAD = FTHREADS * CPT;
     cudaStream_t st = ctx->stream;
-    const std::string key = alc_shape_key("alc_f32", CPT, a.nmax, a.p, a.mean != nullptr);
+    const std::string key = alc_shape_key(DT > DBASE ? "alc_f32wide" : "alc_f32", CPT, a.nmax, a.p, a.mean != nullptr);
     // (a CTA alone on its SM has shared memory for the largest batch: the 2-d
     // toy 1.53 -> 1.31 ms.  The wide candidate sets re-score many contenders a
     // step: the slab 51.4 -> 49.1 ms, the uneven borehole 348 -> 326 ms at two

@@ -818,7 +818,8 @@ lagp_status launch_alc_f64(lagp_ctx *ctx, const AlcArgs &args) {
         cudaFuncSetAttribute(kern_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fx);
         int occ = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern_fx, PF_THREADS, smem_fx);
-        int per_sm = alc_ctas_per_sm(ctx, alc_shape_key("alc_f64", 0, a.nmax, a.p, a.mean != nullptr), 2);
+        int per_sm = alc_ctas_per_sm(ctx, alc_shape_key(kern_fx == alc_f64fx_kernel<4> ? "alc_f64fx" : "alc_f64fxwide", 0,
+                                                        a.nmax, a.p, a.mean != nullptr), 2);
         if (occ > 0 && per_sm > occ) per_sm = occ;
         grid_fx = std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * per_sm, a.M));
     }

@@ -903,9 +903,10 @@ lagp_status launch_cpt(lagp_ctx *ctx, const AlcArgs &a) {
     const size_t smem = etab_smem ? smem_tab : smem_notab;
     if (!etab_smem) occ = occ_notab;
     const bool f64state = sizeof(T) == 8;  // (or fixed point)
-    int per_sm = alc_ctas_per_sm(ctx, alc_shape_key(f64state ? "alc_f64schur" : "alc_f32x64", CPT, a.nmax, a.p,
-                                                    a.mean != nullptr),
-                                 std::is_same_v<T, long long> ? 4 : (f64state ? 2 : 4));
+    constexpr bool fxstate = std::is_same_v<T, long long>;
+    int per_sm = alc_ctas_per_sm(ctx, alc_shape_key(fxstate ? "alc_fxschur" : (f64state ? "alc_f64schur" : "alc_f32x64"),
+                                                    CPT, a.nmax, a.p, a.mean != nullptr),
+                                 fxstate ? 4 : (f64state ? 2 : 4));
     if (occ > 0 && per_sm > occ) per_sm = occ;
     int64_t grid = (int64_t)ctx->num_sms * per_sm;
     if (grid > a.M) grid = a.M;
@@ -952,9 +953,12 @@ lagp_status launch_alc_f64schur(lagp_ctx *ctx, const AlcArgs &a) {
     AlcArgs f = a;
     f.fail_count = left;
     LAGP_TRY(launch_bulk<long long>(ctx, f));
+    const std::string key = ctx->last_alc_key;  // (the autotuner records under the fixed-point kernel's key)
     AlcArgs r = a;
     r.retry_count = left;
     r.retry_status = FX_REDO;
-    return launch_bulk<double>(ctx, r);
+    const lagp_status rc = launch_bulk<double>(ctx, r);
+    ctx->last_alc_key = key;
+    return rc;
 }
 lagp_status launch_alc_f32x64(lagp_ctx *ctx, const AlcArgs &a) { return launch_bulk<float>(ctx, a); }

@@ -53,7 +53,12 @@ extern "C" lagp_status lagp_autotune(lagp_ctx *ctx, const void *X, int64_t N, in
     cudaEvent_t e0, e1;
     LAGP_CUDA(ctx, cudaEventCreate(&e0));
     LAGP_CUDA(ctx, cudaEventCreate(&e1));
-    const int max_cps = (prec == LAGP_PREC_F32BULK || prec == LAGP_PREC_F32BULK_F64) ? 4 : 3;
+    // Counts of CTAs whose grid the sample's locations would cap are all the same
+    // launch: they are not tried, and what was timed among the others says
+    // nothing about a larger batch, so that the default stays.
+    const int all_cps = (prec == LAGP_PREC_F32BULK || prec == LAGP_PREC_F32BULK_F64) ? 4 : 3;
+    const bool capped = Ms < (int64_t)ctx->num_sms * all_cps;
+    const int max_cps = capped ? (int)((Ms + ctx->num_sms - 1) / ctx->num_sms) : all_cps;
     // the FP32-bulk kernel's re-score batch too (unless the user fixed it)
     const bool tune_b = prec == LAGP_PREC_F32BULK && ctx->tuning.rescore_max == 0;
     const int batches[3] = {16, 8, 4};
@@ -95,7 +100,7 @@ extern "C" lagp_status lagp_autotune(lagp_ctx *ctx, const void *X, int64_t N, in
     cudaEventDestroy(e1);
     if (rc != LAGP_OK) return rc;
     // recorded under the key the launcher looked up during the trials
-    ctx->tuned_ctas[key] = best;
+    if (!capped) ctx->tuned_ctas[key] = best;
     if (tune_b) ctx->tuned_tmax[key] = best_b;
     if (best_ctas_per_sm) *best_ctas_per_sm = best;
     if (best_rescore_max) *best_rescore_max = tune_b ? best_b : alc_rescore_batch(ctx, key);
