@@ -56,7 +56,8 @@ extern "C" lagp_status lagp_autotune(lagp_ctx *ctx, const void *X, int64_t N, in
     // Counts of CTAs whose grid the sample's locations would cap are all the same
     // launch: they are not tried, and what was timed among the others says
     // nothing about a larger batch, so that the default stays.
-    const int all_cps = (prec == LAGP_PREC_F32BULK || prec == LAGP_PREC_F32BULK_F64) ? 4 : 3;
+    // (at least the kernels' own defaults are tried: four, the plain form's two)
+    const int all_cps = prec == LAGP_PREC_F64 ? 3 : 4;
     const bool capped = Ms < (int64_t)ctx->num_sms * all_cps;
     const int max_cps = capped ? (int)((Ms + ctx->num_sms - 1) / ctx->num_sms) : all_cps;
     // the FP32-bulk kernel's re-score batch too (unless the user fixed it)

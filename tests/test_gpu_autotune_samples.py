@@ -25,3 +25,11 @@ def test_few_locations_time_only_the_grids_that_differ(L, prec):
         best = L.lagp_autotune(X, Xr, idx, 6, n, w.d, w.g, prec=prec)
         assert best["ctas_per_sm"] == 1
         assert torch.equal(L.lagp_alc_select(X, Xr, idx, 6, n, w.d, w.g, prec=prec)["sel"], before)
+
+
+def test_schur_form_tries_its_default(L):
+    """Four CTAs an SM, the fixed-point state's default, is 10% faster than three
+    here: tuned, the search keeps it."""
+    w, X, Xr, idx = problem(L, 2432, 1000)
+    best = L.lagp_autotune(X, Xr, idx, 6, 50, w.d, w.g, prec="f64schur")
+    assert best["ctas_per_sm"] == 4
