@@ -16,7 +16,8 @@ struct MleOut {
 
 // gp_fixed.cu.  counters: zeroed words, one a size class (at most 8); redo:
 // zeroed word that counts the locations left (status FX_REDO, outputs not
-// final, d unchanged).  ws: gp_fixed_workspace bytes.
+// final, d unchanged).  ws: gp_fixed_workspace bytes (the MLE's squared
+// distances, a CTA's own; less than the FP64 kernel's matrices).
 bool gp_fixed_supported(lagp_ctx *ctx, const GpArgs &a, bool mle);
 size_t gp_fixed_workspace(lagp_ctx *ctx, const GpArgs &a);
 lagp_status launch_predict_fixed(lagp_ctx *ctx, const GpArgs &a, const double *d, double *mean, double *s2,

@@ -429,7 +429,8 @@ bool gp_fixed_supported(lagp_ctx *ctx, const GpArgs &a, bool mle) {
 }
 
 size_t gp_fixed_workspace(lagp_ctx *ctx, const GpArgs &a) {
-    return (size_t)ctx->num_sms * 16 * ((size_t)a.nmax * (a.nmax + 1) / 2) * 8;
+    const size_t ctas = (size_t)std::min<int64_t>((int64_t)ctx->num_sms * 16, a.M);
+    return ctas * ((size_t)a.nmax * (a.nmax + 1) / 2) * 8;
 }
 
 lagp_status launch_predict_fixed(lagp_ctx *ctx, const GpArgs &a, const double *d, double *mean, double *s2,

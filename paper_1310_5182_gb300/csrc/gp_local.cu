@@ -676,7 +676,7 @@ struct GpLaunch {
 };
 
 template <typename Kern>
-lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, bool fixed, GpLaunch &L) {
+lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, bool fixed, size_t fx_bytes, GpLaunch &L) {
     const int ld = (a.nmax + 31) & ~31;
     L.smem = ((size_t)a.nmax * a.p + (size_t)a.nmax * 10 + (size_t)a.p + EXP64_TABLE_SIZE + 4) * 8 + 64;
     if (L.smem > ctx->smem_optin) return lagp_fail(ctx, LAGP_EINVAL, "n_max x p too large");
@@ -689,7 +689,7 @@ lagp_status prepare(lagp_ctx *ctx, const GpArgs &a, Kern kern, bool fixed, GpLau
     if (grid < 1) grid = 1;
     L.grid = (int)grid;
     size_t bytes = (size_t)grid * 6 * a.nmax * ld * 8 + 256;
-    if (fixed) bytes = std::max(bytes, gp_fixed_workspace(ctx, a));
+    bytes = std::max(bytes, fx_bytes);
     L.ws = static_cast<double *>(lagp_ws(ctx, WS_GP_MAT, bytes));
     int *words = static_cast<int *>(lagp_ws(ctx, WS_ALC_COUNTER, 256));
     if (!L.ws || !words) return LAGP_ENOMEM;
@@ -710,7 +710,7 @@ lagp_status launch_predict(lagp_ctx *ctx, const GpArgs &a, const double *d, doub
                            double *s2, double *df, int32_t *status) {
     GpLaunch L;
     const bool fixed = gp_fixed_supported(ctx, a, false);
-    LAGP_TRY(prepare(ctx, a, predict_kernel, fixed, L));
+    LAGP_TRY(prepare(ctx, a, predict_kernel, fixed, 0, L));
     if (fixed) LAGP_TRY(launch_predict_fixed(ctx, a, d, mean, s2, df, status, L.fx_counters, L.redo));
     predict_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, L.counter, L.ws, L.redo, mean, s2, df, status);
     ctx->launches++;
@@ -723,7 +723,7 @@ lagp_status launch_mle(lagp_ctx *ctx, const GpArgs &a, double *d, double dmin, d
                        int32_t *iters, int32_t *status) {
     GpLaunch L;
     const bool fixed = gp_fixed_supported(ctx, a, true);
-    LAGP_TRY(prepare(ctx, a, mle_kernel, fixed, L));
+    LAGP_TRY(prepare(ctx, a, mle_kernel, fixed, fixed ? gp_fixed_workspace(ctx, a) : 0, L));
     MleOut o{llik, dllik, d2llik, iters, status};
     int *ac = nullptr;
     unsigned long long *aw = nullptr;
@@ -742,7 +742,7 @@ lagp_status launch_predict_grad(lagp_ctx *ctx, const GpArgs &a, const double *d,
                                 double *ds2_dg, double *dllik_dd, double *dllik_dg,
                                 int32_t *status) {
     GpLaunch L;
-    LAGP_TRY(prepare(ctx, a, grad_kernel, false, L));
+    LAGP_TRY(prepare(ctx, a, grad_kernel, false, 0, L));
     GradOut o{dmean_dd, dmean_dg, ds2_dd, ds2_dg, dllik_dd, dllik_dg, status};
     grad_kernel<<<L.grid, GP_THREADS, L.smem, ctx->stream>>>(a, d, L.counter, L.ws, o);
     ctx->launches++;
