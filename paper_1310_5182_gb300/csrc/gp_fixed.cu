@@ -142,8 +142,24 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
                 // beside far larger ones has fewer bits than in FP64 (responses
                 // over twelve decades, K nearly diagonal: relative 3e-9 against
                 // 1e-14).  It goes there when 2^-58 (|w|_1 + |z|_1) exceeds both
-                // 2^-47 of its terms' magnitudes and 2^-44 of itself.
-                if (0x1p-14 * part > fabs(v[0])) {
+                // 2^-47 of its terms' magnitudes and 2^-44 of itself and K is within
+                // e^{-n/8} of its diagonal's determinant; with rows that are
+                // coupled FP64's z carries the rounding of the largest entries too.
+                bool few = 0x1p-14 * part > fabs(v[0]);
+                if (few) {  // (block-uniform)
+                    float ld = 0.f;  // log2 of det(K)^(-1/2)
+                    for (int i = b.tid; i < nm; i += FXT)
+                        ld += __log2f((float)(int)(fx_ry(F)[i] >> 30) * 0x1p-29f) + (float)fx_rt(F)[i];
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) ld += __shfl_xor_sync(LAGP_FULL_MASK, ld, o);
+                    __syncthreads();  // s_part was read
+                    if (b.lane == 0) s_part[b.warp] = ld;
+                    __syncthreads();
+                    ld = 0.f;
+                    for (int q = 0; q < FXW; q++) ld += s_part[q];
+                    few = ld < nm * (0.09f - 0.5f * __log2f(1.f + (float)g));
+                }
+                if (few) {
                     st = FX_REDO;
                 } else {
                     mu = scalbn(v[0], zs + ws);
