@@ -98,7 +98,9 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
             const FxFactor F{f.words, nm, m, f.words * 16, nmax};
             st = FX_REDO;
             int zs = 0, ws = 0;
-            for (int wide = 0; wide < 2 && st != LAGP_OK; wide++) {
+            // (responses that are all zero, or not finite, go to FP64 at once)
+            const int ey = fx_exponent(y, nm, red, b);
+            for (int wide = 0; wide < 2 && st != LAGP_OK && ey != INT32_MAX; wide++) {
                 bool odd = false;  // a distance that is not finite
                 for (int e = b.tid; e < nm * (nm + 1) / 2 + nm; e += FXT) {
                     int i, k;
@@ -110,8 +112,8 @@ predict_fx_kernel(GpArgs a, FxLaunch f, const double *__restrict__ dv, double *m
                     if (cross) kx[k] = E;
                     else *fx_raw(F, 0, fx_slot(i, k, m)) = fx_from(i == k ? E + g : E);
                 }
-                const int ex = fx_exponent(kx, nm, red, b), ey = fx_exponent(y, nm, red, b);
-                if (__syncthreads_or(odd) || ex == INT32_MAX || ey == INT32_MAX) break;
+                const int ex = fx_exponent(kx, nm, red, b);
+                if (__syncthreads_or(odd) || ex == INT32_MAX) break;
                 zs = ey + (wide ? FX_Z1 : FX_Z0);
                 ws = ex + 2;
                 for (int k = b.tid; k < nm; k += FXT) {
@@ -302,8 +304,9 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
         if (st == LAGP_OK) {
             const double g = a.g;
             d = fmin(fmax(d, dmin), dmax);
-            bool odd = false;
-            for (int e = b.tid; e < nm * (nm + 1) / 2; e += T) {
+            const int ey = fx_exponent<T>(y, nm, red, b);
+            bool odd = ey == INT32_MAX;
+            for (int e = b.tid; e < nm * (nm + 1) / 2 && !odd; e += T) {
                 int i, k;
                 fx_tri(e, i, k);
                 const double D = sqd(xd + (size_t)i * p, xd + (size_t)k * p, p);
@@ -314,8 +317,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
                 const double hn = 0.5 * nm;
                 s_lgam = lgamma(hn) - hn * log(2.0 * CUDART_PI);
             }
-            const int ey = fx_exponent<T>(y, nm, red, b);
-            odd = __syncthreads_or(odd) || ey == INT32_MAX;
+            odd = __syncthreads_or(odd);
             const double lgam = s_lgam;
             const FxFactor F{f.words, nm, nm + 1, y_at, nmax};
             int zs = ey + FX_Z0;

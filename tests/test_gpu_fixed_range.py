@@ -201,3 +201,25 @@ def test_alc_eval_status_and_values_agree(L):
             assert np.isnan(delta).all(), (trial, n, d)
         both |= 1 << st
     assert both == 5
+
+
+def test_zero_responses_cost_what_fp64_costs(L):
+    """All responses zero: nothing to scale, every location goes to the FP64
+    kernel, before any of the fixed-point work is done (g = 1 goes there by the
+    launcher's rule; the same arithmetic)."""
+    w = W.borehole(seed=1, N=4_000, M=2_000, n=60, Np=200)
+    X, Xr, Y = dev(w.X), dev(w.Xref), dev(np.zeros(w.N))
+    sel = L.lagp_knn(X, Xr, 100)[0]
+
+    def ms(g):
+        out = []
+        for _ in range(20):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            r = L.lagp_predict(X, Y, Xr, sel, 100, 2.0, g)
+            e[1].record()
+            torch.cuda.synchronize()
+            out.append(e[0].elapsed_time(e[1]))
+        assert (r["status"] == 0).all() and (r["mean"] == 0).all() and (r["s2"] == 0).all()
+        return sorted(out)[10]
+    assert ms(1e-4) <= 1.15 * ms(1.0)  # 1.02; 1.28 when found after the covariances
