@@ -191,7 +191,8 @@ __device__ __forceinline__ void fx_sums(const FxFactor &F, int c, int lane, int 
         if (ks < 4 && i < m && j < n) {
             const int slot = fx_slot(i, j, m);
 #pragma unroll
-            for (int g = 0; g < NM; g++) *fx_raw(F, g, slot) -= v[g];
+            // (each share that is not empty was rounded down, by a half on average)
+            for (int g = 0; g < NM; g++) *fx_raw(F, g, slot) -= v[g] + min(KS, c >> 1) / 2;
         }
     }
 }
@@ -247,6 +248,7 @@ __device__ __forceinline__ unsigned fx_diagonal(const FxFactor &F, FxDiag *diag,
             long long v = (hi[g] << 1) + (mid[g] >> 29);
 #pragma unroll
             for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(LAGP_FULL_MASK, v, o);
+            v += min(8, c >> 1) / 2;  // (shares rounded down)
 #pragma unroll
             for (int x = 0; x < 3; x++) S[x][g] -= __shfl_sync(LAGP_FULL_MASK, v, 8 * x);
         }

@@ -223,3 +223,30 @@ def test_zero_responses_cost_what_fp64_costs(L):
         assert (r["status"] == 0).all() and (r["mean"] == 0).all() and (r["s2"] == 0).all()
         return sorted(out)[10]
     assert ms(1e-4) <= 1.15 * ms(1.0)  # 1.02; 1.28 when found after the covariances
+
+
+def test_sums_of_the_factorisation_are_not_biased(L):
+    """s2 = |z|^2 (1 + g - |w|^2) / n with K nearly diagonal and responses of one
+    sign, where every inner product is rounded alike.  The mean of the relative
+    errors over the locations: 60 rounded sums each, of either sign, so that a
+    mean beyond 4 2^-53 is a bias (it was 12 with every share of a sum rounded
+    down)."""
+    LD = np.longdouble
+    g, n, d = 1e-3, 60, 0.01
+    w = W.borehole(seed=31, N=4_000, M=100, n=n, Np=200, g=g)
+    sel = np.argsort(((w.X[None] - w.Xref[:, None]) ** 2).sum(-1), axis=1, kind="stable")[:, :n].astype(np.int32)
+    Y = 2.0 + 0.1 * w.Y
+    out = L.lagp_predict(dev(w.X), dev(Y), dev(w.Xref), dev(sel), n, d, g)
+    rel = []
+    for m in range(w.M):
+        A, q = w.X[sel[m]].astype(LD), w.Xref[m].astype(LD)
+        K = np.exp(-((A[:, None] - A[None]) ** 2).sum(-1) / LD(d)) + LD(g) * np.eye(n)
+        v = np.stack([np.exp(-((A - q) ** 2).sum(-1) / LD(d)), Y[sel[m]].astype(LD)], 1)
+        for c in range(n):  # K = L L^T in place, L^{-1} v beside it
+            K[c:, c] -= K[c:, :c] @ K[c, :c]
+            K[c, c] = np.sqrt(K[c, c])
+            K[c + 1:, c] /= K[c, c]
+            v[c] = (v[c] - K[c, :c] @ v[:c]) / K[c, c]
+        s2 = (v[:, 1] ** 2).sum() * (1 + LD(g) - (v[:, 0] ** 2).sum()) / n
+        rel.append(float((LD(out["s2"][m].item()) - s2) / s2))
+    assert abs(np.mean(rel)) <= 4 * 2.0 ** -53
