@@ -443,6 +443,12 @@ alc_f64_kernel(AlcArgs a, int *__restrict__ counter, double *__restrict__ panel_
 constexpr int PF_THREADS = 512;
 constexpr int PF_BMAX = 8;
 constexpr int PF_HEAD = 4;
+// Products between folds of a middle sum: covariances are at most 1 and K^{-1}'s
+// limbs at most 2^-4, so that 28 products stay below 2^63; c_t and a are below 2,
+// so that the up to 8 rows of a block do (3 2^58 each).  Without folds a sum
+// of 56 equal products wrapped (equidistant rows), and at n = 112 of dense rows
+// the largest of 10^6 came to 0.65 2^63.
+constexpr int PF_FOLD = 24;
 
 __host__ __device__ inline int pf_ld(int nmax) { return nmax | 1; }
 __host__ __device__ inline int pf_ldk(int nmax) { return (nmax + PF_BMAX - 1) / PF_BMAX * PF_BMAX; }
@@ -554,18 +560,23 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
                         long long hi[B], mid[B];
 #pragma unroll
                         for (int r = 0; r < B; r++) hi[r] = 0, mid[r] = FX_HALF;
+                        for (int i0 = 0; i0 < t0; i0 += PF_FOLD) {
+                            const int i1 = min(i0 + PF_FOLD, t0);
 #pragma unroll 2
-                        for (int i = 0; i < t0; i++) {
-                            const int2 u = pc[(size_t)i * Npmax];
-                            const int4 *row = reinterpret_cast<const int4 *>(KL + (size_t)i * ldk + t0);
+                            for (int i = i0; i < i1; i++) {
+                                const int2 u = pc[(size_t)i * Npmax];
+                                const int4 *row = reinterpret_cast<const int4 *>(KL + (size_t)i * ldk + t0);
 #pragma unroll
-                            for (int r = 0; r < B; r += 2) {
-                                const int4 l = row[r / 2];
-                                hi[r] = fx_mad(u.x, l.x, hi[r]);
-                                mid[r] = fx_mad(u.y, l.x, fx_mad(u.x, l.y, mid[r]));
-                                hi[r + 1] = fx_mad(u.x, l.z, hi[r + 1]);
-                                mid[r + 1] = fx_mad(u.y, l.z, fx_mad(u.x, l.w, mid[r + 1]));
+                                for (int r = 0; r < B; r += 2) {
+                                    const int4 l = row[r / 2];
+                                    hi[r] = fx_mad(u.x, l.x, hi[r]);
+                                    mid[r] = fx_mad(u.y, l.x, fx_mad(u.x, l.y, mid[r]));
+                                    hi[r + 1] = fx_mad(u.x, l.z, hi[r + 1]);
+                                    mid[r + 1] = fx_mad(u.y, l.z, fx_mad(u.x, l.w, mid[r + 1]));
+                                }
                             }
+#pragma unroll
+                            for (int r = 0; r < B; r++) fx_fold_half(hi[r], mid[r]);
                         }
 #pragma unroll
                         for (int r = 0; r < B; r++) {  // the diagonal block (its diagonal halved)
@@ -584,6 +595,8 @@ alc_f64fx_kernel(AlcArgs a, int *__restrict__ counter, int *__restrict__ redo, i
                             xh = fx_hi(xh, Fx{al.x, al.y}, uf);
                             xm = fx_mid(xm, Fx{al.x, al.y}, uf);
                         }
+                        fx_fold(qh, qm);
+                        fx_fold(xh, xm);
                     }
                     const double quad = fx_double(fx_sum(qh, qm), es + 1), kxb = fx_double(fx_sum(xh, xm), es);
                     const double minv = (1.0 + g) - quad;  // m_j^{-1}(x_c), Eq. (piedef)

@@ -55,6 +55,19 @@ __device__ __forceinline__ long long fx_mid(long long mid, Fx x, Fx c) {
 __device__ __forceinline__ long long fx_sum(long long base, long long mid) { return base + (mid >> 29); }
 __device__ __forceinline__ long long fx_hi(long long sum, Fx x, Fx c) { return fx_mad(x.h, 2 * c.h, sum); }
 
+// Range of the middle sum: a product adds up to (|x| + |c|) 2^58 to it, and it
+// wraps at 2^63.  Where nothing bounds the norms of both factors, what is above
+// its low bits moves to the high sum now and then (exact); hi is doubled at the
+// end where it is a sum of h h' alone.
+__device__ __forceinline__ void fx_fold_half(long long &hi, long long &mid) {
+    hi += mid >> 30;
+    mid &= (1ll << 30) - 1;
+}
+__device__ __forceinline__ void fx_fold(long long &sum, long long &mid) {
+    sum += mid >> 29;
+    mid &= (1ll << 29) - 1;
+}
+
 __device__ __forceinline__ long long fx_mul(Fx a, Fx b) { return fx_hi(fx_mid(FX_HALF, a, b) >> 29, a, b); }
 
 __device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }

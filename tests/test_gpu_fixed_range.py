@@ -8,7 +8,7 @@ import torch
 
 import workloads as W
 from test_gpu_fixed import check_mle
-from test_gpu_parity import L, O, check_pred, compare_selection, dev  # noqa: F401  (fixtures)
+from test_gpu_parity import L, O, alc_atol, check_pred, compare_selection, dev  # noqa: F401  (fixtures)
 
 pytestmark = pytest.mark.gpu
 
@@ -250,3 +250,27 @@ def test_sums_of_the_factorisation_are_not_biased(L):
         s2 = (v[:, 1] ** 2).sum() * (1 + LD(g) - (v[:, 0] ** 2).sum()) / n
         rel.append(float((LD(out["s2"][m].item()) - s2) / s2))
     assert abs(np.mean(rel)) <= 4 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("M", [4, 200])  # both layouts
+def test_plain_search_with_equidistant_rows(L, O, M):
+    """A regular simplex as the seeds: K^{-1} has one value off its diagonal, a
+    candidate above the centre one covariance with all rows, and the middle
+    limbs' sums of 56 equal products are the largest there can be: for some of
+    the candidates above 2^63, for others, further up, not.  Lengthscales in
+    small steps, so that the low limb takes all values."""
+    p, n0, n, g = 60, 56, 60, 1e-2
+    rng = np.random.default_rng(23)
+    C = 1.0 / n0 * (np.arange(p) < n0) + 1e-2 * rng.normal(size=(100, p))
+    C[:, 57] += np.sqrt(rng.uniform(0, 3, size=100)) * rng.choice([-1, 1], 100)
+    X = np.concatenate([np.eye(p)[:n0], C])
+    Xref = np.tile(1.0 / n0 * (np.arange(p) < n0) + 0.3 * (np.arange(p) == 57), (M, 1))
+    idx = np.tile(np.arange(len(X), dtype=np.int32), (M, 1))
+    d = 20.0 + 0.37 * np.arange(M) if M > 100 else np.array([20.0, 31.7, 47.3, 66.1])
+    out = L.lagp_alc_select(dev(X), dev(Xref), dev(idx), n0, n, d, g, prec="f64", want_alc=True)
+    ref = O.alc_select(X, Xref, idx, n0, n, d, g, topk=4)
+    assert (out["status"].cpu().numpy() == 0).all()
+    diverged = compare_selection(out["sel"].cpu().numpy(), ref, np.full(M, n, np.int32), n0, g)
+    same = [m for m in range(M) if m not in diverged]
+    assert len(same) >= 0.9 * M
+    np.testing.assert_allclose(out["alc"].cpu().numpy()[same, n0:], ref["alc"][same, n0:n], rtol=1e-6, atol=alc_atol(g))
