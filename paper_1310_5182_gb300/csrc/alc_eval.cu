@@ -260,6 +260,20 @@ eval_prep_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const 
         for (int k = b.tid; k < n; k += FXT) *fx_raw(F, 0, fx_slot(n, k, m)) = fx_from(fx_shift(kx[k], -(ex + 2)));
         ok = !fx_factorise<1>(F, b);
     }
+    if (ok) {
+        bool big = false;  // |z|^2 >= 63 (entries are below 1: only beyond 64 rows)
+        if (n >= 64 && b.tid < 32) {
+            float s = 0.f;
+            for (int i = b.tid; i < n; i += 32) {
+                const float v = (float)fx_split(fx_load(F, 0, fx_slot(n, i, m))).h * 0x1p-29f;
+                s = fmaf(v, v, s);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(LAGP_FULL_MASK, s, o);
+            big = s >= 63.f;
+        }
+        ok = !__syncthreads_or(big);
+    }
     if (!ok) {
         if (b.tid == 0) {
             *status = FX_REDO;
@@ -375,6 +389,7 @@ eval_cands_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const
     const int e2 = (int)fminf(near / (float)d * 1.4426950f, 900.f) - EF_HEAD;
     unsigned bad = !(near < CUDART_INF_F);
     long long sh = 0, sm = FX_HALF, qh = 0, qm = FX_HALF;  // |u|^2 and z^T u
+    float norm2 = 0.f;                                     // |u|^2 in FP32: whether they hold
     const int nb = np / EF_B;
     for (int I = 0; I < nb; I++) {
         long long hi[EF_B], mid[EF_B];
@@ -433,6 +448,8 @@ eval_cands_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const
             const long long S = fx_from(kv >= 1.0 ? 0.0 : kv) - (hi[r] << 1) - (mid[r] >> 29);
             const Fx u = fx_split(fx_scaled(S, s_t[r], Fx{y2.x, y2.y}, bad));
             bad |= fx_beyond_h(u);
+            const float uf = (float)u.h * 0x1p-29f;
+            norm2 = fmaf(uf, uf, norm2);
             sh = fx_mad(u.h, 2 * u.h, sh);
             sm = fx_mid(sm, u, u);
             qh = fx_mad(u.h, 2 * z2.x, qh);
@@ -453,9 +470,10 @@ eval_cands_fx_kernel(const void *X, int p, lagp_dtype dt, const double *x, const
             sk = fma(df, df, sk);
         }
         const double kap = exp64_tang(sk * ninv_d, exp64_table_g);  // K(x_c, x)
-        // |u|^2 < 4 in its scale, so that neither sum has wrapped
+        // |u|^2 < 3.9 in its scale, so that neither sum has wrapped (they hold 16,
+        // and |z| is at most 8).  The sum itself could not tell: 34 looks like 2.
         const long long sv = fx_sum(sh, sm), qv = fx_sum(qh, qm);
-        bad |= (unsigned long long)sv >= (1ull << 61);
+        bad |= !(norm2 < 3.9f);
         const double s = scalbn(fx_double(sv), -2 * e2), q = scalbn(fx_double(qv), *wsp - e2);
         const double minv = (1.0 + g) - s;  // m^{-1}(x_c), Eq. (piedef)
         const double r = kap - q;

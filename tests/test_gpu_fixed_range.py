@@ -274,3 +274,24 @@ def test_plain_search_with_equidistant_rows(L, O, M):
     same = [m for m in range(M) if m not in diverged]
     assert len(same) >= 0.9 * M
     np.testing.assert_allclose(out["alc"].cpu().numpy()[same, n0:], ref["alc"][same, n0:n], rtol=1e-6, atol=alc_atol(g))
+
+
+@pytest.mark.parametrize("n,p,d", [(300, 2, 3.0), (600, 3, 2.0), (128, 2, 1.0)])
+def test_alc_eval_of_candidates_beyond_a_dense_design(L, O, n, p, d):
+    """Candidates outside a dense design with a tiny nugget: |L^{-1} k|^2, scaled
+    by its largest covariance, passes through every size up to far above 32,
+    where the fixed-point sum has wrapped once round, with all entries in range.
+    Bar: 3 cond(K) 2^-53 of max(delta, K^2)."""
+    rng = np.random.default_rng(29)
+    g = 1e-8
+    A = rng.uniform(size=(n, p))
+    C = np.full((240, p), 0.5)
+    C[:, 0] = np.linspace(1 + 2.7 * np.sqrt(d), 1 + 3.2 * np.sqrt(d), 240)
+    X = np.concatenate([A, C])
+    x = np.array([1.0 + 2 * np.sqrt(d)] + [0.45] * (p - 1))
+    design, cands = np.arange(n, dtype=np.int32), np.arange(n, n + 240, dtype=np.int32)
+    delta, st = L.lagp_alc_eval(dev(X), x, dev(design), dev(cands), d, g)
+    assert int(st.cpu()[0]) == 0
+    ref = exact_eval(X, x, design, cands, d, g).astype(np.float64)
+    kap2 = np.exp(-2 * ((C - x) ** 2).sum(-1) / d)
+    assert np.all(np.abs(delta.cpu().numpy() - ref) <= 3 * n / g * 2.0 ** -53 * np.maximum(ref, kap2))
