@@ -7,6 +7,8 @@
 #include "lagp_internal.h"
 
 // Status of a location that the fixed-point kernels leave to the FP64 ones.
+// The MLE leaves FX_REDO - k where the first k iterations hold: d is then the
+// point that they came to.
 constexpr int FX_REDO = -1;
 
 struct MleOut {
@@ -15,8 +17,8 @@ struct MleOut {
 };
 
 // gp_fixed.cu.  counters: zeroed words, one a size class (at most 8); redo:
-// zeroed word that counts the locations left (status FX_REDO, outputs not
-// final, d unchanged).  ws: gp_fixed_workspace bytes (the MLE's squared
+// zeroed word that counts the locations left (status FX_REDO or below, outputs
+// not final).  ws: gp_fixed_workspace bytes (the MLE's squared
 // distances, a CTA's own; less than the FP64 kernel's matrices).
 bool gp_fixed_supported(lagp_ctx *ctx, const GpArgs &a, bool mle);
 size_t gp_fixed_workspace(lagp_ctx *ctx, const GpArgs &a);

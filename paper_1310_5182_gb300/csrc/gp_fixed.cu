@@ -299,7 +299,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
         int st = load_design<T>(a, loc, nm, dv, xd, y, &s_flag, b);
         const unsigned long long n3 = (unsigned long long)nm * nm * nm;
         FxEval r{CUDART_NAN, CUDART_NAN, CUDART_NAN, 0};
-        int it = 0;
+        int it = 0, kept = 0;  // iterations; those that FP64 takes over
         double d = dv[loc];
         if (st == LAGP_OK) {
             const double g = a.g;
@@ -362,9 +362,11 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
                             }
                             delta *= 0.5;
                         }
-                        // (flag 2: only a point that is taken needs its derivatives)
+                        // (flag 2: only a point that is taken needs its derivatives;
+                        // FP64 goes on from the point before it, whose own hold)
                         if (t.flag == 1 || (accepted && t.flag)) {
                             st = FX_REDO;
+                            if (t.flag == 2) kept = it - 1;
                             break;
                         }
                         if (!accepted) break;
@@ -376,7 +378,7 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
                     }
                 }
             }
-            if (st != FX_REDO) {
+            if (st != FX_REDO || kept) {
                 n_llik += ll;
                 n_derivs += de;
             }
@@ -384,12 +386,12 @@ mle_fx_kernel(GpArgs a, FxLaunch f, double *dv, double dmin, double dmax, int ma
         if (b.tid == 0) {
             const bool ok = st == LAGP_OK;
             if (st == FX_REDO) atomicAdd(f.redo, 1);
-            if (ok) dv[loc] = d;
+            if (ok || kept) dv[loc] = d;
             if (o.llik) o.llik[loc] = ok ? r.l : CUDART_NAN;
             if (o.dllik) o.dllik[loc] = ok ? r.dl : CUDART_NAN;
             if (o.d2llik) o.d2llik[loc] = ok ? r.d2l : CUDART_NAN;
             if (o.iters) o.iters[loc] = it;
-            o.status[loc] = st;
+            o.status[loc] = st - kept;
         }
         __syncthreads();
     }

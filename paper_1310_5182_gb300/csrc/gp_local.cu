@@ -462,13 +462,13 @@ mle_kernel(GpArgs a, double *dv, double dmin, double dmax, int max_iter, int *co
         const int64_t loc = s_loc;
         __syncthreads();
         if (loc >= a.M) break;
-        if (redo && o.status[loc] != FX_REDO) continue;
+        if (redo && o.status[loc] > FX_REDO) continue;
         const int nm = a.n ? a.n[loc] : nmax;
         int st = load_design(a, loc, nm, dv, S.xd, S.y, &s_flag, b);
         const unsigned long long n3 = (unsigned long long)nm * nm * nm;
         double l = CUDART_NAN, psi = 0.0;
         Derivs dr{CUDART_NAN, CUDART_NAN};
-        int it = 0;
+        int it = redo ? FX_REDO - o.status[loc] : 0;  // (iterations that the fixed-point kernel made)
         double d = dv[loc];
         if (st == LAGP_OK) {
             const double g = a.g;

@@ -295,3 +295,28 @@ def test_alc_eval_of_candidates_beyond_a_dense_design(L, O, n, p, d):
     ref = exact_eval(X, x, design, cands, d, g).astype(np.float64)
     kap2 = np.exp(-2 * ((C - x) ** 2).sum(-1) / d)
     assert np.all(np.abs(delta.cpu().numpy() - ref) <= 3 * n / g * 2.0 ** -53 * np.maximum(ref, kap2))
+
+
+@pytest.mark.parametrize("n", [20, 60])
+def test_estimates_that_run_into_nearly_diagonal_k(L, O, n):
+    """Noise responses: steps towards the lower bound, begun in fixed point and
+    finished by the FP64 kernel from the last point that holds.  As the oracle's;
+    all iterations count, and all evaluations."""
+    g, M = 1e-2, 200
+    w = W.borehole(seed=92, N=4_000, M=M, n=n, Np=200, g=g)
+    sel = O.knn(w.X, w.Xref, n).astype(np.int32)
+    Y = np.random.default_rng(92).normal(size=w.N)
+    n_arr, d0 = np.full(M, n, np.int32), np.full(M, 0.5)
+    for max_iter in (0, 1, 2, 3, 30):
+        L.mle_work(torch.device("cuda", 0))
+        out = L.lagp_mle_step(dev(w.X), dev(Y), dev(sel), n, d0, g, 1e-2, 20.0, max_iter)
+        work = L.mle_work(torch.device("cuda", 0))
+        ref = O.mle(w.X, Y, sel, n_arr, d0, g, 1e-2, 20.0, max_iter)
+        it = out["iters"].cpu().numpy()
+        assert (out["status"].cpu().numpy() == 0).all()
+        same = it == ref["iters"]  # (the last step may differ where the likelihood is flat to rounding)
+        assert same.mean() >= (0.95 if max_iter == 30 else 1.0)
+        np.testing.assert_allclose(out["d"].cpu().numpy()[same], ref["d"][same], rtol=1e-6)
+        np.testing.assert_allclose(out["llik"].cpu().numpy(), ref["llik"], rtol=1e-9, atol=1e-9)
+        assert work["llik_n3"] >= (it.sum() + M) * n ** 3
+    assert (out["d"].cpu().numpy() <= 0.05).mean() > 0.2  # (the case that is meant does occur)
