@@ -1678,15 +1678,18 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     // overflow, and so an exact retry over the whole design (one CTA's pass
     // over all N rows: at N = 4M it sets the pass's duration), to about one
     // query in 1e9.  At least 2 N' + 1024, and no more than the power of two
-    // at or above that (the second sort launch's shared memory, sized by
-    // that power of two, keeps its resident CTAs), nor than the sort holds.
+    // at or above that, or 4,096 where that is more: with few neighbours of many
+    // rows the error margin widens the threshold most, and a capacity of 2,048
+    // left a query in 30 to the exact retry (N = 1.4M, N' = 88, p = 2, 116
+    // queries: 6.5 ms with three of them, 2.1 without).  Above 4,096 the rank takes 512 threads a
+    // query, a third slower.
     int32_t Cmax = std::min(2 * Npmax + 1024, CAND_CAP);
     if (stride > 1) {
         int32_t pow2 = 1;
         while (pow2 < Cmax) pow2 <<= 1;
         const int64_t rt = sample_rank(Npmax, stride, nsamp);
         const double want = (double)rt * stride + 6.0 * std::sqrt((double)rt) * stride + 512.0;
-        Cmax = (int32_t)std::min<double>(std::max<double>(Cmax, std::ceil(want)), std::min(pow2, CAND_CAP));
+        Cmax = (int32_t)std::min<double>(std::max<double>(Cmax, std::ceil(want)), std::min(std::max(pow2, 4096), CAND_CAP));
     }
     char *meta = static_cast<char *>(lagp_ws(ctx, WS_KNN_META, META_HEAD + (size_t)M * 12));
     int32_t *cand = static_cast<int32_t *>(lagp_ws(ctx, WS_KNN_CAND, (size_t)M * Cmax * 4));
