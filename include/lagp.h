@@ -406,7 +406,8 @@ lagp_status lagp_predict_grad(lagp_ctx *ctx, const void *X, const void *Y, int64
 
 /* ----------------------------------------- a7 without device allocation
  * The paper has no counterpart to this entry point.  It computes what
- * lagp_predict computes (in FP64), for callers that cannot allocate device memory:
+ * lagp_predict computes (in FP64 throughout; the two agree to rounding), for
+ * callers that cannot allocate device memory:
  * applications whose own allocator owns all device memory after start-up,
  * services under a device-memory budget fixed when they start, and
  * latency-critical paths that cannot afford cudaMalloc's implicit device

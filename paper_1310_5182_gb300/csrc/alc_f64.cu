@@ -438,7 +438,7 @@ alc_f64_kernel(AlcArgs a, int *__restrict__ counter, double *__restrict__ panel_
 // t at a time share a candidate's k_i (8 bytes from the panel) and read the
 // limbs of K^{-1} as broadcasts (no result depends on B).  Measured: 100
 // locations of the 2-d toy, n = 50, N' = 1000, 20.7 -> 2.9 ms (one CTA an SM, B
-// = 8; two with B = 4: 3.2); 1,000 locations in 5 dimensions 186 -> 16.4 ms
+// = 8; two with B = 4: 3.2; 2.84 now); 1,000 locations in 5 dimensions 186 -> 16.4 ms
 // (two CTAs, B = 4; one with B = 8: 19.5; 256 threads: 20.7).
 constexpr int PF_THREADS = 512;
 constexpr int PF_BMAX = 8;

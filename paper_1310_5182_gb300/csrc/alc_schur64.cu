@@ -751,7 +751,7 @@ alc_bulk_kernel(F32Params P) {
                 break;
             }
             if (j + 1 >= nm) break;
-            // ---------------- FP32 Schur recurrence with pivot x* (new column j of U)
+            // ---------------- Schur recurrence with pivot x* (new column j of U)
             {
                 T un[CPT];
                 if constexpr (FXS) {

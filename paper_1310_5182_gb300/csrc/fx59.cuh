@@ -10,12 +10,14 @@
 //
 // Why it is there: this GPU's FP64 unit takes a warp instruction every 64
 // cycles of a sub-partition, whatever its lanes; the integer pipe takes a
-// 32 x 32 -> 64 multiply-add every 2.1 (both measured), so a product costs
-// about 6.4 cycles instead of 64.  Why it is exact enough: a correlation
+// 32 x 32 -> 64 multiply-add every 4 (both measured), so a product costs
+// about 12 cycles instead of 64.  Why it is exact enough: a correlation
 // matrix with nugget g < 1 has a diagonal of 1 + g < 2, so the rows of its
 // factor have norm < sqrt(2) and every entry and every inner product is of
 // order one; a fixed 2^-59 is then finer than FP64's rounding of those sums
-// (2^-53 of the partial sums).
+// (2^-53 of the partial sums).  Where it is not: whatever is small as a whole
+// (means, criteria and derivatives far below the entries that they are made
+// of).  Each kernel says which of those it leaves to FP64.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

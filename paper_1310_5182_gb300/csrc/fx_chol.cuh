@@ -304,7 +304,7 @@ __device__ __forceinline__ unsigned fx_diagonal(const FxFactor &F, FxDiag *diag,
 // The factorisation (and its derivatives for NM = 3), in place; shared memory holds
 // the raw values on entry and the limbs of L (L1, L2) after.  Two phases a
 // pair of columns: one thread a row finishes the two columns, then one warp
-// makes the next diagonal block (a serial chain of some 1,500 cycles) while
+// makes the next diagonal block (a serial chain) while
 // the others form the sums of the next two columns.  Returns true when a value
 // left the range, as soon as the pair of columns is done.  The verdict travels
 // with the barriers and not through a word of shared memory, so that every

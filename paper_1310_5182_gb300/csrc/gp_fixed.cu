@@ -19,8 +19,10 @@
 //   of order one (t e^-t <= 1/e, |t^2 - 2t| e^-t <= 0.47, |L| < sqrt(2)), which
 //   is what fixed point asks for; z is scaled by a power of two.
 //
-// Bound: the integer multiply pipe (the inner products) and the FP64 unit
-// (the n^2/2 exponentials and their products with powers of t) about evenly.
+// Bound: latency and instruction fetch between short barriers (MLE, n = 60, four
+// CTAs an SM: issue 37%, barrier stalls 3.0 and no instruction 1.8 per issued
+// instruction, ALU 34%, FP64 20%); the prediction's n^2/2 exponentials on the
+// FP64 unit (62% busy at n = 60).
 // Two columns a step: the sums run with a 2 x 2 tile of (rows, columns) a
 // thread, so that a 16-byte shared-memory load (two k) feeds four products,
 // and 4 to 16 lanes share a row's sum, so that the threads stay busy as the
@@ -29,15 +31,26 @@
 //
 // Measured against the FP64 kernels (gp_local.cu), whole calls: the MLE of
 // 20,000 slab locations, n = 60, 4.1 evaluations each, 79.9 -> 29.7 ms; the
-// prediction at 100 locations, n = 50, 112 -> 64 us.  Errors against 64-bit
-// references no larger (l'' 10 to 100 times smaller than from explicit
-// inverses).  The line: above 128 rows the three matrices no longer fit in
+// prediction at 100 locations, n = 50, 112 -> 66 us.  Errors against 80-bit
+// references over lengthscales from nearly diagonal to ill-conditioned K, n = 8
+// and 60: medians as from the FP64 kernels (l'' up to five times smaller where
+// K is ill-conditioned).  The line: above 128 rows the three matrices no longer fit in
 // shared memory; from g = 1 on the factor's entries leave the range.
 //
 // A location whose values leave the fixed-point range (|x| < 2; 1 in the
-// further rows) first widens the scale of z, then goes to the FP64 kernels of
-// gp_local.cu: its status is FX_REDO when this kernel ends, and a second launch redoes it
-// (returning at once when there is none).  Non-finite inputs go there too.
+// further rows) first widens the scale of z (K's own rounding times its
+// condition number is then what counts, not that of the responses), then goes
+// to the FP64 kernels of gp_local.cu: its status is FX_REDO or below when this
+// kernel ends, and a second launch redoes it (returning at once when there is
+// none).  So do locations with non-finite inputs or without a nonzero response,
+// means of small responses beside large ones, and estimates at nearly diagonal K.
+//
+// Range of the sums: |S| holds 16 and wraps round at 32.  Rows of L have norms
+// below sqrt(2) whatever the data, and z rows, with entries below 1, at most
+// 11.4; the derivative rows' norms came to 1.7 and 5.1 (L1, L2) over kernels,
+// dimensions, lengthscales and nuggets down to 1e-8 with every entry in range,
+// so that S2 stays below 22, and 2^63 lies 17 standard deviations from the
+// middle sums of a share (a quarter of the columns).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -1706,7 +1706,7 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     unsigned long long *kmin = reinterpret_cast<unsigned long long *>(meta + 768);
     int32_t *cc = reinterpret_cast<int32_t *>(meta + META_HEAD);
     int32_t *retry = cc + M;
-    int32_t *bigf = retry + M;  // queries with more survivors than the first sort holds
+    int32_t *bigf = retry + M;  // queries that the rank leaves to the general sort
     LAGP_CUDA(ctx, cudaMemsetAsync(meta, 0, META_HEAD, st));
     LAGP_CUDA(ctx, cudaMemsetAsync(bigf, 0, (size_t)M * 4, st));
     const int blocks = ctx->num_sms * 4;
@@ -1803,7 +1803,7 @@ lagp_status launch_knn(lagp_ctx *ctx, const void *X, int64_t N, int p, lagp_dtyp
     }
     LAGP_CUDA(ctx, cudaGetLastError());
     if (tc_ws) {
-        // collection on the tensor cores, the sort (which checks each query's
+        // collection on the tensor cores, the rank (which checks each query's
         // collection), the exact retry of the flagged queries and their sort
         LAGP_TRY(launch_knn_tc_collect(ctx, tc_ws, N, p, Xref, dtype, M, Np, Npmax, kmax, kmin, order, cand, Cmax, cc,
                                        status, retry, tc_err, counters + 2, rcol, nullptr));

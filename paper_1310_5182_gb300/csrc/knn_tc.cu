@@ -19,9 +19,9 @@
 // Exactness: the rows with s <= tau2 are collected, tau2 a rigorous widening
 // (tc_margin) of the sampled threshold tau0 (itself widened by 2 E_tc so that
 // rows at the sample's boundary fall inside whatever the rounding of either
-// pass).  The sort then checks that the N'-th collected row lies within the
+// pass).  The rank then checks that the N'-th collected row lies within the
 // radius that tau2 guarantees collected (tc_collected_radius, stored per
-// query); a query that
+// query), also before it leaves a query to the general sort; a query that
 // fails, or whose buffer overflows, goes to the exact CUDA-core retry.  E_tc
 // (knn_common.cuh) assumes that one tensor-core instruction adds its products
 // and accumulator with an error of at most TC_ACC_ULPS = 64 units of 2^-24
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) knn_screen_tc(TcArgs a) {
         }
         __syncthreads();
         // per-query results: the collected rows and the threshold they were
-        // collected under (the sort checks that the N'-th of them lies within
+        // collected under (the rank checks that the N'-th of them lies within
         // the radius that threshold guarantees); an overflowing or
         // unscreened query goes to the exact retry
         const bool failed = *err != 0;
@@ -485,9 +485,8 @@ size_t knn_tc_workspace(int64_t N, int64_t M, int p) {
     return (size_t)(Npad + M) * K * 2 + (size_t)M * 8 + 256;
 }
 
-// Design and query operands, the sampled thresholds (tau0, filled by the
-// CUDA-core screen's passes A and B between the two launches), and the
-// collection pass.  ws: knn_tc_workspace(N, M, p) bytes.
+// Design and query operands, the sampled thresholds (tau0, filled by knn_sample
+// between the two launches), and the collection pass.  ws: knn_tc_workspace(N, M, p) bytes.
 lagp_status launch_knn_tc_prep(lagp_ctx *ctx, void *ws, const void *X, int64_t N, int p, lagp_dtype dtype,
                                const void *Xref, int64_t M, const unsigned long long *kmax,
                                const unsigned long long *kmin, const KnnOrder &order, float **tau0, float **rcol) {
@@ -537,9 +536,7 @@ lagp_status launch_knn_tc_collect(lagp_ctx *ctx, void *ws, int64_t N, int p, con
     a.stall = ctx->knn_tc_stall;
     ctx->knn_tc_stall = 0;
     // blocks: a multiple of the SM count (balanced waves), at most TC_QMAX
-    // queries each, taken from a counter (with boxes they cost unevenly;
-    // smaller blocks have smaller boxes, but blocks of 32 and 64 queries were
-    // no faster than 128)
+    // queries each, taken from a counter (with boxes they cost unevenly)
     const int64_t sms = ctx->num_sms;
     const int64_t nb_min = (M + TC_QMAX - 1) / TC_QMAX;
     const int64_t nb = std::min<int64_t>(M, round_up(nb_min, sms));

@@ -221,7 +221,7 @@ def test_zero_responses_cost_what_fp64_costs(L):
             torch.cuda.synchronize()
             out.append(e[0].elapsed_time(e[1]))
         assert (r["status"] == 0).all() and (r["mean"] == 0).all() and (r["s2"] == 0).all()
-        return sorted(out)[10]
+        return min(out)
     assert ms(1e-4) <= 1.15 * ms(1.0)  # 1.02; 1.28 when found after the covariances
 
 
