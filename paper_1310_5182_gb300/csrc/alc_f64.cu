@@ -428,9 +428,8 @@ alc_f64_kernel(AlcArgs a, int *__restrict__ counter, double *__restrict__ panel_
 // times the first.  The winner's criterion is evaluated again in FP64, from the
 // products that the update of K^{-1} needs.  A location with a step that is not
 // trusted is left to the FP64 kernel, and so is one whose nearest candidate
-// has K(x_c, x) < 2^-6 or whose values leave the range.  (Candidates many
-// lengthscales apart: the first of them are taken as before, and the others'
-// criterion was noise.)
+// has K(x_c, x) < 2^-6 or whose values leave the range.  (With candidates many
+// lengthscales apart the criterion of all but the nearest would be noise.)
 //
 // Bound: the integer multiply pipe; a product costs three multiply-adds, 12
 // cycles a warp against 64 on the FP64 unit, and half as many are made; the
